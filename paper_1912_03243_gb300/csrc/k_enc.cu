@@ -15,17 +15,32 @@
 // reproducible bit for bit by a CPU implementation of the same steps.
 //
 // Work mapping: one warp per 256-amplitude block, 8 amplitudes (16 code
-// bytes, one 16-byte load) per lane.  Target bits 0-2 pair amplitudes inside
-// a lane, bits 3-7 pair lanes (register exchange by shuffle), bits >= 8 pair
+// bytes, one 16-byte load, four words of two amplitudes) per lane.  Target
+// bits 0-2 pair amplitudes inside a lane, bits 3-7 pair lanes, bits >= 8 pair
 // two blocks that the same warp holds side by side.  A control bit >= 8
 // selects whole blocks; blocks whose control bit is 0 are not touched
 // (decode followed by encode with an unchanged scale returns the same codes).
+//
+// What bounds it: instruction issue.  A gate decodes, updates, measures and
+// re-encodes 16 components per lane, so the instructions per component decide
+// (about 150 per lane, block and gate; 420 for an in-block gate of a run
+// before).  The FP32 work is packed: the real (imaginary) parts of a word's
+// two amplitudes form one f32x2 operand, and mul / add / fma.rn.f32x2 round
+// each half as the scalar instruction does, so the codes stay bit-exact at
+// half the issue slots.  The decode table is addressed with one byte permute,
+// the block maximum is 3-input absolute maxima and one warp reduction (REDUX
+// on the bits: non-negative floats order as integers), and in-block pairs are
+// formed by exchanging packed codes.  28 qubits, one gate per pass: H inside
+// the blocks 255-274 us (319-385 before), H across them 240 (268), SX across
+// 244 (298), T across 129 (155); 27 qubits, 160 gates in runs: 11.0 ms
+// (17.5 with runs of in-block gates only).
 #include "sv_internal.h"
 
 namespace sv {
 namespace {
 
 constexpr int kWarpsPerCta = 8;
+constexpr int kGateWarps = 16;  // warps that share a decode table
 
 struct EncGateArgs {
     uint64_t nwork;     // warps of work (blocks or block pairs)
@@ -58,37 +73,9 @@ __device__ __forceinline__ uint64_t insert_zeros(uint64_t x, int nins, int p0, i
     return x;
 }
 
-// Signed table, indexed by the code's byte u = (uint8)q: tab[u * 32 + lane] =
-// sign(q) fl(|q| / 127), replicated per bank.  fl(s * (-t)) = -fl(s * t), so
-// s * tab[u] is exactly sign(q) fl(s T[|q|]).
-constexpr int kTabFloats = 256 * 32;
-__device__ __forceinline__ void load_table(float *tab) {
-    for (int i = threadIdx.x; i < kTabFloats; i += blockDim.x) {
-        const int q = int((signed char)(i >> 5));
-        const int a = q < 0 ? -q : q;
-        const float t = __fdiv_rn(float(a > 127 ? 127 : a), 127.0f);
-        tab[i] = q < 0 ? -t : t;
-    }
-    __syncthreads();
-}
-
-__device__ __forceinline__ float dec1(uint32_t u, float s, const float *tab, int lane) {
-    return __fmul_rn(s, tab[u * 32 + lane]);
-}
-
 // rint(x * fl(127/s)).  No clamp is needed: s is the exact maximum of |x| over
 // the block, so |x * fl(127/s)| <= 127 (1 + 2^-24)^2 < 127.5.
 __device__ __forceinline__ int enc1(float x, float inv) { return __float2int_rn(__fmul_rn(x, inv)); }
-
-// The same code as a byte, without a float-to-integer conversion: for
-// |v| < 2^22 the sum v + 1.5 * 2^23 lies in [2^23, 2^24), where the float
-// spacing is 1, so the (round-to-nearest-even) addition yields exactly
-// rint(v) + 1.5 * 2^23, whose bit pattern is 0x4B400000 + rint(v).  Its low
-// byte is rint(v) mod 256, the two's-complement code byte.  The product is
-// rounded on its own first (no contraction), as in enc1.
-__device__ __forceinline__ uint32_t enc_bits(float x, float inv) {
-    return __float_as_uint(__fadd_rn(__fmul_rn(x, inv), 12582912.0f));
-}
 
 __device__ __forceinline__ void gate_pair(const float *u, float &ar, float &ai, float &br, float &bi) {
     const float r0 = __fmaf_rn(u[0], ar, __fmaf_rn(-u[1], ai, __fmaf_rn(u[2], br, -__fmul_rn(u[3], bi))));
@@ -101,212 +88,446 @@ __device__ __forceinline__ void gate_pair(const float *u, float &ar, float &ai, 
     bi = i1;
 }
 
-// Shape of the 2x2 matrix, chosen on the host from exact zeros: the general
-// fixed-order update above, or the same update with the terms of zero
-// coefficients left out.  A left-out term contributes fmaf(0, x, y) = y up to
-// the sign of a zero, and a zero (of either sign) encodes to code 0 and does
-// not change a block maximum, so the codes are those of the general form.
-enum EncShape { ENC_GENERAL = 0, ENC_REAL = 1, ENC_DIAG = 2, ENC_DIAG1 = 3 };
+// ---- packed FP32 pairs (each half rounded as the scalar instruction)
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 pk(float x, float y) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ void upk(F2 r, float &x, float &y) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(r));
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ F2 dup2(float x) { return pk(x, x); }
 
-template <int SHAPE>
-__device__ __forceinline__ void gate_pair_s(const float *u, float &ar, float &ai, float &br, float &bi) {
-    if constexpr (SHAPE == ENC_REAL) {  // every imaginary part 0 (u[1] = u[3] = u[5] = u[7] = 0)
-        const float r0 = __fmaf_rn(u[0], ar, __fmul_rn(u[2], br));
-        const float i0 = __fmaf_rn(u[0], ai, __fmul_rn(u[2], bi));
-        const float r1 = __fmaf_rn(u[4], ar, __fmul_rn(u[6], br));
-        const float i1 = __fmaf_rn(u[4], ai, __fmul_rn(u[6], bi));
-        ar = r0;
-        ai = i0;
-        br = r1;
-        bi = i1;
-    } else if constexpr (SHAPE == ENC_DIAG || SHAPE == ENC_DIAG1) {  // u01 = u10 = 0
-        if constexpr (SHAPE == ENC_DIAG) {  // (u00 = 1: a unchanged)
-            const float r0 = __fmaf_rn(u[0], ar, -__fmul_rn(u[1], ai));
-            const float i0 = __fmaf_rn(u[0], ai, __fmul_rn(u[1], ar));
-            ar = r0;
-            ai = i0;
-        }
-        const float r1 = __fmaf_rn(u[6], br, -__fmul_rn(u[7], bi));
-        const float i1 = __fmaf_rn(u[6], bi, __fmul_rn(u[7], br));
-        br = r1;
-        bi = i1;
-    } else {
-        gate_pair(u, ar, ai, br, bi);
-    }
+// max(|a|, |b|, |c|) (a NaN loses, as in fmaxf)
+__device__ __forceinline__ float max3abs(float a, float b, float c) {
+    float d;
+    asm("max.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
 }
 
+// Warp maximum of non-negative floats: their bit patterns order as integers.
 __device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
 
-struct Lane8 {
-    float re[8], im[8];
+// The two amplitudes of a word, as packed real and imaginary parts.
+struct Amp2 {
+    F2 re, im;
 };
 
-// Byte k of w, zero-extended (one byte permute).
-__device__ __forceinline__ uint32_t byte_of(uint32_t w, int k) { return __byte_perm(w, 0u, 0x4440u | uint32_t(k)); }
+// A code byte 0x80 (-128, which no encoder writes) reads as -127: 0x80 -> 0x81.
+__device__ __forceinline__ uint32_t clamp_codes(uint32_t w) {
+    const uint32_t a = (w & 0x7f7f7f7fu) + 0x7f7f7f7fu;
+    return w + ((~(a | (w ^ 0x80808080u)) & 0x80808080u) >> 7);
+}
+__device__ __forceinline__ int4 clamp_codes(int4 v) {
+    return make_int4(int(clamp_codes(uint32_t(v.x))), int(clamp_codes(uint32_t(v.y))),
+                     int(clamp_codes(uint32_t(v.z))), int(clamp_codes(uint32_t(v.w))));
+}
 
-__device__ __forceinline__ void decode_lane(const int4 raw, float s, const float *tab, int lane, Lane8 &x) {
-    const uint32_t w[4] = {uint32_t(raw.x), uint32_t(raw.y), uint32_t(raw.z), uint32_t(raw.w)};
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const uint32_t word = w[j >> 1];
-        const int k = (j & 1) * 2;
-        x.re[j] = dec1(byte_of(word, k), s, tab, lane);
-        x.im[j] = dec1(byte_of(word, k + 1), s, tab, lane);
+// sign(q) fl(s fl(|q| / 127)) of a word's four codes.  q: the byte with its
+// sign bit flipped is q + 128, and 0x4B000000 + (q + 128) is the float
+// 2^23 + q + 128, from which 2^23 + 128 is taken exactly.  fl(q / 127):
+// 1/127 = hi + lo with hi = fl(1/127), and fma(q, hi, fl(q lo)) equals the
+// correctly rounded quotient for every |q| <= 127 (all 255 checked).
+__device__ __forceinline__ void dec_word(uint32_t w, F2 s2, Amp2 &x) {
+    const uint32_t o = w ^ 0x80808080u;
+    const F2 off = dup2(-8388736.0f), hi = dup2(__uint_as_float(0x3c010204u)), lo = dup2(2.9332994e-11f);
+    const F2 qr = add2(pk(__uint_as_float(__byte_perm(o, 0x4B000000u, 0x7440)),
+                          __uint_as_float(__byte_perm(o, 0x4B000000u, 0x7442))), off);
+    const F2 qi = add2(pk(__uint_as_float(__byte_perm(o, 0x4B000000u, 0x7441)),
+                          __uint_as_float(__byte_perm(o, 0x4B000000u, 0x7443))), off);
+    x.re = mul2(s2, fma2(qr, hi, mul2(qr, lo)));
+    x.im = mul2(s2, fma2(qi, hi, mul2(qi, lo)));
+}
+
+// The same from a table of fl(q / 127) in shared memory: row u = the code
+// byte, 64 floats per row of which lane l reads the l-th (no bank conflicts,
+// and one byte permute builds the byte offset 256 u + 4 l).  A code byte 0x80
+// reads as -127.
+constexpr int kTabBytes = 256 * 256;
+struct DecTable {
+    const unsigned char *tab;
+    uint32_t lane4;
+    __device__ __forceinline__ float at(uint32_t w, uint32_t sel) const {
+        return *reinterpret_cast<const float *>(tab + __byte_perm(w, lane4, sel));
     }
+    __device__ __forceinline__ void operator()(uint32_t w, F2 s2, Amp2 &x) const {
+        x.re = mul2(s2, pk(at(w, 0x5504), at(w, 0x5524)));
+        x.im = mul2(s2, pk(at(w, 0x5514), at(w, 0x5534)));
+    }
+};
+__device__ __forceinline__ void fill_table(unsigned char *smem) {
+    float *tab = reinterpret_cast<float *>(smem);
+    for (int i = threadIdx.x; i < 256 * 32; i += blockDim.x) {
+        const float q = float(int((signed char)(i >> 5)));
+        tab[(i >> 5) * 64 + (i & 31)] = __fdiv_rn(fmaxf(q, -127.0f), 127.0f);
+    }
+}
+
+// The codes of a word's two amplitudes.  The code byte comes without a
+// float-to-integer conversion: for |v| < 2^22 the sum v + 1.5 * 2^23 lies in
+// [2^23, 2^24), where the float spacing is 1, so the (round-to-nearest-even)
+// addition yields exactly rint(v) + 1.5 * 2^23, whose bit pattern is
+// 0x4B400000 + rint(v).  Its low byte is rint(v) mod 256, the
+// two's-complement code byte.  The product is rounded on its own first, as in
+// enc1: scalar multiplications, because ptxas contracts a packed
+// multiplication and addition in spite of their .rn.
+__device__ __forceinline__ uint32_t enc_word(const Amp2 &x, float inv) {
+    const F2 magic = dup2(12582912.0f);
+    float r0, r1, i0, i1;
+    upk(x.re, r0, r1);
+    upk(x.im, i0, i1);
+    upk(add2(pk(__fmul_rn(r0, inv), __fmul_rn(r1, inv)), magic), r0, r1);
+    upk(add2(pk(__fmul_rn(i0, inv), __fmul_rn(i1, inv)), magic), i0, i1);
+    const uint32_t lo = __byte_perm(__float_as_uint(r0), __float_as_uint(i0), 0x0040u);
+    const uint32_t hi = __byte_perm(__float_as_uint(r1), __float_as_uint(i1), 0x0040u);
+    return __byte_perm(lo, hi, 0x5410u);
+}
+
+__device__ __forceinline__ float amp_max(float m, const Amp2 &x) {
+    float a, b, c, d;
+    upk(x.re, a, b);
+    upk(x.im, c, d);
+    return max3abs(max3abs(m, a, b), c, d);
+}
+
+// A lane's 8 amplitudes of a block.
+struct Lane8 {
+    Amp2 w[4];
+};
+
+__device__ __forceinline__ void decode_lane(const DecTable &dec, const int4 raw, float s, Lane8 &x) {
+    const F2 s2 = dup2(s);
+    dec(uint32_t(raw.x), s2, x.w[0]);
+    dec(uint32_t(raw.y), s2, x.w[1]);
+    dec(uint32_t(raw.z), s2, x.w[2]);
+    dec(uint32_t(raw.w), s2, x.w[3]);
 }
 
 __device__ __forceinline__ float lane_absmax(const Lane8 &x) {
     float m = 0.0f;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) m = fmaxf(m, fmaxf(fabsf(x.re[j]), fabsf(x.im[j])));
+    for (int k = 0; k < 4; ++k) m = amp_max(m, x.w[k]);
     return m;
+}
+
+// Codes of a lane's 8 amplitudes, inv = fl(127 / s).
+__device__ __forceinline__ int4 enc_words(const Amp2 (&w)[4], float inv) {
+    return make_int4(int(enc_word(w[0], inv)), int(enc_word(w[1], inv)), int(enc_word(w[2], inv)),
+                     int(enc_word(w[3], inv)));
 }
 
 // Encode a lane's 8 amplitudes with the block scale s (warp-uniform).
 __device__ __forceinline__ int4 encode_lane(const Lane8 &x, float s) {
     if (s == 0.0f) return make_int4(0, 0, 0, 0);
-    const float inv = __fdiv_rn(127.0f, s);
-    uint32_t w[4];
+    return enc_words(x.w, __fdiv_rn(127.0f, s));
+}
+
+// Encode a lane's share of two blocks with their scales: even lanes divide
+// for the first block, odd lanes for the second.
+__device__ __forceinline__ void encode_two(const Amp2 (&x)[4], float s0, const Amp2 (&y)[4], float s1, int lane,
+                                           int4 &v0, int4 &v1) {
+    const float inv = __fdiv_rn(127.0f, lane & 1 ? s1 : s0);
+    v0 = enc_words(x, __shfl_sync(0xffffffffu, inv, 0));
+    v1 = enc_words(y, __shfl_sync(0xffffffffu, inv, 1));
+    if (s0 == 0.0f) v0 = make_int4(0, 0, 0, 0);
+    if (s1 == 0.0f) v1 = make_int4(0, 0, 0, 0);
+}
+
+// Shape of the 2x2 matrix, chosen on the host from exact zeros: the general
+// fixed-order update (gate_pair), or the same update with the terms of zero
+// coefficients left out.  A left-out term contributes fmaf(0, x, y) = y up to
+// the sign of a zero, and a zero (of either sign) encodes to code 0 and does
+// not change a block maximum, so the codes are those of the general form.
+enum EncShape { ENC_GENERAL = 0, ENC_REAL = 1, ENC_DIAG = 2, ENC_DIAG1 = 3 };
+
+// The matrix as packed operands; -u for the products the update subtracts
+// (a product with a negated factor is the negated product).
+template <int SHAPE>
+struct Mat2 {
+    F2 u[8], n[8];
+    __device__ __forceinline__ explicit Mat2(const float *m) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            u[k] = dup2(m[k]);
+            n[k] = dup2(-m[k]);
+        }
+    }
+};
+
+// (a, b) <- U (a, b) on two amplitude pairs.
+template <int SHAPE>
+__device__ __forceinline__ void gate2(const Mat2<SHAPE> &m, Amp2 &a, Amp2 &b) {
+    const F2 ar = a.re, ai = a.im, br = b.re, bi = b.im;
+    if constexpr (SHAPE == ENC_REAL) {  // every imaginary part 0
+        a.re = fma2(m.u[0], ar, mul2(m.u[2], br));
+        a.im = fma2(m.u[0], ai, mul2(m.u[2], bi));
+        b.re = fma2(m.u[4], ar, mul2(m.u[6], br));
+        b.im = fma2(m.u[4], ai, mul2(m.u[6], bi));
+    } else if constexpr (SHAPE == ENC_DIAG || SHAPE == ENC_DIAG1) {  // u01 = u10 = 0
+        if constexpr (SHAPE == ENC_DIAG) {  // (u00 = 1: a unchanged)
+            a.re = fma2(m.u[0], ar, mul2(m.n[1], ai));
+            a.im = fma2(m.u[0], ai, mul2(m.u[1], ar));
+        }
+        b.re = fma2(m.u[6], br, mul2(m.n[7], bi));
+        b.im = fma2(m.u[6], bi, mul2(m.u[7], br));
+    } else {
+        a.re = fma2(m.u[0], ar, fma2(m.n[1], ai, fma2(m.u[2], br, mul2(m.n[3], bi))));
+        a.im = fma2(m.u[0], ai, fma2(m.u[1], ar, fma2(m.u[2], bi, mul2(m.u[3], br))));
+        b.re = fma2(m.u[4], ar, fma2(m.n[5], ai, fma2(m.u[6], br, mul2(m.n[7], bi))));
+        b.im = fma2(m.u[4], ai, fma2(m.u[5], ar, fma2(m.u[6], bi, mul2(m.u[7], br))));
+    }
+}
+
+// old where the half's bit of the two control bits in `bits` is 0 (bit masks,
+// not selects: eight loop-invariant predicates would not fit a warp's seven).
+__device__ __forceinline__ F2 keep_where(F2 now, F2 old, uint32_t bits) {
+    const uint32_t m0 = uint32_t(int(bits << 31) >> 31), m1 = uint32_t(int(bits << 30) >> 31);
+    const F2 m = F2(m0) | F2(m1) << 32;
+    return (now & m) | (old & ~m);
+}
+
+// gate2 on the pairs whose control bit is set: bits (two, for the word's two
+// amplitudes) of the lane's control mask.
+template <int SHAPE>
+__device__ __forceinline__ void gate2_ctl(const Mat2<SHAPE> &m, Amp2 &a, Amp2 &b, uint32_t bits) {
+    const Amp2 a0 = a, b0 = b;
+    gate2<SHAPE>(m, a, b);
+    a.re = keep_where(a.re, a0.re, bits);
+    a.im = keep_where(a.im, a0.im, bits);
+    b.re = keep_where(b.re, b0.re, bits);
+    b.im = keep_where(b.im, b0.im, bits);
+}
+
+// Update of a block on an in-block target t.  The words are first rearranged
+// so that words 0, 1 hold the lower and words 2, 3 the upper amplitudes of
+// the lane's four pairs (pair p = word p / 2, half p % 2): t = 2 as stored;
+// t = 1: words 1 and 2 swap; t = 0: halves; t >= 3: the lower lane of a pair
+// of lanes takes the pairs of words 0, 1 and the upper lane those of words
+// 2, 3 (two shuffles of packed codes instead of sixteen of amplitudes, and
+// no pair computed twice).  Each rearrangement undoes itself.
+__device__ __forceinline__ void arrange(uint4 &v, int t, int lane) {
+    if (t == 2) return;
+    if (t == 1) {
+        const uint32_t s = v.y;
+        v.y = v.z;
+        v.z = s;
+    } else if (t == 0) {
+        const uint4 o = v;
+        v.x = __byte_perm(o.x, o.y, 0x5410u);
+        v.y = __byte_perm(o.z, o.w, 0x5410u);
+        v.z = __byte_perm(o.x, o.y, 0x7632u);
+        v.w = __byte_perm(o.z, o.w, 0x7632u);
+    } else {
+        const bool up = lane >> (t - 3) & 1;
+        const uint32_t r0 = __shfl_xor_sync(0xffffffffu, up ? v.x : v.z, 1 << (t - 3));
+        const uint32_t r1 = __shfl_xor_sync(0xffffffffu, up ? v.y : v.w, 1 << (t - 3));
+        v.x = up ? r0 : v.x;
+        v.y = up ? r1 : v.y;
+        v.z = up ? v.z : r0;
+        v.w = up ? v.w : r1;
+    }
+}
+__device__ __forceinline__ void arrange_back(uint4 &v, int t, int lane) {
+    if (t == 0) {
+        const uint4 o = v;
+        v.x = __byte_perm(o.x, o.z, 0x5410u);
+        v.y = __byte_perm(o.x, o.z, 0x7632u);
+        v.z = __byte_perm(o.y, o.w, 0x5410u);
+        v.w = __byte_perm(o.y, o.w, 0x7632u);
+    } else {
+        arrange(v, t, lane);
+    }
+}
+
+// Control mask of the four rearranged pairs of a lane (bit p: pair p's
+// amplitudes have bit c of the in-block index set; all ones without a
+// control).
+__device__ __forceinline__ uint32_t pair_ctl(int t, int c, int lane) {
+    if (c < 0) return 15u;
+    uint32_t m = 0;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+        const int k = p >> 1, h = p & 1;
+        const bool up = t >= 3 && (lane >> (t - 3) & 1);
+        const int j = t == 2 ? 2 * k + h : t == 1 ? 4 * k + h : t == 0 ? 4 * k + 2 * h : (up ? 4 : 0) + 2 * k + h;
+        if ((lane * 8 + j) >> c & 1) m |= 1u << p;
+    }
+    return m;
+}
+// Control mask of a lane's 8 amplitudes.
+__device__ __forceinline__ uint32_t amp_ctl(int c, int lane) {
+    if (c < 0) return 255u;
+    if (c >= 3) return lane >> (c - 3) & 1 ? 255u : 0u;
+    return c == 0 ? 0xAAu : c == 1 ? 0xCCu : 0xF0u;
+}
+
+template <int SHAPE, bool CTL>
+__device__ __forceinline__ void gate2_sel(const Mat2<SHAPE> &m, Amp2 &a, Amp2 &b, uint32_t bits) {
+    if constexpr (CTL)
+        gate2_ctl<SHAPE>(m, a, b, bits);
+    else
+        gate2<SHAPE>(m, a, b);
+}
+
+// The rearranged words of a block, decoded and updated; returns the lane's
+// absolute maximum.  cm: pair_ctl.
+template <int SHAPE, bool CTL>
+__device__ __forceinline__ float update_in(const DecTable &dec, const Mat2<SHAPE> &m, uint32_t cm, const uint4 &v,
+                                           float s, Amp2 (&x)[4]) {
+    const F2 s2 = dup2(s);
+    dec(v.x, s2, x[0]);
+    dec(v.y, s2, x[1]);
+    dec(v.z, s2, x[2]);
+    dec(v.w, s2, x[3]);
+    gate2_sel<SHAPE, CTL>(m, x[0], x[2], cm);
+    gate2_sel<SHAPE, CTL>(m, x[1], x[3], cm >> 2);
+    float mx = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) mx = amp_max(mx, x[k]);
+    return mx;
+}
+__device__ __forceinline__ uint4 as_u4(const int4 &v) {
+    return make_uint4(uint32_t(v.x), uint32_t(v.y), uint32_t(v.z), uint32_t(v.w));
+}
+
+// One in-block gate on a block: codes v, scale s.
+template <int SHAPE, bool CTL>
+__device__ __forceinline__ void block_gate_in(const DecTable &dec, const Mat2<SHAPE> &m, int t, uint32_t cm, int lane, uint4 &v, float &s) {
+    arrange(v, t, lane);
+    Lane8 x;
+    s = warp_max(update_in<SHAPE, CTL>(dec, m, cm, v, s, x.w));
+    v = as_u4(encode_lane(x, s));
+    arrange_back(v, t, lane);
+}
+
+// The same on two blocks at once (independent instructions to issue).
+template <int SHAPE, bool CTL>
+__device__ __forceinline__ void block_gate_in2(const DecTable &dec, const Mat2<SHAPE> &m, int t, uint32_t cm, int lane, uint4 &v0, float &s0,
+                                               uint4 &v1, float &s1) {
+    arrange(v0, t, lane);
+    arrange(v1, t, lane);
+    Amp2 x[4], y[4];
+    const float m0 = update_in<SHAPE, CTL>(dec, m, cm, v0, s0, x), m1 = update_in<SHAPE, CTL>(dec, m, cm, v1, s1, y);
+    s0 = warp_max(m0);
+    s1 = warp_max(m1);
+    int4 e0, e1;
+    encode_two(x, s0, y, s1, lane, e0, e1);
+    v0 = as_u4(e0);
+    v1 = as_u4(e1);
+    arrange_back(v0, t, lane);
+    arrange_back(v1, t, lane);
+}
+
+// One gate on a pair of blocks that differ in the target bit.  ENC_DIAG1
+// leaves the lower block as it is: its codes are not needed.
+template <int SHAPE, bool CTL>
+__device__ __forceinline__ void block_gate_pair(const DecTable &dec, const Mat2<SHAPE> &m, uint32_t cm, int lane, int4 &v0, float &s0,
+                                                int4 &v1, float &s1) {
+    Lane8 x, y;
+    if constexpr (SHAPE != ENC_DIAG1) decode_lane(dec, v0, s0, x);
+    decode_lane(dec, v1, s1, y);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        // low bytes of the four sums: (re, im) of amplitudes 2k and 2k + 1
-        const uint32_t lo = __byte_perm(enc_bits(x.re[2 * k], inv), enc_bits(x.im[2 * k], inv), 0x0040u);
-        const uint32_t hi = __byte_perm(enc_bits(x.re[2 * k + 1], inv), enc_bits(x.im[2 * k + 1], inv), 0x0040u);
-        w[k] = __byte_perm(lo, hi, 0x5410u);
+        if constexpr (SHAPE == ENC_DIAG1) x.w[k] = y.w[k];  // not used by the update
+        gate2_sel<SHAPE, CTL>(m, x.w[k], y.w[k], cm >> (2 * k));
     }
-    return make_int4(int(w[0]), int(w[1]), int(w[2]), int(w[3]));
-}
-
-// Does amplitude j of this lane (in-block index lane*8 + j) satisfy the control?
-__device__ __forceinline__ bool ctl_ok(int c, int lane, int j) {
-    if (c < 0 || c >= kEncBlockLog2) return true;
-    const int idx = lane * 8 + j;
-    return (idx >> c) & 1;
-}
-
-// Pairs inside a lane (target bit TB < 8 of the lane's 8 amplitudes); the
-// bit is a compile-time constant so the registers are indexed statically.
-template <int SHAPE, int TB>
-__device__ __forceinline__ void lane_pairs(const EncGateArgs &a, int lane, Lane8 &x) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        if (j & TB) continue;
-        if (!ctl_ok(a.c, lane, j)) continue;
-        gate_pair_s<SHAPE>(a.u, x.re[j], x.im[j], x.re[j | TB], x.im[j | TB]);
+    if constexpr (SHAPE != ENC_DIAG1) {
+        s0 = warp_max(lane_absmax(x));
+        s1 = warp_max(lane_absmax(y));
+        encode_two(x.w, s0, y.w, s1, lane, v0, v1);
+    } else {
+        s1 = warp_max(lane_absmax(y));
+        v1 = encode_lane(y, s1);
     }
 }
 
 // Target inside the block (t < 8).
 template <int SHAPE>
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_enc_gate_in(int4 *__restrict__ codes, float *__restrict__ scales,
+__global__ void __launch_bounds__(32 * kGateWarps, 3) k_enc_gate_in(uint4 *__restrict__ codes, float *__restrict__ scales,
                                                                    EncGateArgs a) {
-    __shared__ float tab[kTabFloats];
-    load_table(tab);
+    extern __shared__ __align__(16) unsigned char smem[];
+    fill_table(smem);
+    __syncthreads();
     const int lane = threadIdx.x & 31;
-    const uint64_t wid = uint64_t(blockIdx.x) * kWarpsPerCta + (threadIdx.x >> 5);
-    const uint64_t nw = uint64_t(gridDim.x) * kWarpsPerCta;
+    const DecTable dec{smem, uint32_t(lane) * 4u};
+    const uint64_t wid = uint64_t(blockIdx.x) * kGateWarps + (threadIdx.x >> 5);
+    const uint64_t nw = uint64_t(gridDim.x) * kGateWarps;
+    const Mat2<SHAPE> m(a.u);
+    const bool ctl = a.c >= 0 && a.c < kEncBlockLog2;
+    const uint32_t cm = pair_ctl(a.t, ctl ? a.c : -1, lane);
     for (uint64_t w = wid; w < a.nwork; w += nw) {
-        uint64_t b = w;
-        b = insert_zeros(b, a.nins, a.ins[0], a.ins[1]);
-        b |= a.set_mask;
-        int4 raw = codes[b * 32 + lane];
-        const float s = scales[b];
-        Lane8 x;
-        decode_lane(raw, s, tab, lane, x);
-        if (a.t < 3) {
-            if (a.t == 0)
-                lane_pairs<SHAPE, 1>(a, lane, x);
-            else if (a.t == 1)
-                lane_pairs<SHAPE, 2>(a, lane, x);
-            else
-                lane_pairs<SHAPE, 4>(a, lane, x);
-        } else {
-            const int lb = 1 << (a.t - 3);
-            const bool upper = lane & lb;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float pr = __shfl_xor_sync(0xffffffffu, x.re[j], lb);
-                const float pi = __shfl_xor_sync(0xffffffffu, x.im[j], lb);
-                if (!ctl_ok(a.c, lane, j)) continue;
-                float ar = upper ? pr : x.re[j], ai = upper ? pi : x.im[j];
-                float br = upper ? x.re[j] : pr, bi = upper ? x.im[j] : pi;
-                gate_pair_s<SHAPE>(a.u, ar, ai, br, bi);
-                x.re[j] = upper ? br : ar;
-                x.im[j] = upper ? bi : ai;
-            }
-        }
-        const float ns = warp_max(lane_absmax(x));
-        codes[b * 32 + lane] = encode_lane(x, ns);
-        if (lane == 0) scales[b] = ns;
+        const uint64_t b = insert_zeros(w, a.nins, a.ins[0], a.ins[1]) | a.set_mask;
+        uint4 v = codes[b * 32 + lane];
+        float s = scales[b];
+        if (ctl)
+            block_gate_in<SHAPE, true>(dec, m, a.t, cm, lane, v, s);
+        else
+            block_gate_in<SHAPE, false>(dec, m, a.t, cm, lane, v, s);
+        codes[b * 32 + lane] = v;
+        if (lane == 0) scales[b] = s;
     }
 }
+
+// CTAs per SM by matrix shape: the pair of blocks of a full update takes 64
+// registers per thread, the single block of ENC_DIAG1 fits 3 CTAs.
+constexpr int kAcrossCtas[4] = {2, 2, 2, 3};
 
 // Target across blocks (t >= 8): the warp holds block b0 and b0 + 2^(t-8).
+// A diagonal gate with u00 = 1 (T, P, ...) keeps the blocks with the target
+// bit 0, hence their scale and codes (decoding and re-encoding with an
+// unchanged scale is the identity), so ENC_DIAG1 reads and rewrites only the
+// blocks with the target bit 1: half the traffic, the same codes.
 template <int SHAPE>
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_enc_gate_across(int4 *__restrict__ codes,
+__global__ void __launch_bounds__(32 * kGateWarps, kAcrossCtas[SHAPE]) k_enc_gate_across(int4 *__restrict__ codes,
                                                                        float *__restrict__ scales, EncGateArgs a) {
-    __shared__ float tab[kTabFloats];
-    load_table(tab);
+    extern __shared__ __align__(16) unsigned char smem[];
+    fill_table(smem);
+    __syncthreads();
     const int lane = threadIdx.x & 31;
-    const uint64_t wid = uint64_t(blockIdx.x) * kWarpsPerCta + (threadIdx.x >> 5);
-    const uint64_t nw = uint64_t(gridDim.x) * kWarpsPerCta;
+    const DecTable dec{smem, uint32_t(lane) * 4u};
+    const uint64_t wid = uint64_t(blockIdx.x) * kGateWarps + (threadIdx.x >> 5);
+    const uint64_t nw = uint64_t(gridDim.x) * kGateWarps;
+    const Mat2<SHAPE> m(a.u);
+    const bool ctl = a.c >= 0 && a.c < kEncBlockLog2;
+    const uint32_t cm = amp_ctl(ctl ? a.c : -1, lane);
     for (uint64_t w = wid; w < a.nwork; w += nw) {
-        uint64_t b0 = w;
-        b0 = insert_zeros(b0, a.nins, a.ins[0], a.ins[1]);
-        b0 |= a.set_mask;
+        const uint64_t b0 = insert_zeros(w, a.nins, a.ins[0], a.ins[1]) | a.set_mask;
         const uint64_t b1 = b0 | a.tbit;
-        int4 r0 = codes[b0 * 32 + lane], r1 = codes[b1 * 32 + lane];
-        const float s0 = scales[b0], s1 = scales[b1];
-        Lane8 x, y;
-        decode_lane(r0, s0, tab, lane, x);
-        decode_lane(r1, s1, tab, lane, y);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (!ctl_ok(a.c, lane, j)) continue;
-            gate_pair_s<SHAPE>(a.u, x.re[j], x.im[j], y.re[j], y.im[j]);
+        int4 v0 = make_int4(0, 0, 0, 0), v1 = codes[b1 * 32 + lane];
+        float s0 = 0.0f, s1 = scales[b1];
+        if constexpr (SHAPE != ENC_DIAG1) {
+            v0 = codes[b0 * 32 + lane];
+            s0 = scales[b0];
         }
-        const float n0 = warp_max(lane_absmax(x));
-        const float n1 = warp_max(lane_absmax(y));
-        codes[b0 * 32 + lane] = encode_lane(x, n0);
-        codes[b1 * 32 + lane] = encode_lane(y, n1);
-        if (lane == 0) {
-            scales[b0] = n0;
-            scales[b1] = n1;
+        if (ctl)
+            block_gate_pair<SHAPE, true>(dec, m, cm, lane, v0, s0, v1, s1);
+        else
+            block_gate_pair<SHAPE, false>(dec, m, cm, lane, v0, s0, v1, s1);
+        if constexpr (SHAPE != ENC_DIAG1) {
+            codes[b0 * 32 + lane] = v0;
+            if (lane == 0) scales[b0] = s0;
         }
-    }
-}
-
-// Diagonal gate with u00 = 1 (T, P, ...) on a target at or above bit 8: the
-// blocks with the target bit 0 keep their amplitudes, hence their scale and
-// codes (decoding and re-encoding with an unchanged scale is the identity), so
-// only the blocks with the target bit 1 are read and rewritten: half the
-// traffic of the block-pair kernel, the same codes.
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_enc_phase_blocks(int4 *__restrict__ codes,
-                                                                        float *__restrict__ scales, EncGateArgs a) {
-    __shared__ float tab[kTabFloats];
-    load_table(tab);
-    const int lane = threadIdx.x & 31;
-    const uint64_t wid = uint64_t(blockIdx.x) * kWarpsPerCta + (threadIdx.x >> 5);
-    const uint64_t nw = uint64_t(gridDim.x) * kWarpsPerCta;
-    for (uint64_t w = wid; w < a.nwork; w += nw) {
-        const uint64_t b = insert_zeros(w, a.nins, a.ins[0], a.ins[1]) | a.set_mask | a.tbit;
-        const int4 raw = codes[b * 32 + lane];
-        const float s = scales[b];
-        Lane8 y;
-        decode_lane(raw, s, tab, lane, y);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (!ctl_ok(a.c, lane, j)) continue;
-            float ar = 0.0f, ai = 0.0f;  // the lower amplitude is left out (u00 = 1, u01 = u10 = 0)
-            gate_pair_s<ENC_DIAG1>(a.u, ar, ai, y.re[j], y.im[j]);
-        }
-        const float ns = warp_max(lane_absmax(y));
-        codes[b * 32 + lane] = encode_lane(y, ns);
-        if (lane == 0) scales[b] = ns;
+        codes[b1 * 32 + lane] = v1;
+        if (lane == 0) scales[b1] = s1;
     }
 }
 
@@ -340,9 +561,12 @@ __global__ void k_enc_gate_small(signed char *codes, float *scales, int n, EncGa
     }
 }
 
-// c64 -> codes: one warp per block (n >= 8).
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_encode(const float4 *__restrict__ psi, int4 *__restrict__ codes,
-                                                              float *__restrict__ scales, uint64_t nblocks) {
+// c64 -> codes: one warp per block (n >= 8).  Word w of a block (amplitudes
+// 2w, 2w + 1) goes to lane w % 32, so every 16-byte load and 4-byte store of
+// the warp is contiguous.
+__global__ void __launch_bounds__(32 * kWarpsPerCta) k_encode(const float4 *__restrict__ psi,
+                                                              uint32_t *__restrict__ codes, float *__restrict__ scales,
+                                                              uint64_t nblocks) {
     const int lane = threadIdx.x & 31;
     const uint64_t wid = uint64_t(blockIdx.x) * kWarpsPerCta + (threadIdx.x >> 5);
     const uint64_t nw = uint64_t(gridDim.x) * kWarpsPerCta;
@@ -350,32 +574,41 @@ __global__ void __launch_bounds__(32 * kWarpsPerCta) k_encode(const float4 *__re
         Lane8 x;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float4 v = psi[(b * 256 + lane * 8) / 2 + k];
-            x.re[2 * k] = v.x;
-            x.im[2 * k] = v.y;
-            x.re[2 * k + 1] = v.z;
-            x.im[2 * k + 1] = v.w;
+            const float4 v = psi[b * 128 + k * 32 + lane];
+            x.w[k].re = pk(v.x, v.z);
+            x.w[k].im = pk(v.y, v.w);
         }
         const float s = warp_max(lane_absmax(x));
-        codes[b * 32 + lane] = encode_lane(x, s);
+        const int4 e = encode_lane(x, s);
+        codes[b * 128 + lane] = uint32_t(e.x);
+        codes[b * 128 + 32 + lane] = uint32_t(e.y);
+        codes[b * 128 + 64 + lane] = uint32_t(e.z);
+        codes[b * 128 + 96 + lane] = uint32_t(e.w);
         if (lane == 0) scales[b] = s;
     }
 }
 
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_decode(const int4 *__restrict__ codes,
+// The same word order: contiguous 4-byte loads, contiguous 16-byte stores.
+__global__ void __launch_bounds__(32 * kWarpsPerCta) k_decode(const uint32_t *__restrict__ codes,
                                                               const float *__restrict__ scales,
                                                               float4 *__restrict__ psi, uint64_t nblocks) {
-    __shared__ float tab[kTabFloats];
-    load_table(tab);
     const int lane = threadIdx.x & 31;
     const uint64_t wid = uint64_t(blockIdx.x) * kWarpsPerCta + (threadIdx.x >> 5);
     const uint64_t nw = uint64_t(gridDim.x) * kWarpsPerCta;
     for (uint64_t b = wid; b < nblocks; b += nw) {
-        Lane8 x;
-        decode_lane(codes[b * 32 + lane], scales[b], tab, lane, x);
+        const F2 s2 = dup2(scales[b]);
+        uint32_t w[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            psi[(b * 256 + lane * 8) / 2 + k] = make_float4(x.re[2 * k], x.im[2 * k], x.re[2 * k + 1], x.im[2 * k + 1]);
+        for (int k = 0; k < 4; ++k) w[k] = codes[b * 128 + k * 32 + lane];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            Amp2 x;
+            dec_word(clamp_codes(w[k]), s2, x);
+            float4 v;
+            upk(x.re, v.x, v.z);
+            upk(x.im, v.y, v.w);
+            psi[b * 128 + k * 32 + lane] = v;
+        }
     }
 }
 
@@ -451,6 +684,7 @@ __global__ void __launch_bounds__(256) k_enc_xin(uint4 *__restrict__ codes, EncG
     const int lane = threadIdx.x & 31;
     const uint64_t wid = uint64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
     const uint64_t nw = uint64_t(gridDim.x) * 8;
+    const uint32_t cm = amp_ctl(a.c < kEncBlockLog2 ? a.c : -1, lane);
     for (uint64_t w = wid; w < a.nwork; w += nw) {
         uint64_t b = w;
         b = insert_zeros(b, a.nins, a.ins[0], a.ins[1]);
@@ -478,7 +712,7 @@ __global__ void __launch_bounds__(256) k_enc_xin(uint4 *__restrict__ codes, EncG
             uint32_t bm = 0;
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-                if (ctl_ok(a.c, lane, 2 * k + h)) bm |= 0xFFFFu << (16 * h);
+                if (cm >> (2 * k + h) & 1u) bm |= 0xFFFFu << (16 * h);
             out[k] = (xv[k] & ~bm) | (xp[k] & bm);
         }
         codes[b * 32 + lane] = make_uint4(out[0], out[1], out[2], out[3]);
@@ -508,93 +742,217 @@ __global__ void __launch_bounds__(256) k_enc_xblocks(uint4 *__restrict__ codes, 
     }
 }
 
-// ---------------------------------------------------------------- runs of in-block gates
-// A run of consecutive gates that each act inside blocks (2x2 updates with a
-// target below bit 8, any control) or are sign flips (+-1 diagonals on any
-// qubits) is applied in one pass: each warp holds one block's codes and
-// scale in registers and goes through the run in circuit order.  A gate is
-// the same decode -> FP32 update -> block maximum -> encode as in
-// k_enc_gate_in (the same functions, in the same order), and a flip negates
-// codes as k_enc_flip does, so every block's codes and scale after the run
-// are those of the gates applied one pass at a time: bit-exact.  A gate whose
-// block-level control is 0 leaves the block as it is (decoding and
-// re-encoding with an unchanged scale is the identity).
+// ---------------------------------------------------------------- runs of gates
+// A run of consecutive gates goes through one pass: each warp holds a tile of
+// 2^B blocks (the blocks that differ in B chosen block-index bits) and applies
+// every gate of the run whose target is an in-block qubit or one of those
+// bits, and every sign flip, in circuit order.  A gate is the same decode ->
+// FP32 update -> block maximum -> encode as in its own pass (the same
+// functions), so every block's codes and scale after the run are those of the
+// gates applied one pass at a time: bit-exact.  A gate whose block-level
+// control is 0 leaves the block as it is (decoding and re-encoding with an
+// unchanged scale is the identity).
+//
+// The tile's codes sit in shared memory, 16 bytes per lane and block, and are
+// only ever touched by their own lane (gates across blocks keep the lane,
+// in-block ones exchange codes by shuffles), so no gate needs a barrier; lane
+// k holds the scale of block k.  Bound: instruction issue (66-69% active, FMA
+// pipe 59%, ALU pipe 51%) on about 150 instructions per block and gate; the
+// HBM traffic, 1 KB per block and run, hides behind it.  B = 4: 8 KB per warp
+// and the 64 KB table leave 16 warps on an SM at 128 registers.  (Decoding by
+// arithmetic instead of the table: 11.7 against 11.0 ms on 27 qubits and 160
+// gates; 24 warps at 80 registers: spills, 11.9 against 11.7.)
 
-template <int SHAPE>
-__device__ __forceinline__ void run_gate_in(const EncRunOp &op, int lane, Lane8 &x) {
-    EncGateArgs a{};
-    a.t = op.t;
-    a.c = op.c;
+constexpr int kRunWarps = 16;
+
+struct EncRunArgs {
+    uint64_t ntiles;
+    int nops, nbits;
+    int pos[kEncRunMaxBits];  // ascending block-index positions of the tile bits
+};
+
+// Negate the codes of the amplitudes in the 8-bit mask m (bytewise, 0 - q).
+__device__ __forceinline__ uint4 flip_codes(uint4 v, uint32_t m) {
+    uint32_t *x = reinterpret_cast<uint32_t *>(&v);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) a.u[k] = op.u[k];
-    if (op.t < 3) {
-        if (op.t == 0)
-            lane_pairs<SHAPE, 1>(a, lane, x);
-        else if (op.t == 1)
-            lane_pairs<SHAPE, 2>(a, lane, x);
-        else
-            lane_pairs<SHAPE, 4>(a, lane, x);
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t bm = (m >> (2 * k) & 1u ? 0x0000FFFFu : 0u) | (m >> (2 * k + 1) & 1u ? 0xFFFF0000u : 0u);
+        const uint32_t a = x[k] ^ bm, one = bm & 0x01010101u;  // ~q + 1 in the masked bytes, no carry between bytes
+        x[k] = ((a & 0x7f7f7f7fu) + one) ^ (a & 0x80808080u);
+    }
+    return v;
+}
+
+// The gate `op` on every block (or pair of blocks) of the tile that meets its
+// block-level condition.  base: block index of the tile; tile block k is
+// base | spread[k].  In-block gates take two blocks at a time.
+template <int SHAPE, bool CTL>
+__device__ __forceinline__ void run_gate(const DecTable &dec, const EncRunOp &op, uint4 *tile, float &sc, uint32_t base,
+                                         const uint32_t *spread, int nblk, int lane) {
+    const Mat2<SHAPE> m(op.u);
+    const uint32_t hm = uint32_t(op.hi_mask), hv = uint32_t(op.hi_val);
+    const int t = op.t;
+    uint4 *mine = tile + lane;
+    if (op.kind == ENC_OP_IN) {
+        const uint32_t cm = pair_ctl(t, op.c, lane);
+        for (int k0 = 0; k0 < nblk; k0 += 2) {
+            const int k1 = nblk > 1 ? k0 + 1 : 0;
+            const bool on0 = ((base | spread[k0]) & hm) == hv, on1 = ((base | spread[k1]) & hm) == hv;
+            if (!on0 && !on1) continue;
+            uint4 v0 = mine[k0 * 32], v1 = mine[k1 * 32];
+            float s0 = __shfl_sync(0xffffffffu, sc, k0), s1 = __shfl_sync(0xffffffffu, sc, k1);
+            block_gate_in2<SHAPE, CTL>(dec, m, t, cm, lane, v0, s0, v1, s1);
+            if (on0) {
+                mine[k0 * 32] = v0;
+                sc = lane == k0 ? s0 : sc;
+            }
+            if (on1) {
+                mine[k1 * 32] = v1;
+                sc = lane == k1 ? s1 : sc;
+            }
+        }
     } else {
-        const int lb = 1 << (op.t - 3);
-        const bool upper = lane & lb;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float pr = __shfl_xor_sync(0xffffffffu, x.re[j], lb);
-            const float pi = __shfl_xor_sync(0xffffffffu, x.im[j], lb);
-            if (!ctl_ok(a.c, lane, j)) continue;
-            float ar = upper ? pr : x.re[j], ai = upper ? pi : x.im[j];
-            float br = upper ? x.re[j] : pr, bi = upper ? x.im[j] : pi;
-            gate_pair_s<SHAPE>(a.u, ar, ai, br, bi);
-            x.re[j] = upper ? br : ar;
-            x.im[j] = upper ? bi : ai;
+        const uint32_t cm = amp_ctl(op.c, lane);
+        const int hi = 1 << t;
+        for (int k0 = 0; k0 < nblk; k0 = ((k0 | hi) + 1) & ~hi) {
+            const int k1 = k0 | hi;
+            if (((base | spread[k0]) & hm) != hv) continue;
+            int4 v0 = make_int4(0, 0, 0, 0), v1 = *reinterpret_cast<const int4 *>(mine + k1 * 32);
+            float s0 = 0.0f, s1 = __shfl_sync(0xffffffffu, sc, k1);
+            if (SHAPE != ENC_DIAG1) {
+                v0 = *reinterpret_cast<const int4 *>(mine + k0 * 32);
+                s0 = __shfl_sync(0xffffffffu, sc, k0);
+            }
+            block_gate_pair<SHAPE, CTL>(dec, m, cm, lane, v0, s0, v1, s1);
+            if (SHAPE != ENC_DIAG1) {
+                mine[k0 * 32] = as_u4(v0);
+                sc = lane == k0 ? s0 : sc;
+            }
+            mine[k1 * 32] = as_u4(v1);
+            sc = lane == k1 ? s1 : sc;
         }
     }
 }
 
-__global__ void __launch_bounds__(32 * kWarpsPerCta) k_enc_run_in(int4 *__restrict__ codes, float *__restrict__ scales,
-                                                                  uint64_t nblocks, const EncRunOp *__restrict__ gops,
-                                                                  int nops) {
-    __shared__ float tab[kTabFloats];
+template <int NB>  // tile bits, or -1: a.nbits
+__global__ void __launch_bounds__(32 * kRunWarps, 1) k_enc_run_in(uint4 *__restrict__ codes,
+                                                                     float *__restrict__ scales,
+                                                                     const EncRunOp *__restrict__ gops,
+                                                                     const EncRunArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
     __shared__ EncRunOp ops[kEncRunMaxOps];
-    for (int i = threadIdx.x; i < nops; i += blockDim.x) ops[i] = gops[i];
-    load_table(tab);  // (its barrier also publishes the ops)
+    __shared__ uint32_t spread[1 << kEncRunMaxBits];
+    const int nblk = NB >= 0 ? 1 << NB : 1 << a.nbits;
+    fill_table(smem);
+    for (int i = threadIdx.x; i < a.nops; i += blockDim.x) ops[i] = gops[i];
+    if (threadIdx.x < nblk) {
+        uint32_t s = 0;
+#pragma unroll
+        for (int j = 0; j < kEncRunMaxBits; ++j)
+            if (j < a.nbits && (threadIdx.x >> j & 1u)) s |= 1u << a.pos[j];
+        spread[threadIdx.x] = s;
+    }
+    __syncthreads();
     const int lane = threadIdx.x & 31;
-    const uint64_t wid = uint64_t(blockIdx.x) * kWarpsPerCta + (threadIdx.x >> 5);
-    const uint64_t nw = uint64_t(gridDim.x) * kWarpsPerCta;
-    for (uint64_t b = wid; b < nblocks; b += nw) {
-        int4 raw = codes[b * 32 + lane];
-        float s = scales[b];
-        for (int i = 0; i < nops; ++i) {
+    const DecTable dec{smem, uint32_t(lane) * 4u};
+    uint4 *tile = reinterpret_cast<uint4 *>(smem + kTabBytes) + (threadIdx.x >> 5) * (nblk * 32);
+    const uint64_t wid = uint64_t(blockIdx.x) * kRunWarps + (threadIdx.x >> 5);
+    const uint64_t nw = uint64_t(gridDim.x) * kRunWarps;
+    for (uint64_t w = wid; w < a.ntiles; w += nw) {
+        uint64_t b64 = w;
+#pragma unroll
+        for (int j = 0; j < kEncRunMaxBits; ++j)
+            if (NB == kEncRunMaxBits || j < a.nbits) b64 = insert_zero(b64, a.pos[j]);
+        const uint32_t base = uint32_t(b64);  // at most 2^32 blocks (n <= 40)
+        const uint32_t mine = base | spread[lane & (nblk - 1)];
+        float sc = scales[mine];
+#pragma unroll
+        for (int k = 0; k < nblk; ++k) {
+            tile[k * 32 + lane] = codes[uint64_t(base | spread[k]) * 32 + lane];
+        }
+        for (int i = 0; i < a.nops; ++i) {
             const EncRunOp &op = ops[i];
-            if ((b & op.hi_mask) != op.hi_val) continue;  // block-level condition not met
-            if (op.kind == 1) {  // sign flip of the codes whose in-block bits match
-                uint32_t *x = reinterpret_cast<uint32_t *>(&raw);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    uint32_t bm = 0;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint32_t idx = uint32_t(lane) * 8 + 2 * k + h;
-                        if ((idx & op.lo_mask) == op.lo_val) bm |= 0xFFFFu << (16 * h);
+            if (op.kind == ENC_OP_FLIP) {
+                // the consecutive flips from here on: one mask per block, applied once
+                int e = i + 1;
+                while (e < a.nops && ops[e].kind == ENC_OP_FLIP) ++e;
+                for (int k = 0; k < nblk; ++k) {
+                    const uint32_t b = base | spread[k];
+                    uint32_t m = 0;
+                    for (int f = i; f < e; ++f) {
+                        const EncRunOp &g = ops[f];
+                        const bool on = (b & uint32_t(g.hi_mask)) == uint32_t(g.hi_val) &&
+                                        (uint32_t(lane * 8) & g.lo_mask & 0xF8u) == (g.lo_val & 0xF8u);
+                        m ^= on ? g.amps : 0u;
                     }
-                    x[k] = (x[k] & ~bm) | (__vneg4(x[k]) & bm);
+                    if (__any_sync(0xffffffffu, m != 0)) tile[k * 32 + lane] = flip_codes(tile[k * 32 + lane], m);
+                }
+                i = e - 1;
+                continue;
+            }
+            if (op.kind == ENC_OP_SWAP) {  // X on a tile bit: the blocks change places
+                const uint32_t hm = uint32_t(op.hi_mask), hv = uint32_t(op.hi_val);
+                for (int k = 0; k < nblk; ++k) {
+                    const int k1 = k | (1 << op.t);
+                    if (k == k1 || ((base | spread[k]) & hm) != hv) continue;
+                    const uint4 v = tile[k * 32 + lane];
+                    tile[k * 32 + lane] = tile[k1 * 32 + lane];
+                    tile[k1 * 32 + lane] = v;
+                    const float s0 = __shfl_sync(0xffffffffu, sc, k), s1 = __shfl_sync(0xffffffffu, sc, k1);
+                    sc = lane == k ? s1 : lane == k1 ? s0 : sc;
                 }
                 continue;
             }
-            Lane8 x;
-            decode_lane(raw, s, tab, lane, x);
             switch (op.shape) {
-                case ENC_REAL: run_gate_in<ENC_REAL>(op, lane, x); break;
-                case ENC_DIAG: run_gate_in<ENC_DIAG>(op, lane, x); break;
-                case ENC_DIAG1: run_gate_in<ENC_DIAG1>(op, lane, x); break;
-                default: run_gate_in<ENC_GENERAL>(op, lane, x); break;
+                case ENC_REAL:
+                    if (op.c >= 0)
+                        run_gate<ENC_REAL, true>(dec, op, tile, sc, base, spread, nblk, lane);
+                    else
+                        run_gate<ENC_REAL, false>(dec, op, tile, sc, base, spread, nblk, lane);
+                    break;
+                case ENC_DIAG:
+                    if (op.c >= 0)
+                        run_gate<ENC_DIAG, true>(dec, op, tile, sc, base, spread, nblk, lane);
+                    else
+                        run_gate<ENC_DIAG, false>(dec, op, tile, sc, base, spread, nblk, lane);
+                    break;
+                case ENC_DIAG1:
+                    if (op.c >= 0)
+                        run_gate<ENC_DIAG1, true>(dec, op, tile, sc, base, spread, nblk, lane);
+                    else
+                        run_gate<ENC_DIAG1, false>(dec, op, tile, sc, base, spread, nblk, lane);
+                    break;
+                default:
+                    if (op.c >= 0)
+                        run_gate<ENC_GENERAL, true>(dec, op, tile, sc, base, spread, nblk, lane);
+                    else
+                        run_gate<ENC_GENERAL, false>(dec, op, tile, sc, base, spread, nblk, lane);
+                    break;
             }
-            s = warp_max(lane_absmax(x));
-            raw = encode_lane(x, s);
         }
-        codes[b * 32 + lane] = raw;
-        if (lane == 0) scales[b] = s;
+#pragma unroll
+        for (int k = 0; k < nblk; ++k) codes[uint64_t(base | spread[k]) * 32 + lane] = tile[k * 32 + lane];
+        if (lane < nblk) scales[mine] = sc;
     }
+}
+
+// Dynamic shared memory above 48 KB: the decode table, and the tiles of a run.
+cudaError_t enc_attrs(int device) {
+    static std::atomic<uint64_t> configured{0};
+    if (!attrs_needed(configured, device)) return cudaSuccess;
+    auto set = [](auto *fn, int bytes) {
+        return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    };
+    const int run = kTabBytes + kRunWarps * (512 << kEncRunMaxBits);  // 192 KB
+    for (const cudaError_t e :
+         {set(k_enc_gate_in<ENC_GENERAL>, kTabBytes), set(k_enc_gate_in<ENC_REAL>, kTabBytes),
+          set(k_enc_gate_in<ENC_DIAG>, kTabBytes), set(k_enc_gate_in<ENC_DIAG1>, kTabBytes),
+          set(k_enc_gate_across<ENC_GENERAL>, kTabBytes), set(k_enc_gate_across<ENC_REAL>, kTabBytes),
+          set(k_enc_gate_across<ENC_DIAG>, kTabBytes), set(k_enc_gate_across<ENC_DIAG1>, kTabBytes),
+          set(k_enc_run_in<kEncRunMaxBits>, run), set(k_enc_run_in<-1>, run)})
+        if (e != cudaSuccess) return e;
+    attrs_set(configured, device);
+    return cudaSuccess;
 }
 
 int enc_grid(uint64_t nwork) {
@@ -664,6 +1022,7 @@ cudaError_t launch_enc_gate1(sv_state *h, const Gate1 &g) {
     a.nins = ni;
     a.nwork = uint64_t(1) << (nb_log - ni);
     int4 *codes = static_cast<int4 *>(h->data);
+    uint4 *ucodes = static_cast<uint4 *>(h->data);
     if (xgate && a.t < kEncBlockLog2) {  // permutation inside blocks
         k_enc_xin<<<enc_grid(a.nwork), 256, 0, h->stream>>>(reinterpret_cast<uint4 *>(codes), a);
         return cudaGetLastError();
@@ -677,20 +1036,27 @@ cudaError_t launch_enc_gate1(sv_state *h, const Gate1 &g) {
     const bool diag = a.u[2] == 0.0f && a.u[3] == 0.0f && a.u[4] == 0.0f && a.u[5] == 0.0f;
     const bool one = diag && a.u[0] == 1.0f && a.u[1] == 0.0f;
     const int shape = one ? ENC_DIAG1 : diag ? ENC_DIAG : real ? ENC_REAL : ENC_GENERAL;
-    const unsigned grid = enc_grid(a.nwork), block = 32 * kWarpsPerCta;
+    const cudaError_t ea = enc_attrs(h->device);
+    if (ea != cudaSuccess) return ea;
+    const uint64_t want = (a.nwork + kGateWarps - 1) / kGateWarps;
+    // persistent CTAs (each fills a decode table): 3 per SM where the registers
+    // of one block's update allow it, 2 for pairs of blocks (28 qubits: H inside
+    // the blocks 255 us against 276 us with 2, H across them 240 against 290 with 3)
+    const unsigned cap = 152u * unsigned(a.t < kEncBlockLog2 ? 3 : kAcrossCtas[shape]);
+    const unsigned grid = unsigned(want < cap ? want : cap), block = 32 * kGateWarps;
     if (a.t < kEncBlockLog2) {
         switch (shape) {
-            case ENC_REAL: k_enc_gate_in<ENC_REAL><<<grid, block, 0, h->stream>>>(codes, h->scales, a); break;
-            case ENC_DIAG: k_enc_gate_in<ENC_DIAG><<<grid, block, 0, h->stream>>>(codes, h->scales, a); break;
-            case ENC_DIAG1: k_enc_gate_in<ENC_DIAG1><<<grid, block, 0, h->stream>>>(codes, h->scales, a); break;
-            default: k_enc_gate_in<ENC_GENERAL><<<grid, block, 0, h->stream>>>(codes, h->scales, a); break;
+            case ENC_REAL: k_enc_gate_in<ENC_REAL><<<grid, block, kTabBytes, h->stream>>>(ucodes, h->scales, a); break;
+            case ENC_DIAG: k_enc_gate_in<ENC_DIAG><<<grid, block, kTabBytes, h->stream>>>(ucodes, h->scales, a); break;
+            case ENC_DIAG1: k_enc_gate_in<ENC_DIAG1><<<grid, block, kTabBytes, h->stream>>>(ucodes, h->scales, a); break;
+            default: k_enc_gate_in<ENC_GENERAL><<<grid, block, kTabBytes, h->stream>>>(ucodes, h->scales, a); break;
         }
     } else {
         switch (shape) {
-            case ENC_REAL: k_enc_gate_across<ENC_REAL><<<grid, block, 0, h->stream>>>(codes, h->scales, a); break;
-            case ENC_DIAG: k_enc_gate_across<ENC_DIAG><<<grid, block, 0, h->stream>>>(codes, h->scales, a); break;
-            case ENC_DIAG1: k_enc_phase_blocks<<<grid, block, 0, h->stream>>>(codes, h->scales, a); break;
-            default: k_enc_gate_across<ENC_GENERAL><<<grid, block, 0, h->stream>>>(codes, h->scales, a); break;
+            case ENC_REAL: k_enc_gate_across<ENC_REAL><<<grid, block, kTabBytes, h->stream>>>(codes, h->scales, a); break;
+            case ENC_DIAG: k_enc_gate_across<ENC_DIAG><<<grid, block, kTabBytes, h->stream>>>(codes, h->scales, a); break;
+            case ENC_DIAG1: k_enc_gate_across<ENC_DIAG1><<<grid, block, kTabBytes, h->stream>>>(codes, h->scales, a); break;
+            default: k_enc_gate_across<ENC_GENERAL><<<grid, block, kTabBytes, h->stream>>>(codes, h->scales, a); break;
         }
     }
     return cudaGetLastError();
@@ -716,21 +1082,25 @@ bool enc_run_op(int n, const Gate1 &g, EncRunOp *op) {
             m |= uint64_t(1) << g.target;
             if (is(u[3], -1)) v |= uint64_t(1) << g.target;
         }
-        op->kind = 1;
+        op->kind = ENC_OP_FLIP;
         op->lo_mask = uint32_t(m & 0xFFu);
         op->lo_val = uint32_t(v & 0xFFu);
         op->hi_mask = m >> kEncBlockLog2;
         op->hi_val = v >> kEncBlockLog2;
-        if (is(u[0], 1) && is(u[3], 1)) {  // identity: a flip that matches no amplitude
-            op->lo_mask = 0;
-            op->lo_val = 1;
-        }
+        if (is(u[0], 1) && is(u[3], 1)) return true;  // identity: a flip of no amplitude (amps = 0)
+        for (uint32_t j = 0; j < 8; ++j)
+            if ((j & op->lo_mask & 7u) == (op->lo_val & 7u)) op->amps |= 1u << j;
         return true;
     }
-    if (g.target >= kEncBlockLog2) return false;
-    op->kind = 0;
-    op->t = g.target;
     op->c = g.control >= 0 && g.control < kEncBlockLog2 ? g.control : -1;
+    if (g.target < kEncBlockLog2) {
+        op->kind = ENC_OP_IN;
+        op->t = g.target;
+    } else {
+        const bool x = is(u[0], 0) && is(u[3], 0) && is(u[1], 1) && is(u[2], 1);
+        op->kind = x && op->c < 0 ? ENC_OP_SWAP : ENC_OP_PAIR;
+        op->t = g.target - kEncBlockLog2;  // a block-index bit: the caller maps it to a tile bit
+    }
     if (g.control >= kEncBlockLog2) op->hi_mask = op->hi_val = uint64_t(1) << (g.control - kEncBlockLog2);
     for (int k = 0; k < 4; ++k) {
         op->u[2 * k] = float(g.u[k].re);
@@ -740,10 +1110,23 @@ bool enc_run_op(int n, const Gate1 &g, EncRunOp *op) {
     return true;
 }
 
-cudaError_t launch_enc_run(sv_state *h, const EncRunOp *d_ops, int nops) {
-    const uint64_t nb = uint64_t(1) << (h->n - kEncBlockLog2);
-    k_enc_run_in<<<enc_grid(nb), 32 * kWarpsPerCta, 0, h->stream>>>(static_cast<int4 *>(h->data), h->scales, nb,
-                                                                    d_ops, nops);
+cudaError_t launch_enc_run(sv_state *h, const EncRunOp *d_ops, int nops, int nbits, const int *pos) {
+    EncRunArgs a{};
+    a.ntiles = uint64_t(1) << (h->n - kEncBlockLog2 - nbits);
+    a.nops = nops;
+    a.nbits = nbits;
+    for (int j = 0; j < nbits; ++j) a.pos[j] = pos[j];
+    uint4 *codes = static_cast<uint4 *>(h->data);
+    const unsigned block = 32 * kRunWarps;
+    const int smem = kTabBytes + kRunWarps * (512 << nbits);
+    const cudaError_t e = enc_attrs(h->device);
+    if (e != cudaSuccess) return e;
+    const uint64_t want = (a.ntiles + kRunWarps - 1) / kRunWarps;
+    const unsigned grid = unsigned(want < 152 ? want : 152);
+    if (nbits == kEncRunMaxBits)
+        k_enc_run_in<kEncRunMaxBits><<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a);
+    else
+        k_enc_run_in<-1><<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a);
     return cudaGetLastError();
 }
 
@@ -755,7 +1138,8 @@ cudaError_t launch_encode(const sv_state *src, sv_state *dst) {
     } else {
         const uint64_t nb = uint64_t(1) << (n - kEncBlockLog2);
         k_encode<<<enc_grid(nb), 32 * kWarpsPerCta, 0, dst->stream>>>(static_cast<const float4 *>(src->data),
-                                                                      static_cast<int4 *>(dst->data), dst->scales, nb);
+                                                                      static_cast<uint32_t *>(dst->data), dst->scales,
+                                                                      nb);
     }
     return cudaGetLastError();
 }
@@ -767,7 +1151,7 @@ cudaError_t launch_decode(const sv_state *src, sv_state *dst) {
                                                   static_cast<float2 *>(dst->data), n);
     } else {
         const uint64_t nb = uint64_t(1) << (n - kEncBlockLog2);
-        k_decode<<<enc_grid(nb), 32 * kWarpsPerCta, 0, dst->stream>>>(static_cast<const int4 *>(src->data), src->scales,
+        k_decode<<<enc_grid(nb), 32 * kWarpsPerCta, 0, dst->stream>>>(static_cast<const uint32_t *>(src->data), src->scales,
                                                                       static_cast<float4 *>(dst->data), nb);
     }
     return cudaGetLastError();
@@ -801,21 +1185,30 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 // partial sums, FP64 beyond; one partial per CTA.
 __global__ void __launch_bounds__(256) k_enc_norm(const int4 *__restrict__ codes, const float *__restrict__ scales,
                                                   uint64_t nblocks, double *__restrict__ partials) {
-    __shared__ float tab[kTabFloats];
     __shared__ double sh[8];
-    load_table(tab);
     const int lane = threadIdx.x & 31;
     const uint64_t wid = uint64_t(blockIdx.x) * 8 + (threadIdx.x >> 5);
     const uint64_t nw = uint64_t(gridDim.x) * 8;
     double acc = 0.0;
     for (uint64_t b = wid; b < nblocks; b += nw) {
         Lane8 x;
-        decode_lane(codes[b * 32 + lane], scales[b], tab, lane, x);
+        const int4 c = clamp_codes(codes[b * 32 + lane]);
+        const F2 s2 = dup2(scales[b]);
+        dec_word(uint32_t(c.x), s2, x.w[0]);
+        dec_word(uint32_t(c.y), s2, x.w[1]);
+        dec_word(uint32_t(c.z), s2, x.w[2]);
+        dec_word(uint32_t(c.w), s2, x.w[3]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             float s = 0.0f;
 #pragma unroll
-            for (int j = 4 * h; j < 4 * h + 4; ++j) s = fmaf(x.re[j], x.re[j], fmaf(x.im[j], x.im[j], s));
+            for (int k = 2 * h; k < 2 * h + 2; ++k) {
+                float r0, r1, i0, i1;
+                upk(x.w[k].re, r0, r1);
+                upk(x.w[k].im, i0, i1);
+                s = fmaf(r0, r0, fmaf(i0, i0, s));
+                s = fmaf(r1, r1, fmaf(i1, i1, s));
+            }
             acc += double(s);
         }
     }

@@ -370,7 +370,7 @@ const char *gate1_kernel_name(const sv_state *h, const Gate1 &g) {
         // diagonal with u00 = 1 in the FP32 entries the kernels use: only the upper blocks
         auto zero32 = [](const Cplx &z) { return float(z.re) == 0.0f && float(z.im) == 0.0f; };
         if (zero32(u[1]) && zero32(u[2]) && float(u[0].re) == 1.0f && float(u[0].im) == 0.0f)
-            return "k_enc_phase_blocks";
+            return "k_enc_gate_across<diag1>";
         return "k_enc_gate_across";
     }
     const bool diag = g.u[1].re == 0 && g.u[1].im == 0 && g.u[2].re == 0 && g.u[2].im == 0;

@@ -1,4 +1,5 @@
 // Plan creation and replay.
+#include <algorithm>
 #include <cstdlib>
 #include <string>
 
@@ -19,7 +20,7 @@ double gate1_bytes(const sv_state *h, const Gate1 &g) {
         int blockbits = 0;
         if (g.control >= kEncBlockLog2) ++blockbits;
         const bool flip = k == "k_enc_flip";
-        if (k == "k_enc_phase_blocks") ++blockbits;  // the blocks with the target bit set
+        if (k == "k_enc_gate_across<diag1>") ++blockbits;  // the blocks with the target bit set
         if (flip) {
             const bool both = g.u[0].re == -1 && g.u[3].re == -1;
             if (!both && g.target >= kEncBlockLog2) ++blockbits;
@@ -82,10 +83,13 @@ sv_status build_fused_plan(sv_state *h, const Circuit &c, sv_plan_s *p, int kfix
     return SV_OK;
 }
 
-// Two-byte code: runs of consecutive in-block gates and sign flips become one
-// pass each (k_enc_run_in) where the run's gates, one pass each, would move
-// more bytes than one pass over the code; the other gates keep their own
-// passes.  SV_ENC_RUNS=0 keeps one pass per gate.
+// Two-byte code: a run of consecutive gates whose targets are in-block qubits
+// or at most B block bits, and sign flips, becomes one pass (k_enc_run_in)
+// where its gates, one pass each, would move more bytes than one pass over
+// the code; the other gates keep their own passes.  A warp takes a tile of
+// 2^B blocks through the whole run, so B is the largest that still leaves
+// about 2^10 tiles (7 warps per SM): B = 4 from 22 qubits on, 1 up to 19.
+// SV_ENC_RUNS=0 keeps one pass per gate.
 bool enc_runs_enabled() {
     const char *e = std::getenv("SV_ENC_RUNS");
     return !(e && e[0] == '0');
@@ -95,6 +99,8 @@ sv_status build_enc_runs(sv_state *h, sv_plan_s *p) {
     if (h->n < kEncBlockLog2 || !enc_runs_enabled()) return SV_OK;
     const double amps = double(uint64_t(1) << h->n);
     const double pass_bytes = 2.0 * amps * 2.0 + 2.0 * (amps / kEncBlock) * 4.0;
+    const int nb_log = h->n - kEncBlockLog2;
+    const int bmax = std::min(nb_log, std::max(1, std::min(kEncRunMaxBits, nb_log - 10)));
     std::vector<EncRunOp> ops;
     const size_t ng = p->pergate.size();
     size_t i = 0;
@@ -102,15 +108,27 @@ sv_status build_enc_runs(sv_state *h, sv_plan_s *p) {
         EncRunOp op;
         size_t j = i;
         double alone = 0.0;
+        std::vector<int> bits;  // block bits of the run's tiles, ascending
         while (j < ng && j - i < size_t(kEncRunMaxOps) && enc_run_op(h->n, p->pergate[j], &op)) {
+            if (op.kind == ENC_OP_PAIR || op.kind == ENC_OP_SWAP) {
+                const auto it = std::lower_bound(bits.begin(), bits.end(), op.t);
+                if (it == bits.end() || *it != op.t) {
+                    if (int(bits.size()) == bmax) break;
+                    bits.insert(it, op.t);
+                }
+            }
             alone += gate1_bytes(h, p->pergate[j]);
             ++j;
         }
         if (j - i >= 2 && alone > pass_bytes) {
             PlanLaunch l{4, int(p->encruns.size()), pass_bytes};
-            p->encruns.push_back({int(ops.size()), int(j - i), int(j - i)});
+            sv_plan_s::EncRun run{int(ops.size()), int(j - i), int(bits.size()), {0, 0, 0, 0}};
+            for (size_t k = 0; k < bits.size(); ++k) run.pos[k] = bits[k];
+            p->encruns.push_back(run);
             for (size_t k = i; k < j; ++k) {
                 enc_run_op(h->n, p->pergate[k], &op);
+                if (op.kind == ENC_OP_PAIR || op.kind == ENC_OP_SWAP)
+                    op.t = int(std::lower_bound(bits.begin(), bits.end(), op.t) - bits.begin());
                 ops.push_back(op);
             }
             p->launches.push_back(l);
@@ -181,7 +199,7 @@ cudaError_t launch_one(sv_plan_s *p, const PlanLaunch &l) {
     }
     if (l.kind == 4) {
         const sv_plan_s::EncRun &r = p->encruns[size_t(l.index)];
-        return launch_enc_run(p->h, p->d_encops + r.first, r.count);
+        return launch_enc_run(p->h, p->d_encops + r.first, r.count, r.nbits, r.pos);
     }
     return launch_jit_pass(p->h, p->tfns[size_t(l.index)], p->h->n, p->tile_rb);
 }

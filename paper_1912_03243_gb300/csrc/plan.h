@@ -47,7 +47,7 @@ const char *gate1_kernel_name(const sv_state *h, const Gate1 &g);
 struct PlanLaunch {
     int kind;      // 0: per-gate update pergate[index]; 1: compiled tile pass tfns[index];
                    // 2: tensor-core block tcargs[index]; 3: CUDA-core block blocks[index];
-                   // 4: run of in-block two-byte-code gates encruns[index]
+                   // 4: run of two-byte-code gates encruns[index]
     int index;
     double bytes;  // algorithmic bytes
     double lane_ops = 0.0;  // compiled tile passes: FP32 lane operations per amplitude (at least)
@@ -60,9 +60,10 @@ struct sv_plan_s {
     int64_t gates = 0;                     // gates of the circuit text
     std::vector<sv::Gate1> pergate;        // per-gate updates
     struct EncRun {
-        int first, count, gates;           // ops d_encops[first .. first + count), circuit gates they apply
+        int first, count;                  // ops d_encops[first .. first + count)
+        int nbits, pos[sv::kEncRunMaxBits];  // block-index bits of its tiles
     };
-    std::vector<EncRun> encruns;           // two-byte code: runs of in-block gates, one pass each
+    std::vector<EncRun> encruns;           // two-byte code: runs of gates, one pass each
     sv::EncRunOp *d_encops = nullptr;      // their ops (device)
     std::vector<void *> tfns;              // compiled tile passes
     int tile_rb = 0;                       // their register bits per thread

@@ -169,3 +169,44 @@ def test_in_block_runs_equal_one_pass_per_gate(S, monkeypatch):
         enc.free()
     assert np.array_equal(out[0][0], out[1][0])
     assert np.array_equal(out[0][1].view(np.uint32), out[1][1].view(np.uint32))
+
+
+def _mixed_on(n, qubits, count, seed):
+    """A mixed circuit (every gate kind) whose gates act on the given qubits of an n-qubit register."""
+    small = C.random_unitary_gates(len(qubits), count, seed)
+    c = C.Circuit(n)
+    for name, qs, ps in small.gates:
+        c.add(name, *(qubits[q] for q in qs), params=ps)
+    return c
+
+
+@pytest.mark.parametrize("n,blockq", [(8, []), (9, [8]), (12, [9, 11]), (17, [10, 16]), (20, [8, 19]), (21, [8, 14, 20]),
+                                      (22, [9, 13, 18, 21]), (23, [8, 9, 10, 22]), (23, [11, 12, 13, 14, 15])])
+def test_runs_across_blocks_bit_exact(S, orc, monkeypatch, n, blockq):
+    """Runs that hold gates across blocks (tiles of 1 to 16 blocks, more target
+    bits than one tile takes, X on blocks, controls inside and outside the
+    blocks and the tile) write the codes of one pass per gate, and at small n
+    those of the CPU codec mirror."""
+    circs = [_mixed_on(n, [0, 1, 2, 4, 7] + blockq, 150, n), C.random_unitary_gates(n, 60, 9 + n)]
+    psi = rand_c64(n, 5)
+    src = S.StateVector(n, "c64")
+    src.from_numpy(psi)
+    for circ in circs:
+        out = []
+        for runs in ("1", "0"):
+            monkeypatch.setenv("SV_ENC_RUNS", runs)
+            enc = S.StateVector(n, "enc2b")
+            enc.encode_from(src)
+            p = enc.plan(circ, "pergate")
+            if runs == "1":
+                assert p.passes < p.gates
+            p.execute()
+            p.free()
+            out.append(enc.codes())
+            enc.free()
+        assert np.array_equal(out[0][0], out[1][0])
+        assert np.array_equal(out[0][1].view(np.uint32), out[1][1].view(np.uint32))
+        if n <= 17:
+            rc, rs = orc.enc_run(circ, None, *orc.enc_encode(psi))
+            assert np.array_equal(out[0][0], rc)
+            assert np.array_equal(out[0][1].view(np.uint32), rs.view(np.uint32))
