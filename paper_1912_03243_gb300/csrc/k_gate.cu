@@ -59,24 +59,103 @@ __device__ __forceinline__ uint64_t expand(uint64_t w, const GateArgs<R> &a) {
     return w | a.set_mask;
 }
 
-template <typename R>
+// Form of a 2x2 update, chosen on the host from the matrix's exact values.
+// complex128 is bound by the FP64 pipe (two lanes per SM and clock), not by
+// memory: 16 operations per pair for a general matrix, so the named gates use
+// the fewest their structure allows (each form is one or two roundings per
+// result, as the general one has three):
+//   G_REAL    real entries                                   8 per pair
+//   G_HAD     c [[1, 1], [1, -1]]: c a shared by both rows   6
+//   G_SX(D)   (1 +- i)/2 [[1, -+i], [-+i, 1]]               10
+//   G_SY(D)   (1 + i)/2 [[1, -1], [1, 1]] and its adjoint   10
+//   G_SWAP    [[0, 1], [1, 0]]                               0
+// 26 qubits: H 391 us, SX / SY 645, general 1028 (all three took 1027 before);
+// 20 qubits, 590 gates of the random family: 7.43 ms before, 4.00 ms now.
+enum GateForm { G_GENERAL = 0, G_REAL, G_HAD, G_SX, G_SXD, G_SY, G_SYD, G_SWAP };
+
+template <int F, typename R>
 __device__ __forceinline__ void apply2(const R *u, R &ar, R &ai, R &br, R &bi) {
-    const R nar = u[0] * ar - u[1] * ai + u[2] * br - u[3] * bi;
-    const R nai = u[0] * ai + u[1] * ar + u[2] * bi + u[3] * br;
-    const R nbr = u[4] * ar - u[5] * ai + u[6] * br - u[7] * bi;
-    const R nbi = u[4] * ai + u[5] * ar + u[6] * bi + u[7] * br;
-    ar = nar;
-    ai = nai;
-    br = nbr;
-    bi = nbi;
+    const R h = R(0.5);
+    if constexpr (F == G_REAL) {
+        const R nar = u[0] * ar + u[2] * br, nai = u[0] * ai + u[2] * bi;
+        br = u[4] * ar + u[6] * br;
+        bi = u[4] * ai + u[6] * bi;
+        ar = nar;
+        ai = nai;
+    } else if constexpr (F == G_HAD) {
+        const R c = u[0], p = c * ar, q = c * ai, x = br, y = bi;
+        ar = fma(c, x, p);
+        br = fma(-c, x, p);
+        ai = fma(c, y, q);
+        bi = fma(-c, y, q);
+    } else if constexpr (F == G_SX || F == G_SXD) {
+        // e = (a -+ i b) / 2, f = (b -+ i a) / 2; a' = (1 +- i) e, b' = (1 +- i) f
+        const R p = h * ar, q = h * ai;
+        if constexpr (F == G_SX) {
+            const R er = fma(h, bi, p), ei = fma(-h, br, q), fr = fma(h, br, q), fi = fma(h, bi, -p);
+            ar = er - ei;
+            ai = er + ei;
+            br = fr - fi;
+            bi = fr + fi;
+        } else {
+            const R er = fma(-h, bi, p), ei = fma(h, br, q), fr = fma(h, br, -q), fi = fma(h, bi, p);
+            ar = er + ei;
+            ai = ei - er;
+            br = fr + fi;
+            bi = fi - fr;
+        }
+    } else if constexpr (F == G_SY || F == G_SYD) {
+        const R p = h * ar, q = h * ai;
+        const R sr = fma(h, br, p), si = fma(h, bi, q);
+        if constexpr (F == G_SY) {  // a' = (1 + i) (a - b) / 2, b' = (1 + i) (a + b) / 2
+            const R dr = fma(-h, br, p), di = fma(-h, bi, q);
+            ar = dr - di;
+            ai = dr + di;
+            br = sr - si;
+            bi = sr + si;
+        } else {  // a' = (1 - i) (a + b) / 2, b' = (1 - i) (b - a) / 2
+            const R dr = fma(h, br, -p), di = fma(h, bi, -q);
+            ar = sr + si;
+            ai = si - sr;
+            br = dr + di;
+            bi = di - dr;
+        }
+    } else if constexpr (F == G_SWAP) {
+        const R x = ar, y = ai;
+        ar = br;
+        ai = bi;
+        br = x;
+        bi = y;
+    } else {
+        const R nar = u[0] * ar - u[1] * ai + u[2] * br - u[3] * bi;
+        const R nai = u[0] * ai + u[1] * ar + u[2] * bi + u[3] * br;
+        const R nbr = u[4] * ar - u[5] * ai + u[6] * br - u[7] * bi;
+        const R nbi = u[4] * ai + u[5] * ar + u[6] * bi + u[7] * br;
+        ar = nar;
+        ai = nai;
+        br = nbr;
+        bi = nbi;
+    }
 }
 
-constexpr int kUnr = 4;
-constexpr int kThreads = 256;
+// Vector pairs in flight per thread and threads per CTA.  complex64 is bound
+// by memory and wants bytes in flight; complex128 is bound by the FP64 pipe
+// (0.52 T operations/s measured), where the work has to spread evenly over the
+// SMs at every size: small CTAs (20 qubits, 590 gates: 4.74 ms with 4 x 256,
+// 4.15 with 2 x 128, 4.00 with 1 x 128; 26 qubits: the same within 1%).
+template <typename R>
+struct Shape1 {
+    static constexpr int unr = 4, threads = 256;
+};
+template <>
+struct Shape1<double> {
+    static constexpr int unr = 1, threads = 128;
+};
 
 // Pair across two vectors (target >= W).
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_gate_across(typename VecT<R>::T *__restrict__ v, GateArgs<R> a) {
+template <typename R, int F>
+__global__ void __launch_bounds__(Shape1<R>::threads) k_gate_across(typename VecT<R>::T *__restrict__ v, GateArgs<R> a) {
+    constexpr int kUnr = Shape1<R>::unr;
     using V = typename VecT<R>::T;
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t base = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; base < a.nwork; base += stride * kUnr) {
@@ -96,10 +175,10 @@ __global__ void __launch_bounds__(kThreads) k_gate_across(typename VecT<R>::T *_
             const uint64_t w = base + k * stride;
             if (w < a.nwork) {
                 if constexpr (VecT<R>::W == 1) {
-                    if (!(a.lane_mask & 1)) apply2(a.u, x[k].x, x[k].y, y[k].x, y[k].y);
-                    apply2(a.u, x[k].z, x[k].w, y[k].z, y[k].w);
+                    if (!(a.lane_mask & 1)) apply2<F>(a.u, x[k].x, x[k].y, y[k].x, y[k].y);
+                    apply2<F>(a.u, x[k].z, x[k].w, y[k].z, y[k].w);
                 } else {
-                    apply2(a.u, x[k].x, x[k].y, y[k].x, y[k].y);
+                    apply2<F>(a.u, x[k].x, x[k].y, y[k].x, y[k].y);
                 }
                 v[i0[k]] = x[k];
                 v[i0[k] | a.tbit] = y[k];
@@ -109,7 +188,8 @@ __global__ void __launch_bounds__(kThreads) k_gate_across(typename VecT<R>::T *_
 }
 
 // complex64 target qubit 0: the pair is the two halves of one float4.
-__global__ void __launch_bounds__(kThreads) k_gate_inner(float4 *__restrict__ v, GateArgs<float> a) {
+__global__ void __launch_bounds__(Shape1<float>::threads) k_gate_inner(float4 *__restrict__ v, GateArgs<float> a) {
+    constexpr int kUnr = Shape1<float>::unr;
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t base = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; base < a.nwork; base += stride * kUnr) {
         float4 x[kUnr];
@@ -126,18 +206,40 @@ __global__ void __launch_bounds__(kThreads) k_gate_inner(float4 *__restrict__ v,
         for (int k = 0; k < kUnr; ++k) {
             const uint64_t w = base + k * stride;
             if (w < a.nwork) {
-                apply2(a.u, x[k].x, x[k].y, x[k].z, x[k].w);
+                apply2<G_GENERAL>(a.u, x[k].x, x[k].y, x[k].z, x[k].w);
                 v[i0[k]] = x[k];
             }
         }
     }
 }
 
+// u11 of a diagonal gate with u00 = 1 on one amplitude.  Sign flips and
+// quarter turns (CZ, Z, S) are exact moves: no FP64 operations, and 4 for
+// another phase.
+enum PhaseForm { P_GENERAL = 0, P_NEG, P_I, P_MI };
+
+template <int F, typename R>
+__device__ __forceinline__ void phase1(R pr, R pi, R &x, R &y) {
+    if constexpr (F == P_NEG) {
+        x = -x;
+        y = -y;
+    } else if constexpr (F == P_I || F == P_MI) {
+        const R t = F == P_I ? x : -x;
+        x = F == P_I ? -y : y;
+        y = t;
+    } else {
+        const R r = x * pr - y * pi, i = x * pi + y * pr;
+        x = r;
+        y = i;
+    }
+}
+
 // Diagonal gate with u00 = 1: multiply the amplitudes whose masked bits are
 // all set by u11.  Vectors are enumerated with the vector-level mask bits
 // forced to 1; lane_mask selects amplitudes inside a float4.
-template <typename R>
-__global__ void __launch_bounds__(kThreads) k_phase(typename VecT<R>::T *__restrict__ v, GateArgs<R> a) {
+template <typename R, int F>
+__global__ void __launch_bounds__(Shape1<R>::threads) k_phase(typename VecT<R>::T *__restrict__ v, GateArgs<R> a) {
+    constexpr int kUnr = Shape1<R>::unr;
     using V = typename VecT<R>::T;
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     const R pr = a.u[6], pi = a.u[7];
@@ -157,18 +259,10 @@ __global__ void __launch_bounds__(kThreads) k_phase(typename VecT<R>::T *__restr
             const uint64_t w = base + k * stride;
             if (w < a.nwork) {
                 if constexpr (VecT<R>::W == 1) {
-                    if (!(a.lane_mask & 1)) {
-                        const R r = x[k].x * pr - x[k].y * pi, i = x[k].x * pi + x[k].y * pr;
-                        x[k].x = r;
-                        x[k].y = i;
-                    }
-                    const R r = x[k].z * pr - x[k].w * pi, i = x[k].z * pi + x[k].w * pr;
-                    x[k].z = r;
-                    x[k].w = i;
+                    if (!(a.lane_mask & 1)) phase1<F>(pr, pi, x[k].x, x[k].y);
+                    phase1<F>(pr, pi, x[k].z, x[k].w);
                 } else {
-                    const R r = x[k].x * pr - x[k].y * pi, i = x[k].x * pi + x[k].y * pr;
-                    x[k].x = r;
-                    x[k].y = i;
+                    phase1<F>(pr, pi, x[k].x, x[k].y);
                 }
                 v[i0[k]] = x[k];
             }
@@ -176,10 +270,12 @@ __global__ void __launch_bounds__(kThreads) k_phase(typename VecT<R>::T *__restr
     }
 }
 
+template <typename R>
 int grid_for(uint64_t nwork) {
-    uint64_t b = (nwork + uint64_t(kThreads) * kUnr - 1) / (uint64_t(kThreads) * kUnr);
+    constexpr uint64_t per = uint64_t(Shape1<R>::threads) * Shape1<R>::unr;
+    uint64_t b = (nwork + per - 1) / per;
     if (b < 1) b = 1;
-    const uint64_t cap = 152ull * 32;
+    const uint64_t cap = 152ull * 32 * (256 / Shape1<R>::threads);
     return int(b < cap ? b : cap);
 }
 
@@ -190,6 +286,33 @@ void sort_small(int *p, int n) {
             p[j] = p[j - 1];
             p[j - 1] = t;
         }
+}
+
+template <typename R>
+int gate_form(const R *u) {
+    auto is = [&](R a, R b, R c, R d, R e, R f, R g, R h) {
+        const R w[8] = {a, b, c, d, e, f, g, h};
+        for (int k = 0; k < 8; ++k)
+            if (u[k] != w[k]) return false;
+        return true;
+    };
+    const R h = R(0.5);
+    if (is(0, 0, 1, 0, 1, 0, 0, 0)) return G_SWAP;
+    if (is(h, h, h, -h, h, -h, h, h)) return G_SX;
+    if (is(h, -h, h, h, h, h, h, -h)) return G_SXD;
+    if (is(h, h, -h, -h, h, h, h, h)) return G_SY;
+    if (is(h, -h, h, -h, -h, h, h, -h)) return G_SYD;
+    if (u[1] == 0 && u[3] == 0 && u[5] == 0 && u[7] == 0)
+        return u[0] == u[2] && u[0] == u[4] && u[0] == -u[6] ? G_HAD : G_REAL;
+    return G_GENERAL;
+}
+
+template <typename R>
+int phase_form(const R *u) {
+    if (u[6] == -1 && u[7] == 0) return P_NEG;
+    if (u[6] == 0 && u[7] == 1) return P_I;
+    if (u[6] == 0 && u[7] == -1) return P_MI;
+    return P_GENERAL;
 }
 
 template <typename R>
@@ -227,7 +350,17 @@ cudaError_t gate1_impl(sv_state *h, const Gate1 &g) {
         a.set_mask = setm;
         a.lane_mask = lane;
         a.nwork = uint64_t(1) << (nv_log - ni);
-        k_phase<R><<<grid_for(a.nwork), kThreads, 0, h->stream>>>(v, a);
+        const int grid = grid_for<R>(a.nwork);
+        if constexpr (W == 0) {  // FP64: the forms; complex64 is bound by memory
+            switch (phase_form(a.u)) {
+                case P_NEG: k_phase<R, P_NEG><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                case P_I: k_phase<R, P_I><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                case P_MI: k_phase<R, P_MI><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                default: k_phase<R, P_GENERAL><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+            }
+        } else {
+            k_phase<R, P_GENERAL><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a);
+        }
         return cudaGetLastError();
     }
     int ins[2], ni = 0;
@@ -252,10 +385,24 @@ cudaError_t gate1_impl(sv_state *h, const Gate1 &g) {
     a.lane_mask = lane;
     a.nwork = uint64_t(1) << (nv_log - ni);
     if (t >= W) {
-        k_gate_across<R><<<grid_for(a.nwork), kThreads, 0, h->stream>>>(v, a);
+        const int grid = grid_for<R>(a.nwork);
+        if constexpr (W == 0) {
+            switch (gate_form(a.u)) {
+                case G_REAL: k_gate_across<R, G_REAL><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                case G_HAD: k_gate_across<R, G_HAD><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                case G_SX: k_gate_across<R, G_SX><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                case G_SXD: k_gate_across<R, G_SXD><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                case G_SY: k_gate_across<R, G_SY><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                case G_SYD: k_gate_across<R, G_SYD><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                case G_SWAP: k_gate_across<R, G_SWAP><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+                default: k_gate_across<R, G_GENERAL><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a); break;
+            }
+        } else {
+            k_gate_across<R, G_GENERAL><<<grid, Shape1<R>::threads, 0, h->stream>>>(v, a);
+        }
     } else {
         if constexpr (W == 1) {
-            k_gate_inner<<<grid_for(a.nwork), kThreads, 0, h->stream>>>(reinterpret_cast<float4 *>(v), a);
+            k_gate_inner<<<grid_for<float>(a.nwork), Shape1<float>::threads, 0, h->stream>>>(reinterpret_cast<float4 *>(v), a);
         }
     }
     return cudaGetLastError();

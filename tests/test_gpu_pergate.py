@@ -75,6 +75,34 @@ def test_every_target_and_control(S, orc, dtype, n):
 
 
 @pytest.mark.parametrize("dtype", ["c64", "c128"])
+@pytest.mark.parametrize("n", [1, 2, 5, 11])
+def test_matrix_forms(S, orc, dtype, n):
+    """Every form the per-gate kernels pick from a matrix's exact entries (real,
+    Hadamard, the square roots of X and Y and their adjoints, X, sign flip,
+    quarter turns, scaled and signed neighbours of them that must not be taken
+    for one), with and without a control, against the oracle's Eq. 1 loops."""
+    psi0 = C.random_state(n, 40 + n)
+    mats = [orc.gate_matrix(k) for k in ("H", "SX", "SXDG", "SY", "SYDG", "X", "Y", "Z", "S", "SDG", "T")]
+    th = 0.4
+    mats += [np.array([[np.cos(th), -np.sin(th)], [np.sin(th), np.cos(th)]]), -orc.gate_matrix("H"),
+             1j * orc.gate_matrix("SX"), orc.gate_matrix("SY").T, np.diag([1, 1]), np.diag([1j, 1j])]
+    sv_ = S.StateVector(n, dtype)
+    for u in mats:
+        for t, c in {(0, -1), (n - 1, -1), (n // 2, -1), (0, n - 1), (n - 1, 0), (n // 2, 0)}:
+            if c == t:
+                continue
+            sv_.from_numpy(psi0)
+            sv_.apply_gate(t, u, control=c)
+            if c < 0:
+                ref = orc.apply_1q(psi0, t, u)
+            else:
+                cu = np.eye(4, dtype=complex)
+                cu[np.ix_([1, 3], [1, 3])] = u
+                ref = orc.apply_kq(psi0, [c, t], cu)
+            check(dtype, sv_.to_numpy(), ref)
+
+
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
 @pytest.mark.parametrize("seed", [1, 2, 3])
 def test_random_circuit_20q(S, orc, dtype, seed):
     """20 qubits, depth 20 random circuit, full 16 MB vector against the oracle."""
