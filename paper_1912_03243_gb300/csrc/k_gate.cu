@@ -315,6 +315,12 @@ int phase_form(const R *u) {
     return P_GENERAL;
 }
 
+// Diagonal with u00 = 1: only the amplitudes with the target (and control)
+// bits set change.
+bool is_phase(const Gate1 &g) {
+    return g.u[1].re == 0 && g.u[1].im == 0 && g.u[2].re == 0 && g.u[2].im == 0 && g.u[0].re == 1 && g.u[0].im == 0;
+}
+
 template <typename R>
 cudaError_t gate1_impl(sv_state *h, const Gate1 &g) {
     using V = typename VecT<R>::T;
@@ -327,10 +333,8 @@ cudaError_t gate1_impl(sv_state *h, const Gate1 &g) {
     const int n = h->n;
     const int nv_log = n - W;  // log2 number of vectors
     V *v = static_cast<V *>(h->data);
-    const bool diag = g.u[1].re == 0 && g.u[1].im == 0 && g.u[2].re == 0 && g.u[2].im == 0;
-    const bool unit00 = g.u[0].re == 1 && g.u[0].im == 0;
     const int t = g.target, c = g.control;
-    if (diag && unit00) {
+    if (is_phase(g)) {
         // phase on amplitudes with bit t (and bit c) set
         int ins[2], ni = 0;
         uint64_t setm = 0;
@@ -406,6 +410,199 @@ cudaError_t gate1_impl(sv_state *h, const Gate1 &g) {
         }
     }
     return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------- small states
+// A run of per-gate updates on a state that fits one CTA's shared memory, in
+// one launch: the state is loaded once, the gates are applied in circuit
+// order, and it is stored once.  One launch per gate of such a state is all
+// launch latency (10 qubits, 145 gates, graph replay: 1.2 us per gate).  The
+// gates are taken in stages of consecutive gates with at most S distinct
+// targets (diagonal gates have none): each thread gathers the 2^S amplitudes
+// of those qubits into registers, applies the stage's gates and scatters them
+// back, so a stage costs one shared-memory round trip and one barrier.  The
+// gates come as a
+// kernel parameter, so a launch needs no device memory of its own.
+template <typename R>
+struct SmallOp {
+    uint8_t code;    // pair updates: GateForm * 3 + slot; 24 + PhaseForm; a stage header: number of its gates
+    uint8_t rmask;   // register-index bits that must be 1
+    uint8_t s[2];    // stage header: its first two qubits (the third in imask)
+    uint32_t imask;  // other amplitude-index bits that must be 1
+    R u[8];
+};
+template <typename R>
+struct SmallRun {
+    static constexpr int kMaxOps = sizeof(R) == 4 ? 200 : 112;  // 8 KB of parameters
+    int n, nops;
+    SmallOp<R> op[kMaxOps];
+};
+
+// Swizzled position of amplitude i: rows of 128 bytes, the column permuted by
+// the row number (linear over XOR), so that gathers of low qubits spread over
+// the banks.
+template <typename R>
+__device__ __forceinline__ uint32_t small_pos(uint32_t i) {
+    return sizeof(R) == 4 ? i ^ ((i >> 4) & 15u) : i ^ ((i >> 3) & 7u);
+}
+
+template <int F, int SLOT, int S, typename R>
+__device__ __forceinline__ void small_pairs(C2<R> (&x)[1 << S], const SmallOp<R> &op) {
+    if constexpr (SLOT < S) {
+#pragma unroll
+        for (int v = 0; v < (1 << S); ++v) {
+            if (v >> SLOT & 1) continue;
+            const int w = v | 1 << SLOT;
+            if ((v & op.rmask) == op.rmask) apply2<F>(op.u, x[v].re, x[v].im, x[w].re, x[w].im);
+        }
+    }
+}
+template <int F, int S, typename R>
+__device__ __forceinline__ void small_phase(C2<R> (&x)[1 << S], const SmallOp<R> &op) {
+#pragma unroll
+    for (int v = 0; v < (1 << S); ++v)
+        if ((v & op.rmask) == op.rmask) phase1<F>(op.u[6], op.u[7], x[v].re, x[v].im);
+}
+
+template <int S, typename R>
+__device__ __forceinline__ void small_gate(C2<R> (&x)[1 << S], const SmallOp<R> &op) {
+#define SV_SMALL_FORM(F)                                        \
+    case 3 * F: small_pairs<F, 0, S>(x, op); break;             \
+    case 3 * F + 1: small_pairs<F, 1, S>(x, op); break;         \
+    case 3 * F + 2: small_pairs<F, 2, S>(x, op); break;
+    switch (op.code) {
+        SV_SMALL_FORM(G_GENERAL)
+        SV_SMALL_FORM(G_REAL)
+        SV_SMALL_FORM(G_HAD)
+        SV_SMALL_FORM(G_SX)
+        SV_SMALL_FORM(G_SXD)
+        SV_SMALL_FORM(G_SY)
+        SV_SMALL_FORM(G_SYD)
+        SV_SMALL_FORM(G_SWAP)
+        case 24 + P_NEG: small_phase<P_NEG, S>(x, op); break;
+        case 24 + P_I: small_phase<P_I, S>(x, op); break;
+        case 24 + P_MI: small_phase<P_MI, S>(x, op); break;
+        default: small_phase<P_GENERAL, S>(x, op); break;
+    }
+#undef SV_SMALL_FORM
+}
+
+template <typename R>
+constexpr int kSmallThreads = sizeof(R) == 4 ? 1024 : 512;
+
+template <typename R, int S>
+__global__ void __launch_bounds__(kSmallThreads<R>) k_small_run(C2<R> *__restrict__ psi, const __grid_constant__ SmallRun<R> a) {
+    extern __shared__ __align__(16) unsigned char small_smem[];
+    C2<R> *sm = reinterpret_cast<C2<R> *>(small_smem);
+    __shared__ __align__(16) SmallOp<R> ops[SmallRun<R>::kMaxOps];
+    const uint32_t namps = 1u << a.n;
+    for (uint32_t i = threadIdx.x; i < a.nops * uint32_t(sizeof(SmallOp<R>) / 8); i += blockDim.x)
+        reinterpret_cast<uint2 *>(ops)[i] = reinterpret_cast<const uint2 *>(a.op)[i];
+    for (uint32_t i = threadIdx.x; i < namps; i += blockDim.x) sm[small_pos<R>(i)] = psi[i];
+    __syncthreads();
+    for (int k = 0; k < a.nops;) {
+        const int cnt = ops[k].code;
+        const int s0 = ops[k].s[0], s1 = ops[k].s[1], s2 = int(ops[k].imask);
+        const uint32_t d0 = small_pos<R>(1u << s0), d1 = small_pos<R>(1u << s1), d2 = small_pos<R>(1u << s2);
+        for (uint32_t w = threadIdx.x; w < namps >> S; w += blockDim.x) {
+            uint32_t i = w + (w & ~((1u << s0) - 1));  // a zero bit inserted at s0
+            if (S > 1) i += i & ~((1u << s1) - 1);
+            if (S > 2) i += i & ~((1u << s2) - 1);
+            const uint32_t p = small_pos<R>(i);
+            C2<R> x[1 << S];
+#pragma unroll
+            for (int v = 0; v < (1 << S); ++v)
+                x[v] = sm[p ^ (v & 1 ? d0 : 0u) ^ (v & 2 ? d1 : 0u) ^ (v & 4 ? d2 : 0u)];
+            for (int j = k + 1; j <= k + cnt; ++j) {
+                const SmallOp<R> &op = ops[j];
+                if ((i & op.imask) == op.imask) small_gate<S>(x, op);
+            }
+#pragma unroll
+            for (int v = 0; v < (1 << S); ++v)
+                sm[p ^ (v & 1 ? d0 : 0u) ^ (v & 2 ? d1 : 0u) ^ (v & 4 ? d2 : 0u)] = x[v];
+        }
+        __syncthreads();
+        k += cnt + 1;
+    }
+    for (uint32_t i = threadIdx.x; i < namps; i += blockDim.x) psi[i] = sm[small_pos<R>(i)];
+}
+
+// Fill a with a stage (or the part of it that fits) starting at gate i;
+// returns the next gate.
+template <typename R, int S>
+size_t small_stage(int n, const Gate1 *g, size_t i, size_t count, SmallRun<R> *a) {
+    constexpr int kMax = SmallRun<R>::kMaxOps;
+    uint32_t qs = 0;  // the stage's qubits
+    size_t e = i;
+    for (; e < count && int(e - i) + 1 < kMax - a->nops && e - i < 255; ++e) {
+        if (is_phase(g[e])) continue;
+        const uint32_t b = 1u << g[e].target;
+        if (!(qs & b) && __builtin_popcount(qs) == S) break;
+        qs |= b;
+    }
+    for (int q = n - 1; q >= 0 && __builtin_popcount(qs) < S; --q) qs |= 1u << q;  // high ones: no bank conflicts
+    int slot[32], s[3] = {0, 0, 0}, ns = 0;
+    for (int q = 0; q < n; ++q) {
+        slot[q] = -1;
+        if (qs >> q & 1u) {
+            s[ns] = q;
+            slot[q] = ns++;
+        }
+    }
+    SmallOp<R> &hd = a->op[a->nops++];
+    hd = SmallOp<R>{};
+    hd.code = uint8_t(e - i);
+    hd.s[0] = uint8_t(s[0]);
+    hd.s[1] = uint8_t(s[1]);
+    hd.imask = uint32_t(s[2]);
+    for (; i < e; ++i) {
+        SmallOp<R> &op = a->op[a->nops++];
+        op = SmallOp<R>{};
+        for (int k = 0; k < 4; ++k) {
+            op.u[2 * k] = R(g[i].u[k].re);
+            op.u[2 * k + 1] = R(g[i].u[k].im);
+        }
+        uint32_t cond = g[i].control < 0 ? 0u : 1u << g[i].control;
+        if (is_phase(g[i])) {
+            cond |= 1u << g[i].target;
+            op.code = uint8_t(24 + phase_form(op.u));
+        } else {
+            op.code = uint8_t(3 * gate_form(op.u) + slot[g[i].target]);
+        }
+        for (int q = 0; q < n; ++q)
+            if (cond >> q & 1u) {
+                if (slot[q] >= 0) op.rmask |= uint8_t(1u << slot[q]);
+                else op.imask |= 1u << q;
+            }
+    }
+    return e;
+}
+
+template <typename R, int S>
+cudaError_t small_run(sv_state *h, const Gate1 *g, size_t count) {
+    const int n = h->n;
+    const int tlog = n - S;
+    const int threads = tlog < 5 ? 32 : (1 << tlog) > kSmallThreads<R> ? kSmallThreads<R> : 1 << tlog;
+    const int smem = int(sizeof(C2<R>)) << n;
+    if (smem > 32 * 1024) {
+        static std::atomic<uint64_t> configured{0};
+        if (attrs_needed(configured, h->device)) {
+            const cudaError_t e = cudaFuncSetAttribute(k_small_run<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       int(sizeof(C2<R>)) << small_run_max_n(h->dt));
+            if (e != cudaSuccess) return e;
+            attrs_set(configured, h->device);
+        }
+    }
+    for (size_t i = 0; i < count;) {
+        SmallRun<R> a;
+        a.n = n;
+        a.nops = 0;
+        while (i < count && a.nops + 2 <= SmallRun<R>::kMaxOps) i = small_stage<R, S>(n, g, i, count, &a);
+        k_small_run<R, S><<<1, threads, smem, h->stream>>>(static_cast<C2<R> *>(h->data), a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // ---------------------------------------------------------------- set basis
@@ -520,10 +717,8 @@ const char *gate1_kernel_name(const sv_state *h, const Gate1 &g) {
             return "k_enc_gate_across<diag1>";
         return "k_enc_gate_across";
     }
-    const bool diag = g.u[1].re == 0 && g.u[1].im == 0 && g.u[2].re == 0 && g.u[2].im == 0;
-    const bool unit00 = g.u[0].re == 1 && g.u[0].im == 0;
     const bool c64 = h->dt == SV_C64;
-    if (diag && unit00) return c64 ? "k_phase<f32>" : "k_phase<f64>";
+    if (is_phase(g)) return c64 ? "k_phase<f32>" : "k_phase<f64>";
     if (c64 && g.target == 0) return "k_gate_inner<f32>";
     return c64 ? "k_gate_across<f32>" : "k_gate_across<f64>";
 }
@@ -532,6 +727,21 @@ cudaError_t launch_gate1(sv_state *h, const Gate1 &g) {
     if (h->dt == SV_C64) return gate1_impl<float>(h, g);
     if (h->dt == SV_C128) return gate1_impl<double>(h, g);
     return launch_enc_gate1(h, g);
+}
+
+// Largest small state: complex64 up to 128 KB of shared memory (14 qubits, 205
+// gates: 174 us against 370 with one launch per gate); complex128 while one
+// SM's FP64 pipe beats a launch on all of them (10 qubits, 145 gates: 166
+// against 195 us; 11 qubits, 160 gates: 336 against 215).
+int small_run_max_n(sv_dtype dt) { return dt == SV_C64 ? 14 : dt == SV_C128 ? 10 : 0; }
+
+cudaError_t launch_small_run(sv_state *h, const Gate1 *g, size_t count) {
+    // amplitudes per thread: two target bits up to 11 qubits, where threads are
+    // few (10 qubits, 145 gates: 35 us; 41 with one bit, 39 with three), three
+    // from 12 on (13 qubits, 190 gates: 93 us against 121); one for complex128,
+    // whose FP64 chains want many warps (8 qubits, 115 gates: 60 us against 86)
+    if (h->dt == SV_C128) return small_run<double, 1>(h, g, count);
+    return h->n < 12 ? small_run<float, 2>(h, g, count) : small_run<float, 3>(h, g, count);
 }
 
 cudaError_t launch_set_basis(sv_state *h, uint64_t idx) {

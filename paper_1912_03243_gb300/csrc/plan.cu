@@ -41,8 +41,6 @@ namespace {
 
 void destroy_plan(sv_plan_s *p) {
     if (p->gexec) cudaGraphExecDestroy(p->gexec);
-    for (cudaEvent_t e : p->gev)
-        if (e) cudaEventDestroy(e);
     if (p->gstream) cudaStreamDestroy(p->gstream);
     if (p->d_tcA) cudaFree(p->d_tcA);
     if (p->d_encops) cudaFree(p->d_encops);
@@ -647,7 +645,16 @@ sv_status sv_plan_create(sv_handle h, const char *text, int mode, sv_plan *out) 
 namespace sv {
 namespace {
 
+// A plan of two or more per-gate updates of a state of 2 to
+// small_run_max_n qubits runs in few launches (k_small_run); its launch list keeps one entry per gate, which is
+// what sv_plan_execute_timed and the statistics show.
+bool small_plan(const sv_plan_s *p) {
+    return p->h->n >= 2 && p->h->n <= small_run_max_n(p->h->dt) && p->launches.size() >= 2 &&
+           p->launches.size() == p->pergate.size();
+}
+
 sv_status execute_direct(sv_plan_s *p) {
+    if (small_plan(p)) return check_launch(launch_small_run(p->h, p->pergate.data(), p->pergate.size()), "sv_plan_execute");
     for (const PlanLaunch &l : p->launches) {
         sv_status s = check_launch(launch_one(p, l), "sv_plan_execute");
         if (s) return s;
@@ -659,6 +666,7 @@ sv_status execute_direct(sv_plan_s *p) {
 
 extern "C++" {
 cudaError_t plan_launch_all(sv_plan_s *p) {
+    if (small_plan(p)) return launch_small_run(p->h, p->pergate.data(), p->pergate.size());
     for (const PlanLaunch &l : p->launches) {
         const cudaError_t e = launch_one(p, l);
         if (e != cudaSuccess) return e;
@@ -695,18 +703,12 @@ cudaError_t capture_graph(sv_plan_s *p) {
     sv_state *h = p->h;
     cudaError_t e = cudaSuccess;
     if (!p->gstream) e = cudaStreamCreateWithFlags(&p->gstream, cudaStreamNonBlocking);
-    for (int i = 0; i < 2 && e == cudaSuccess; ++i)
-        if (!p->gev[i]) e = cudaEventCreateWithFlags(&p->gev[i], cudaEventDisableTiming);
     if (e != cudaSuccess) return e;
     const cudaStream_t user = h->stream;
     h->stream = p->gstream;  // the launch functions launch on the handle's stream
     e = cudaStreamBeginCapture(p->gstream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t le = cudaSuccess;
-        for (const PlanLaunch &l : p->launches) {
-            le = launch_one(p, l);
-            if (le != cudaSuccess) break;
-        }
+        const cudaError_t le = plan_launch_all(p);
         cudaGraph_t g = nullptr;
         const cudaError_t ee = cudaStreamEndCapture(p->gstream, &g);
         e = le != cudaSuccess ? le : ee;
@@ -721,13 +723,11 @@ cudaError_t capture_graph(sv_plan_s *p) {
     return e;
 }
 
+// A graph may be launched into any stream, the legacy default stream
+// included (only capture needs a stream of its own), so the replay needs no
+// events between streams.
 sv_status execute_graph(sv_plan_s *p) {
-    sv_state *h = p->h;
-    SV_CUDA_TRY(cudaEventRecord(p->gev[0], h->stream));
-    SV_CUDA_TRY(cudaStreamWaitEvent(p->gstream, p->gev[0], 0));
-    SV_CUDA_TRY(cudaGraphLaunch(p->gexec, p->gstream));
-    SV_CUDA_TRY(cudaEventRecord(p->gev[1], p->gstream));
-    SV_CUDA_TRY(cudaStreamWaitEvent(h->stream, p->gev[1], 0));
+    SV_CUDA_TRY(cudaGraphLaunch(p->gexec, p->h->stream));
     return SV_OK;
 }
 

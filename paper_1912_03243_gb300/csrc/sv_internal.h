@@ -114,6 +114,10 @@ namespace sv {
 // ---------------------------------------------------------------- kernels
 // All launchers enqueue on `st` and return the launch error (if any).
 cudaError_t launch_gate1(sv_state *h, const Gate1 &g);
+// Gates in order on a state of at most small_run_max_n(dt) qubits (0: none):
+// one launch per about a hundred gates, the state in one CTA's shared memory.
+int small_run_max_n(sv_dtype dt);
+cudaError_t launch_small_run(sv_state *h, const Gate1 *g, size_t count);
 cudaError_t launch_set_basis(sv_state *h, uint64_t idx);
 cudaError_t launch_norm(sv_state *h, double *d_out);  // d_out: device double
 cudaError_t launch_gather(sv_state *h, const uint64_t *d_idx, size_t m, double *d_out);

@@ -102,6 +102,37 @@ def test_matrix_forms(S, orc, dtype, n):
             check(dtype, sv_.to_numpy(), ref)
 
 
+@pytest.mark.parametrize("dtype,n", [(d, n) for d, top in (("c64", 15), ("c128", 11)) for n in (1, 2, 3, 5, 8, 10, 11, 12, 14, 15)
+                                     if n <= top])
+def test_small_states_run(S, orc, dtype, n):
+    """Plans of small states run many gates per launch (stages of gates on one to
+    three target qubits, several launches for long circuits): mixed circuits,
+    a QFT, and a run of diagonal gates alone, direct and as a graph replay,
+    against the oracle; one launch per gate (sv_plan_execute_timed) agrees."""
+    import torch
+
+    diag = C.Circuit(n)
+    for q in range(n):
+        diag.add("T", q)
+        diag.add("CZ" if q else "S", *((q, q - 1) if q else (q,)))
+    for c in (C.random_unitary_gates(n, 450 if n >= 5 else 60, n), C.random_circuit(n, 12, 3), C.qft_circuit(n, 1), diag):
+        psi0 = C.random_state(n, 70 + n)
+        ref = orc.run(c, psi=psi0)
+        s = S.StateVector(n, dtype)
+        p = s.plan(c, "pergate")
+        for _ in range(3):  # direct, capture, replay
+            s.from_numpy(psi0)
+            p.execute()
+            check(dtype, s.to_numpy(), ref)
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(p.passes + 1)]
+        for e in ev:
+            e.record(s.stream)
+        s.from_numpy(psi0)
+        p.execute_timed(ev)
+        check(dtype, s.to_numpy(), ref)
+        p.free()
+
+
 @pytest.mark.parametrize("dtype", ["c64", "c128"])
 @pytest.mark.parametrize("seed", [1, 2, 3])
 def test_random_circuit_20q(S, orc, dtype, seed):
