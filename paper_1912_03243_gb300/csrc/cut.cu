@@ -20,13 +20,32 @@
 // and D_s are phases selected by (bit, s_k)).  Branch bits only ever appear
 // in diagonal gates, so the tile planner keeps them outside the tiles (a
 // constant per CTA) and every pass runs over all branches of a half in one
-// launch.  The initial vector has amplitude 1 at index s << n_p for every s
-// (or, with branch-prefix sharing, the branches are forked from branch 0 at
-// their first operator, see run_half).
+// launch.
+//
+// Stages (branch-prefix sharing).  The gates before a branch bit's first
+// operator are the same for both its values, so a stage of gates runs on the
+// branches that are live, and the vector forks to the next branch bits
+// between stages: the first pass of a stage reads the previous stage's smaller
+// vector once per new branch and writes its own, so a fork costs no copy, and
+// a stage of nothing but branch operators joins the next stage's first pass
+// (prepend_diagonals: the same factors in the same order).  The last stage
+// runs in chunks of its top branch bits on one buffer (kChunkQubits), only the
+// amplitudes that the bit strings name are kept of each chunk, and its last
+// pass runs on the tiles that hold one: the 48-qubit grid of 256 branches
+// needs 4.3 GB instead of 64 GB, whose cudaFree alone took 24 ms.
 //
 // Sum (GPU): one warp per output bit string (its partition indices gathered
 // from the string's bits by the first P lanes), lanes over s, products of the
 // P partitions' amplitudes and the sum in FP64, times the weight.
+//
+// 48-qubit grid (2 x 24 qubits, 256 branches, 1024 strings): 161 ms with a copy
+// and a pass for every branch bit and both halves' vectors whole, 72 ms with
+// stages, chunks and wanted tiles, 64 ms with zero tiles written without
+// computing (now: bound by the last stage's three passes over 2 x 2^32
+// amplitudes, HBM and FP32 alike).  (Levels by light cone, each gate on as few branches as its operators
+// allow, would take 27 ms, but reorder gates and so round differently.)
+#include <algorithm>
+#include <cmath>
 #include <complex>
 #include <cstdlib>
 #include <mutex>
@@ -62,7 +81,31 @@ struct CutSumArgs {
     int nlocal[kMaxParts], nbits[kMaxParts];
     uint8_t cutbit[kMaxParts][kMaxCutBits];      // partition bit j <- batched branch bit cutbit[p][j]
     uint8_t qubit[kMaxParts][kMaxPartQubits];    // partition qubit i <- circuit qubit qubit[p][i]
+    uint8_t table[kMaxParts];  // vec[p] holds the strings' amplitudes only: branch s of string j at s m + j
 };
+
+// The index of every bit string inside one partition.
+__global__ void k_cut_index(const uint64_t *__restrict__ z, const CutSumArgs a, int p, uint64_t *__restrict__ zl) {
+    for (uint64_t j = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; j < a.m; j += uint64_t(gridDim.x) * blockDim.x) {
+        uint64_t v = 0;
+        for (int i = 0; i < a.nlocal[p]; ++i) {
+            const int q = a.qubit[p][i];
+            v |= ((z[j * a.nwords + (q >> 6)] >> (q & 63)) & 1ull) << i;
+        }
+        zl[j] = v;
+    }
+}
+
+// Keep the strings' amplitudes of a chunk of branches: out[s m + j] =
+// vec[(s << nlocal) | zl[j]].
+__global__ void k_cut_keep(const float2 *__restrict__ vec, const uint64_t *__restrict__ zl, uint64_t m, int nlocal,
+                           uint64_t nbranch, float2 *__restrict__ out) {
+    const uint64_t total = nbranch * m;
+    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < total; i += uint64_t(gridDim.x) * blockDim.x) {
+        const uint64_t s = i / m, j = i - s * m;
+        out[i] = vec[(s << nlocal) | zl[j]];
+    }
+}
 
 __global__ void k_cut_sum(const uint64_t *__restrict__ z, const CutSumArgs a, double2 *__restrict__ out) {
     const int lane = threadIdx.x & 31;
@@ -85,7 +128,7 @@ __global__ void k_cut_sum(const uint64_t *__restrict__ z, const CutSumArgs a, do
             for (int p = 0; p < a.P; ++p) {
                 uint64_t sp = 0;
                 for (int k = 0; k < a.nbits[p]; ++k) sp |= ((s >> a.cutbit[p][k]) & 1ull) << k;
-                const float2 v = a.vec[p][(sp << a.nlocal[p]) | zl[p]];
+                const float2 v = a.vec[p][a.table[p] ? sp * a.m + j : (sp << a.nlocal[p]) | zl[p]];
                 const double r = pr * v.x - pi * v.y;
                 pi = pr * v.y + pi * v.x;
                 pr = r;
@@ -140,13 +183,12 @@ void append_lowered(const Instr &ins, std::vector<PGate> *out) {
     out->insert(out->end(), g.begin(), g.end());
 }
 
-// One step of a partition's simulation: a stage of compiled tiled passes
-// over the low 2^nrun amplitudes, or (branch-prefix sharing) a fork that
-// copies the live 2^live amplitudes to the slots above them.
-struct HalfStep {
-    std::vector<void *> fns;  // compiled passes of a stage; empty for a fork
-    int nrun = 0, rb = 0;
-    int live = -1;            // fork: live qubits before the copy
+// A stage of a partition's simulation: compiled passes over the vector whose
+// first `level` branch bits are live.
+struct HalfStage {
+    std::vector<void *> fns;
+    int level = 0, rb = 0;
+    uint64_t last_tile = 0;  // tile qubits of the last pass
 };
 
 struct Half {            // one partition
@@ -156,35 +198,35 @@ struct Half {            // one partition
     std::vector<PGate> gates;
     std::vector<int> qubits;   // circuit qubit of local qubit i
     std::vector<int> cutbits;  // batched branch bit of partition bit j
-    float2 *d = nullptr;
+    float2 *d = nullptr;       // the whole vector, or (chunked) the strings' amplitudes
     bool init_all = false;     // every branch starts at its own |0> (no prefix sharing)
-    std::vector<HalfStep> steps;
+    bool remap = false;        // stages read the previous stage's vector (else copies in place)
+    int chunk = 0;             // branch bits of a chunk of the last stage (nbits: one chunk)
+    std::vector<unsigned> want;  // chunked: the tiles of the last pass that hold a string's index (empty: all)
+    const unsigned *d_want = nullptr;
+    std::vector<HalfStage> stages;
 };
 
-// Plan and compile `gates` as tiled passes over the low 2^nrun amplitudes.
-sv_status plan_stage(std::vector<HalfStep> *steps, const std::vector<PGate> &gates, int nrun) {
+// Plan and compile a stage as tiled passes over 2^nrun amplitudes, with the
+// pure branch-operator stages `before` it in its first pass.  With *remap the
+// passes read one vector and write another, which needs every branch bit
+// outside the tiles; *remap is cleared where that fails.
+sv_status plan_stage(HalfStage *st, const std::vector<std::vector<PGate>> &before, const std::vector<PGate> &gates,
+                     int nlocal, int nrun, bool *remap) {
     if (gates.empty()) return SV_OK;
     TilePlan<float> tp;
     sv_status s = plan_tiles<float>(gates, nrun, tile_config64(), &tp);
+    if (!s) s = prepend_diagonals(before, &tp);
     if (s) return s;
-    HalfStep st;
-    s = jit_tile_plan(tp, &st.fns);
-    if (s) return s;
-    st.nrun = nrun;
-    st.rb = tp.rb;
-    steps->push_back(std::move(st));
-    return SV_OK;
+    for (const TilePassArgs &pa : tp.passes) *remap = *remap && int(pa.tile_pos[tp.m - 1]) < nlocal;
+    tp.remap = *remap;
+    st->rb = tp.rb;
+    st->last_tile = 0;
+    for (int k = 0; k < tp.m && !tp.passes.empty(); ++k) st->last_tile |= uint64_t(1) << tp.passes.back().tile_pos[k];
+    return jit_tile_plan(tp, &st->fns);
 }
 
-// Branch-prefix sharing (on unless SV_CUT_PREFIX=0): the gates before the
-// first branch operator are the same for every branch, so they run once on
-// the 2^n_p amplitudes of branch 0; at the first operator on branch bit k the
-// live vector (branches with bits >= k clear, the low 2^(n_p + k) amplitudes)
-// is copied to the slots with bit k set, and the following gates run on the
-// doubled vector.  Work falls from 2^S G to the sum over stages of
-// 2^(n_p + k) G_k.  Amplitudes above the live vector are zero until copied
-// to, and gates keep zeros zero, so a stage may run on more qubits (the tile
-// size) than it has live.
+// Branch-prefix sharing (on unless SV_CUT_PREFIX=0).
 bool prefix_sharing() {
     const char *e = std::getenv("SV_CUT_PREFIX");
     return !(e && e[0] == '0');
@@ -193,8 +235,12 @@ bool prefix_sharing() {
 // Schedules by partition content (its gates, sizes, branch-bit count and the
 // code-generation settings): a repeated decomposition skips the planning, and
 // the compiled passes it names stay loaded for the process.
+struct Schedule {
+    bool init_all, remap;
+    std::vector<HalfStage> stages;
+};
 std::mutex g_sched_mu;
-std::unordered_map<std::string, std::pair<bool, std::vector<HalfStep>>> g_sched;
+std::unordered_map<std::string, Schedule> g_sched;
 constexpr size_t kSchedCacheMax = 256;
 
 std::string schedule_key(const Half &h, int S) {
@@ -225,8 +271,9 @@ sv_status plan_half(Half &h, int S) {
         std::lock_guard<std::mutex> lock(g_sched_mu);
         auto it = g_sched.find(key);
         if (it != g_sched.end()) {
-            h.init_all = it->second.first;
-            h.steps = it->second.second;
+            h.init_all = it->second.init_all;
+            h.remap = it->second.remap;
+            h.stages = it->second.stages;
             return SV_OK;
         }
     }
@@ -234,73 +281,203 @@ sv_status plan_half(Half &h, int S) {
     if (s) return s;
     std::lock_guard<std::mutex> lock(g_sched_mu);
     if (g_sched.size() >= kSchedCacheMax) g_sched.clear();
-    g_sched[key] = std::make_pair(h.init_all, h.steps);
+    g_sched[key] = Schedule{h.init_all, h.remap, h.stages};
     return SV_OK;
 }
 
 sv_status plan_half_uncached(Half &h, int S) {
-    h.steps.clear();
+    h.stages.clear();
     h.init_all = !prefix_sharing();
-    if (h.init_all) return plan_stage(&h.steps, h.gates, h.nq);
-    int live = h.nlocal;  // live amplitudes: 2^live
-    std::vector<PGate> stage;
-    auto fork = [&]() -> sv_status {
-        sv_status s = plan_stage(&h.steps, stage, live > kTileM64 ? live : kTileM64);
-        stage.clear();
-        if (s) return s;
-        HalfStep f;
-        f.live = live++;
-        h.steps.push_back(f);
-        return SV_OK;
-    };
-    for (const PGate &g : h.gates) {
-        // batched branch bits are only ever conditions of diagonal gates
-        const uint64_t branch = g.kind == 1 ? ((g.cmask & kQubitBits) >> h.nlocal) : 0;
-        while (branch >> (live - h.nlocal)) {
-            sv_status s = fork();
-            if (s) return s;
+    h.remap = !h.init_all && h.nlocal >= tile_config64().m;
+    if (h.init_all) {
+        HalfStage st;
+        st.level = S;
+        const sv_status s = plan_stage(&st, {}, h.gates, h.nlocal, h.nq, &h.remap);
+        h.stages.push_back(std::move(st));
+        return s;
+    }
+    // the gates between the first operators of successive branch bits, in
+    // circuit order; entry k runs with k branch bits live
+    std::vector<std::vector<PGate>> at(size_t(S) + 1);
+    {
+        int live = 0;
+        for (const PGate &g : h.gates) {
+            // batched branch bits are only ever conditions of diagonal gates
+            const uint64_t branch = g.kind == 1 ? ((g.cmask & kQubitBits) >> h.nlocal) : 0;
+            while (branch >> live) ++live;
+            at[size_t(live)].push_back(g);
         }
-        stage.push_back(g);
     }
-    while (live < h.nlocal + S) {  // every branch bit has operators; kept for the layout
-        sv_status s = fork();
-        if (s) return s;
+    auto diagonal = [](const std::vector<PGate> &gates) {
+        for (const PGate &g : gates)
+            if (g.kind != 1 || g.scale.re != 1.0 || g.scale.im != 0.0) return false;
+        return true;
+    };
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        h.stages.clear();
+        const bool remap = h.remap;
+        std::vector<std::vector<PGate>> before;
+        for (int k = 0; k <= S; ++k) {
+            if (k > 0 && k < S && diagonal(at[size_t(k)])) {  // joins the next stage (if it is not empty)
+                if (!at[size_t(k)].empty()) before.push_back(at[size_t(k)]);
+                continue;
+            }
+            HalfStage st;
+            st.level = k;
+            const int nrun = k == S ? h.nq : std::max(h.nlocal + k, kTileM64);
+            const sv_status s = plan_stage(&st, before, at[size_t(k)], h.nlocal, nrun, &h.remap);
+            if (s) return s;
+            before.clear();
+            h.stages.push_back(std::move(st));
+        }
+        if (h.remap == remap) break;  // (a stage whose tiles hold branch bits: all of them in place)
     }
-    return plan_stage(&h.steps, stage, h.nq);
+    return SV_OK;
+}
+
+// Amplitudes of the last stage's buffer above which it runs in chunks, and
+// the room the strings' amplitudes may take.
+constexpr int kChunkQubits = 28;
+constexpr size_t kKeepBytes = size_t(1) << 30;
+
+void choose_chunk(Half &h, size_t m) {
+    h.chunk = h.nbits;
+    if (!h.remap || h.nlocal + h.nbits <= kChunkQubits || h.stages.size() < 2) return;
+    if ((m << h.nbits) * sizeof(float2) > kKeepBytes) return;
+    const int prev = h.stages[h.stages.size() - 2].level;
+    h.chunk = std::min(h.nbits, std::max(prev, std::max(0, kChunkQubits - h.nlocal)));
+}
+
+// The tiles of a chunked partition's last pass that hold an amplitude of one
+// of the m strings (each tile of every branch needs running only if it does):
+// 1024 strings name 39% of the 2048 tiles of 24 qubits.
+void choose_tiles(Half &h, size_t m, const uint64_t *z, int nwords) {
+    h.want.clear();
+    const uint64_t ntiles = uint64_t(1) << (h.nlocal - tile_config64().m);
+    if (h.chunk >= h.nbits || m > ntiles) return;
+    const uint64_t tile = h.stages.back().last_tile;
+    for (size_t j = 0; j < m; ++j) {
+        uint64_t t = 0;
+        int k = 0;
+        for (int i = 0; i < h.nlocal; ++i) {
+            if (tile >> i & 1) continue;
+            const int q = h.qubits[size_t(i)];
+            t |= ((z[j * size_t(nwords) + size_t(q >> 6)] >> (q & 63)) & 1u) << k++;
+        }
+        h.want.push_back(unsigned(t));
+    }
+    std::sort(h.want.begin(), h.want.end());
+    h.want.erase(std::unique(h.want.begin(), h.want.end()), h.want.end());
+}
+
+size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
+
+// Bytes of the stage vectors a partition needs besides h.d: every stage but
+// the last, and the chunk buffer of a chunked one.
+size_t work_bytes(const Half &h) {
+    if (!h.remap) return 0;
+    size_t b = 0;
+    for (size_t i = 0; i + 1 < h.stages.size(); ++i) b += align256(sizeof(float2) << (h.nlocal + h.stages[i].level));
+    if (h.chunk < h.nbits) b += align256(sizeof(float2) << (h.nlocal + h.chunk));
+    return b;
+}
+
+// Bytes of h.d.
+size_t result_bytes(const Half &h, size_t m) {
+    return h.chunk < h.nbits ? (m << h.nbits) * sizeof(float2) : sizeof(float2) << h.nq;
 }
 
 // Run a partition's schedule for the branch part whose fixed bits are param.
-sv_status exec_half(Half &h, cudaStream_t st, int S, uint64_t param) {
-    SV_CUDA_TRY(cudaMemsetAsync(h.d, 0, sizeof(float2) << h.nq, st));
-    if (h.init_all) k_branch_init<<<64, 256, 0, st>>>(h.d, h.nlocal, S);
-    else k_branch_init<<<1, 32, 0, st>>>(h.d, h.nlocal, 0);
-    sv_status s = check_launch(cudaGetLastError(), "k_branch_init");
-    if (s) return s;
-    sv_state tmp;
-    tmp.dt = SV_C64;
-    tmp.data = h.d;
-    tmp.stream = st;
-    SV_CUDA_TRY(cudaGetDevice(&tmp.device));
-    for (const HalfStep &step : h.steps) {
-        if (step.fns.empty()) {
-            const size_t bytes = sizeof(float2) << step.live;
-            const cudaError_t e =
-                cudaMemcpyAsync(reinterpret_cast<char *>(h.d) + bytes, h.d, bytes, cudaMemcpyDeviceToDevice, st);
-            if (e != cudaSuccess) {
-                s = cuda_status(e, "cudaMemcpyAsync (branch fork)");
-                break;
+// work: work_bytes(h); zl: the strings' indices in this partition (chunked).
+sv_status exec_half(Half &h, cudaStream_t st, int S, uint64_t param, char *work, const uint64_t *zl, size_t m) {
+    if (!h.remap) {
+        // in place: the live amplitudes grow by copies (zeros above them up to one tile)
+        const size_t live = sizeof(float2) << (h.nlocal > kTileM64 ? h.nlocal : kTileM64);
+        SV_CUDA_TRY(cudaMemsetAsync(h.d, 0, h.init_all ? sizeof(float2) << h.nq : live, st));
+        if (h.init_all) k_branch_init<<<64, 256, 0, st>>>(h.d, h.nlocal, S);
+        else k_branch_init<<<1, 32, 0, st>>>(h.d, h.nlocal, 0);
+        sv_status s = check_launch(cudaGetLastError(), "k_branch_init");
+        if (s) return s;
+        sv_state tmp;
+        tmp.dt = SV_C64;
+        tmp.data = h.d;
+        tmp.stream = st;
+        SV_CUDA_TRY(cudaGetDevice(&tmp.device));
+        int level = h.init_all ? S : 0;
+        for (const HalfStage &stage : h.stages) {
+            for (; level < stage.level; ++level) {
+                const size_t bytes = sizeof(float2) << (h.nlocal + level);
+                const cudaError_t e =
+                    cudaMemcpyAsync(reinterpret_cast<char *>(h.d) + bytes, h.d, bytes, cudaMemcpyDeviceToDevice, st);
+                if (e != cudaSuccess) return cuda_status(e, "cudaMemcpyAsync (branch fork)");
             }
-            continue;
-        }
-        tmp.n = step.nrun;
-        for (void *fn : step.fns) {
-            s = check_launch(launch_jit_pass(&tmp, fn, step.nrun, step.rb, param), "branch pass");
+            tmp.n = h.init_all ? h.nq : std::max(h.nlocal + level, kTileM64);
+            for (void *fn : stage.fns) {
+                s = check_launch(launch_jit_pass(&tmp, fn, tmp.n, stage.rb, param), "branch pass");
+                if (s) break;
+            }
             if (s) break;
         }
-        if (s) break;
+        tmp.data = nullptr;
+        return s;
     }
-    tmp.data = nullptr;
-    return s;
+    const int tile = tile_config64().m;
+    auto tiles = [&](int level) { return uint64_t(1) << (h.nlocal + level - tile); };
+    const float2 *src = nullptr;
+    int src_level = 0;
+    for (size_t i = 0; i < h.stages.size(); ++i) {
+        const HalfStage &stage = h.stages[i];
+        const bool last = i + 1 == h.stages.size();
+        const int live = last ? h.chunk : stage.level;  // branch bits of this stage's vector
+        float2 *dst = h.d;
+        if (!last || h.chunk < h.nbits) {
+            dst = reinterpret_cast<float2 *>(work);
+            work += align256(sizeof(float2) << (h.nlocal + live));
+        }
+        if (i == 0) {  // |0...0> of branch 0
+            SV_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(float2) << h.nlocal, st));
+            k_branch_init<<<1, 32, 0, st>>>(dst, h.nlocal, 0);
+            const sv_status s = check_launch(cudaGetLastError(), "k_branch_init");
+            if (s) return s;
+            src = dst;
+        }
+        for (uint64_t c = 0; c < uint64_t(1) << (stage.level - live); ++c) {
+            const float2 *from = src;
+            uint64_t smask = tiles(src_level) - 1;
+            const uint64_t dmask = tiles(live) - 1;
+            for (size_t k = 0; k < stage.fns.size(); ++k) {
+                RemapTiles r{from, dst, c * tiles(live), tiles(live), smask, dmask};
+                if (smask < dmask) {
+                    // a fork: the tiles that read the same source tile run next
+                    // to each other, so that HBM delivers it once (2^28
+                    // amplitudes from 2^25: 598 us in plain order, 446 so)
+                    r.group = smask + 1;
+                    r.rot = unsigned(live - src_level);
+                }
+                if (last && h.d_want && k + 1 == stage.fns.size()) {
+                    r.list = h.d_want;
+                    r.nlist = unsigned(h.want.size());
+                    r.group = tiles(0);
+                    r.ntiles = uint64_t(h.want.size()) << live;
+                }
+                const sv_status s = check_launch(launch_jit_remap(stage.fns[k], stage.rb, r, param, st), "branch pass");
+                if (s) return s;
+                from = dst;
+                smask = dmask;
+            }
+            if (last && h.chunk < h.nbits) {
+                const uint64_t nb = uint64_t(1) << live;
+                const uint64_t blocks = (nb * m + 255) / 256;
+                k_cut_keep<<<unsigned(blocks < 4096 ? blocks : 4096), 256, 0, st>>>(dst, zl, m, h.nlocal, nb,
+                                                                                    h.d + c * nb * m);
+                const sv_status s = check_launch(cudaGetLastError(), "k_cut_keep");
+                if (s) return s;
+            }
+        }
+        src = dst;
+        src_level = live;
+    }
+    return SV_OK;
 }
 
 }  // namespace
@@ -454,73 +631,100 @@ static sv_status cut_impl(const char *text, int n, const uint8_t *part_of, int P
     if (s) return s;
     if (m == 0) return SV_OK;
 
-    // device memory: the batched vectors + bit strings + results
-    size_t bytesV = 0;
-    for (int p = 0; p < P; ++p) bytesV += sizeof(float2) << parts[p].nq;
-    const size_t bytesZ = m * size_t(nwords) * sizeof(uint64_t), bytesO = m * sizeof(double2);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    for (int p = 0; p < P && s == SV_OK; ++p) s = plan_half(parts[p], parts[p].nbits);
+    if (s) return s;
+    for (int p = 0; p < P; ++p) {
+        choose_chunk(parts[p], m);
+        choose_tiles(parts[p], m, z, nwords);
+    }
+
+    // device memory: the vectors (or kept amplitudes), one workspace for the
+    // partitions, which run one after another, bit strings, indices, results
+    size_t bytesV = 0, bytesW = 0;
+    bool kept = false;
+    for (int p = 0; p < P; ++p) {
+        bytesV += align256(result_bytes(parts[p], m));
+        bytesV += align256(parts[p].want.size() * sizeof(unsigned));
+        bytesW = std::max(bytesW, work_bytes(parts[p]));
+        kept = kept || parts[p].chunk < parts[p].nbits;
+    }
+    const size_t bytesZ = align256(m * size_t(nwords) * sizeof(uint64_t)), bytesO = align256(m * sizeof(double2));
+    const size_t bytesI = kept ? align256(m * sizeof(uint64_t)) : 0;
+    const size_t total = bytesV + bytesW + bytesZ + bytesO + bytesI;
     size_t free_b = 0, total_b = 0;
     SV_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-    if (bytesV + bytesZ + bytesO + (size_t(256) << 20) > free_b) {
-        set_error("decomposition needs %zu bytes of device memory, %zu free", bytesV + bytesZ + bytesO, free_b);
+    if (total + (size_t(256) << 20) > free_b) {
+        set_error("decomposition needs %zu bytes of device memory, %zu free", total, free_b);
         return SV_ERR_OOM;
     }
     if (fault_injected("alloc")) {
         set_error("injected allocation failure");
         return SV_ERR_OOM;
     }
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    uint64_t *dz = nullptr;
-    double2 *dout = nullptr;
-    auto release = [&]() {
-        cudaStreamSynchronize(st);
-        for (int p = 0; p < P; ++p)
-            if (parts[p].d) cudaFree(parts[p].d);
-        if (dz) cudaFree(dz);
-        if (dout) cudaFree(dout);
+    char *mem = nullptr;
+    cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&mem), total);
+    if (e != cudaSuccess) return cuda_status(e, "cudaMalloc (decomposition)");
+    char *at = mem;
+    auto take = [&](size_t b) {
+        char *r = at;
+        at += b;
+        return r;
     };
-    cudaError_t e = cudaSuccess;
-    for (int p = 0; p < P && e == cudaSuccess; ++p) e = cudaMalloc(&parts[p].d, sizeof(float2) << parts[p].nq);
-    if (e == cudaSuccess) e = cudaMalloc(&dz, bytesZ);
-    if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&dout), bytesO);
-    if (e != cudaSuccess) {
-        release();
-        return cuda_status(e, "cudaMalloc (decomposition)");
+    for (int p = 0; p < P; ++p) parts[p].d = reinterpret_cast<float2 *>(take(align256(result_bytes(parts[p], m))));
+    char *work = take(bytesW);
+    uint64_t *dz = reinterpret_cast<uint64_t *>(take(bytesZ));
+    double2 *dout = reinterpret_cast<double2 *>(take(bytesO));
+    uint64_t *dzl = reinterpret_cast<uint64_t *>(take(bytesI));
+    CutSumArgs a{};
+    a.P = P;
+    a.Sv = Svar;
+    a.nwords = nwords;
+    a.m = m;
+    a.w = form == 1 ? std::ldexp(1.0, -S) : 1.0;
+    for (int p = 0; p < P; ++p) {
+        a.vec[p] = parts[p].d;
+        a.nlocal[p] = parts[p].nlocal;
+        a.nbits[p] = parts[p].nbits;
+        a.table[p] = parts[p].chunk < parts[p].nbits;
+        for (int j = 0; j < parts[p].nbits; ++j) a.cutbit[p][j] = uint8_t(parts[p].cutbits[size_t(j)]);
+        for (int i = 0; i < parts[p].nlocal; ++i) a.qubit[p][i] = uint8_t(parts[p].qubits[size_t(i)]);
     }
-    if (s == SV_OK) {
-        e = cudaMemcpyAsync(dz, z, bytesZ, cudaMemcpyHostToDevice, st);
-        if (e != cudaSuccess) s = cuda_status(e, "cudaMemcpyAsync");
+    e = cudaMemcpyAsync(dz, z, m * size_t(nwords) * sizeof(uint64_t), cudaMemcpyHostToDevice, st);
+    for (int p = 0; p < P && e == cudaSuccess; ++p) {
+        parts[p].d_want = nullptr;
+        if (parts[p].want.empty()) continue;
+        const size_t b = parts[p].want.size() * sizeof(unsigned);
+        unsigned *w = reinterpret_cast<unsigned *>(take(align256(b)));
+        e = cudaMemcpyAsync(w, parts[p].want.data(), b, cudaMemcpyHostToDevice, st);
+        parts[p].d_want = w;
     }
-    for (int p = 0; p < P && s == SV_OK; ++p) s = plan_half(parts[p], parts[p].nbits);
+    if (e != cudaSuccess) s = cuda_status(e, "cudaMemcpyAsync");
+    const size_t blocks = (m + 7) / 8 < 4096 ? (m + 7) / 8 : 4096;
     for (size_t ip = 0; ip < todo.size() && s == SV_OK; ++ip) {
         // every part runs the same compiled passes (its fixed branch bits are
         // the launch parameter) on the same buffers; the stream orders its
         // halves after the previous part's sum
-        for (int p = 0; p < P && s == SV_OK; ++p) s = exec_half(parts[p], st, parts[p].nbits, todo[ip]);
-        if (s != SV_OK) break;
-        CutSumArgs a{};
-        a.accumulate = ip > 0;
-        a.P = P;
-        a.Sv = Svar;
-        a.nwords = nwords;
-        a.m = m;
-        a.w = form == 1 ? std::ldexp(1.0, -S) : 1.0;
-        for (int p = 0; p < P; ++p) {
-            a.vec[p] = parts[p].d;
-            a.nlocal[p] = parts[p].nlocal;
-            a.nbits[p] = parts[p].nbits;
-            for (int j = 0; j < parts[p].nbits; ++j) a.cutbit[p][j] = uint8_t(parts[p].cutbits[size_t(j)]);
-            for (int i = 0; i < parts[p].nlocal; ++i) a.qubit[p][i] = uint8_t(parts[p].qubits[size_t(i)]);
+        for (int p = 0; p < P && s == SV_OK; ++p) {
+            if (a.table[p]) {
+                k_cut_index<<<unsigned(blocks), 256, 0, st>>>(dz, a, p, dzl);
+                s = check_launch(cudaGetLastError(), "k_cut_index");
+                if (s) break;
+            }
+            s = exec_half(parts[p], st, parts[p].nbits, todo[ip], work, dzl, m);
         }
-        const size_t blocks = (m + 7) / 8 < 4096 ? (m + 7) / 8 : 4096;
+        if (s != SV_OK) break;
+        a.accumulate = ip > 0;
         k_cut_sum<<<unsigned(blocks), 256, 0, st>>>(dz, a, dout);
         s = check_launch(cudaGetLastError(), "k_cut_sum");
     }
     if (s == SV_OK) {
-        e = cudaMemcpyAsync(out, dout, bytesO, cudaMemcpyDeviceToHost, st);
+        e = cudaMemcpyAsync(out, dout, m * sizeof(double2), cudaMemcpyDeviceToHost, st);
         if (e != cudaSuccess) s = cuda_status(e, "cudaMemcpyAsync");
     }
     if (s == SV_OK) s = sync_stream(st, "sv_cut_amplitudes");
-    release();
+    cudaStreamSynchronize(st);
+    cudaFree(mem);
     return s;
 }
 

@@ -34,6 +34,7 @@ enum TileOpType : int32_t {
     TOP_NEG = 4,     // negate where the condition holds; a = register condition id
     TOP_SEG = 5,     // start segment a (shared-memory transposition)
     TOP_SCALE = 6,   // multiply every amplitude by u[0] + i u[1]
+    TOP_FLUSH = 7,   // apply every register's owed factors now
 };
 
 // Structured kinds: U = c * M with M below; c is deferred to a TOP_SCALE.
@@ -103,6 +104,7 @@ struct TilePlan {
     int ctas = 2;
     bool direct = true;
     bool prefetch = false;
+    bool remap = false;  // passes read one vector and write another (launch_jit_remap)
     std::vector<TilePassArgs> passes;
     std::vector<TileOp<R>> ops;
     std::vector<TileSeg> segs;
@@ -138,6 +140,11 @@ template <typename R>
 sv_status plan_tiles(const Circuit &circ, int n, const TileConfig &cfg, TilePlan<R> *out) {
     return plan_tiles<R>(lower_for_tiles(circ), n, cfg, out);
 }
+
+// Put groups of diagonal gates (no deferred scalars) before everything else in
+// a plan's first pass.  Each group's factors are applied to the amplitudes at
+// its end, so the arithmetic is that of one pass per group before the plan.
+sv_status prepend_diagonals(const std::vector<std::vector<PGate>> &groups, TilePlan<float> *tp);
 
 // Tile geometry of the kernels: complex64 2^13-amplitude tiles with 32
 // amplitudes per thread, complex128 2^12 with 16.
@@ -176,6 +183,21 @@ int tile_low64();
 // Launch one compiled pass over the whole state (grid = 2^(n-m) CTAs of
 // 2^(m-rb) threads); param: the launch parameter bits (kParamBit0).
 cudaError_t launch_jit_pass(sv_state *h, void *fn, int n, int rb, uint64_t param = 0);
+// Launch ntiles tiles of a pass compiled with remap.  The conditions of its
+// gates test the tile number, whose bits under smask (dmask) address the tile
+// in src (dst).  Tile numbers: first, first + 1, ..., in the order of
+// first + group * g + k with g = 0 .. 2^rot - 1 running fastest, or with a list
+// (device array) first + group * g + list[k], k < nlist, for g = 0, 1, ...
+struct RemapTiles {
+    const void *src;
+    void *dst;
+    unsigned long long first, ntiles, smask, dmask;
+    const unsigned *list = nullptr;
+    unsigned nlist = 1;
+    unsigned long long group = 0;
+    unsigned rot = 0;
+};
+cudaError_t launch_jit_remap(void *fn, int rb, const RemapTiles &t, uint64_t param, cudaStream_t st);
 const char *tile_kernel_name(const sv_state *h);
 // The code-generation switches (environment) that shape a compiled pass, as
 // part of a plan-cache key.

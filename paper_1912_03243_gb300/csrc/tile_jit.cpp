@@ -141,7 +141,7 @@ HbmIo hbm_io(const TilePlan<R> &tp, size_t pass) {
     // is free from its gather on and takes the next tile's copy; the first
     // segment then gathers the copied tile from shared memory
     const bool store = on && contiguous(last);
-    const bool prefetch = tp.prefetch && store && first >= 0;
+    const bool prefetch = tp.prefetch && store && first >= 0 && !tp.remap;
     return HbmIo{on && contiguous(first) && !prefetch, store, nseg, prefetch};
 }
 
@@ -191,8 +191,15 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
     int tpos[kTileMaxQ];
     for (int k = 0; k < tbits; ++k) tpos[k] = pa.tile_pos[k + G.EPC_LOG];
     const int ctas = tp.pass_ctas.empty() ? tp.ctas : tp.pass_ctas[pass];
-    o << "extern \"C\" __global__ void __launch_bounds__(" << G.NT << ", " << ctas << ") svp(" << C2T
-      << "* __restrict__ psi, const u64 prm, const u64 ntiles) {\n";
+    o << "extern \"C\" __global__ void __launch_bounds__(" << G.NT << ", " << ctas << ") svp(";
+    // remap: tiles are read from src and written to dst (which may be the same
+    // vector); conditions test the tile number, its masked bits address src and dst
+    if (tp.remap)
+        o << "const " << C2T << "* src, " << C2T << "* dst, const u64 prm, const u64 cta0, const u64 smask, const u64 dmask, const u32* list, const u32 nlist, const u64 group, const u32 rot) {\n";
+    else
+        o << C2T << "* __restrict__ psi, const u64 prm, const u64 ntiles) {\n";
+    const char *LP = tp.remap ? "src" : "psi", *SP = tp.remap ? "dst" : "psi";
+    const char *LC = tp.remap ? "cts" : "cta", *SC = tp.remap ? "ctd" : "cta";
     o << "  extern __shared__ __align__(16) unsigned char smem[];\n";
     o << "  " << C2T << "* sm = reinterpret_cast<" << C2T << "*>(smem);\n";
     // the CTA index is the tile number (persistent CTAs: the loop variable);
@@ -208,7 +215,7 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
         emit_deposit(o, "g0", "t", tpos, tbits, "u64");
         o << "  const u32 s0 = swz(t);\n";
         for (int i = 0; i < iters; ++i)
-            o << "  cpa16(smem + ((s0 ^ " << si[size_t(i)] << "u) << 4), psi + (g0 | " << gi[size_t(i)] << "ull));\n";
+            o << "  cpa16(smem + ((s0 ^ " << si[size_t(i)] << "u) << 4), " << LP << " + (g0 | " << gi[size_t(i)] << "ull));\n";
         o << "  asm volatile(\"cp.async.commit_group;\\n\" ::: \"memory\");\n  }\n";
     };
     if (io.prefetch) {
@@ -216,16 +223,38 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
         emit_tile_copy("u64(blockIdx.x)");
         o << "  for (u64 cta = blockIdx.x; cta < ntiles; cta += gridDim.x) {\n";
         o << "  asm volatile(\"cp.async.wait_group 0;\\n\" ::: \"memory\");\n  __syncthreads();\n";
+    } else if (tp.remap) {
+        o << "  const u64 cta = cta0 + (list ? (blockIdx.x / nlist) * group + list[blockIdx.x % nlist]\n"
+             "      : (blockIdx.x & ((1u << rot) - 1u)) * group + (blockIdx.x >> rot));\n"
+             "  const u64 cts = cta & smask, ctd = cta & dmask;\n";
+        // a factor of zero on whole tiles (a branch projector on outer bits):
+        // those tiles are zero whatever was in them
+        std::string zero;
+        for (int i = pa.op_begin; i < pa.op_end; ++i) {
+            const TileOp<R> &op = tp.ops[size_t(i)];
+            if (op.type != TOP_PHASE || op.u[0] != R(0) || op.u[1] != R(0) || op.rmask || op.tmask || op.pmask || !op.gmask)
+                continue;
+            zero += std::string(zero.empty() ? "" : " || ") + "(cta & " + std::to_string(compress(op.gmask)) +
+                    "ull) == " + std::to_string(compress(op.gval)) + "ull";
+        }
+        if (!zero.empty()) {
+            o << "  if (" << zero << ") {\n  u64 g0 = 0;\n";
+            emit_deposit(o, "g0", "t", tpos, tbits, "u64");
+            emit_deposit(o, "g0", SC, opos, pa.nouter, "u64");
+            for (int i = 0; i < iters; ++i)
+                o << "  *reinterpret_cast<int4*>(" << SP << " + (g0 | " << gi[size_t(i)] << "ull)) = make_int4(0, 0, 0, 0);\n";
+            o << "  return;\n  }\n";
+        }
     } else {
         o << "  const u64 cta = blockIdx.x;\n";
     }
     if (!io.load && !io.prefetch) {
         o << "  {\n  u64 g0 = 0;\n";
-        emit_deposit(o, "g0", "cta", opos, pa.nouter, "u64");
+        emit_deposit(o, "g0", LC, opos, pa.nouter, "u64");
         emit_deposit(o, "g0", "t", tpos, tbits, "u64");
         o << "  const u32 s0 = swz(t);\n";
         for (int i = 0; i < iters; ++i)
-            o << "  cpa16(smem + ((s0 ^ " << si[size_t(i)] << "u) << 4), psi + (g0 | " << gi[size_t(i)] << "ull));\n";
+            o << "  cpa16(smem + ((s0 ^ " << si[size_t(i)] << "u) << 4), " << LP << " + (g0 | " << gi[size_t(i)] << "ull));\n";
         o << "  }\n";
         o << "  asm volatile(\"cp.async.commit_group;\\ncp.async.wait_group 0;\\n\" ::: \"memory\");\n";
         o << "  __syncthreads();\n";
@@ -233,11 +262,11 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
     // Global offset of a segment's registers: the CTA's outer bits and the
     // thread's tile bits (at their global positions) in one per-thread base,
     // plus a constant per register slot (disjoint bits, so + is |).
-    auto emit_thread_base = [&](const TileSeg &sg, const char *name) {
+    auto emit_thread_base = [&](const TileSeg &sg, const char *name, const char *cta) {
         int gpos[kTileMaxQ];
         for (int k = 0; k < tbits; ++k) gpos[k] = pa.tile_pos[sg.tpos[k]];
         o << "  u64 " << name << " = 0;\n";
-        emit_deposit(o, name, "cta", opos, pa.nouter, "u64");
+        emit_deposit(o, name, cta, opos, pa.nouter, "u64");
         emit_deposit(o, name, "t", gpos, tbits, "u64");
     };
     auto reg_goff = [&](const TileSeg &sg, int v) {
@@ -388,7 +417,7 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
             const bool last_seg = seg_index == io.nseg;
             if (from_hbm) {
                 o << "  {\n";
-                emit_thread_base(sg, "gq");
+                emit_thread_base(sg, "gq", LC);
             }
             for (int v = 0; v < G.NR; ++v) {
                 uint32_t d = 0;
@@ -396,7 +425,7 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
                     if (v >> s & 1) d |= 1u << sg.rpos[s];
                 pv[v] = Geo<R>::phys(d);
                 if (from_hbm)
-                    o << "  { const " << C2T << " a = psi[gq + " << reg_goff(sg, v) << "ull]; xr[" << v
+                    o << "  { const " << C2T << " a = " << LP << "[gq + " << reg_goff(sg, v) << "ull]; xr[" << v
                       << "] = a.x; xi[" << v << "] = a.y; }\n";
                 else
                     o << "  { " << C2T << " a = sm[pj ^ " << pv[v] << "u]; xr[" << v << "] = a.x; xi[" << v
@@ -410,6 +439,10 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
                 emit_tile_copy("nxt");
                 o << "  }\n";
             }
+            continue;
+        }
+        if (op.type == TOP_FLUSH) {
+            for (int v = 0; v < G.NR; ++v) materialise(v);
             continue;
         }
         // runtime condition on thread / CTA bits (branch-free select)
@@ -630,11 +663,11 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
         if (cur_seg >= 0) {
             const TileSeg &sg = tp.segs[size_t(cur_seg)];
             o << "  {\n";
-            emit_thread_base(sg, "gq");
+            emit_thread_base(sg, "gq", SC);
             for (int v = 0; v < G.NR; ++v) {
                 if (!rsg[v].empty() || !rph[v].empty() || me[v] != 0) materialise(v);
                 const char *neg = sgn[v] < 0 ? "-" : "";
-                o << "  psi[gq + " << reg_goff(sg, v) << "ull] = make_" << C2T << "(" << neg << "xr[" << v << "], "
+                o << "  " << SP << "[gq + " << reg_goff(sg, v) << "ull] = make_" << C2T << "(" << neg << "xr[" << v << "], "
                   << neg << "xi[" << v << "]);\n";
                 sgn[v] = 1;
             }
@@ -650,10 +683,10 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
     }
     o << "  {\n  u64 g0 = 0;\n";
     emit_deposit(o, "g0", "t", tpos, tbits, "u64");
-    emit_deposit(o, "g0", "cta", opos, pa.nouter, "u64");
+    emit_deposit(o, "g0", SC, opos, pa.nouter, "u64");
     o << "  const u32 s0 = swz(t);\n";
     for (int i = 0; i < iters; ++i)
-        o << "  *reinterpret_cast<int4*>(psi + (g0 | " << gi[size_t(i)] << "ull)) = *reinterpret_cast<const int4*>(smem + ((s0 ^ "
+        o << "  *reinterpret_cast<int4*>(" << SP << " + (g0 | " << gi[size_t(i)] << "ull)) = *reinterpret_cast<const int4*>(smem + ((s0 ^ "
           << si[size_t(i)] << "u) << 4));\n";
     o << "  }\n";
     o << "}\n";
@@ -1078,6 +1111,22 @@ sv_status jit_compile_check(const TilePlan<double> &tp) { return compile_check_i
 const char *tile_kernel_name(const sv_state *h) {
     static const char *n64[] = {"svp<f32,13,4>", "svp<f32,13,5>", "svp<f32,13,6>"};
     return h->dt == SV_C64 ? n64[tile_rb64() - 4] : "svp<f64,12,4>";
+}
+
+cudaError_t launch_jit_remap(void *fn, int rb, const RemapTiles &r, uint64_t param, cudaStream_t st) {
+    int m = 0, smem = 0;
+    {
+        std::lock_guard<std::mutex> lock(g_jit_mu);
+        const auto it = g_jit_smem.find(fn);
+        if (it == g_jit_smem.end()) return cudaErrorInvalidResourceHandle;
+        smem = it->second.smem;
+        m = it->second.m;
+    }
+    RemapTiles t = r;
+    unsigned long long prm = param;
+    void *args[] = {&t.src, &t.dst, &prm, &t.first, &t.smask, &t.dmask, &t.list, &t.nlist, &t.group, &t.rot};
+    return cudaLaunchKernel(static_cast<const void *>(fn), dim3(unsigned(t.ntiles)), dim3(1u << (m - rb)), args,
+                            size_t(smem), st);
 }
 
 cudaError_t launch_jit_pass(sv_state *h, void *fn, int n, int rb, uint64_t param) {

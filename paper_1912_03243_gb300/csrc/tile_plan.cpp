@@ -825,6 +825,60 @@ sv_status plan_tiles_one(const std::vector<PGate> &G, int n, const TileConfig &c
     return SV_OK;
 }
 
+sv_status prepend_diagonals(const std::vector<std::vector<PGate>> &groups, TilePlan<float> *tp) {
+    if (groups.empty()) return SV_OK;
+    if (tp->passes.empty() || tp->ops[size_t(tp->passes[0].op_begin)].type != TOP_SEG) {
+        set_error("no pass to prepend diagonal gates to");
+        return SV_ERR_UNSUPPORTED;
+    }
+    const TilePassArgs &pa = tp->passes[0];
+    const TileSeg &sg = tp->segs[size_t(tp->ops[size_t(pa.op_begin)].a)];
+    int tbit[64], slot[kTileMaxQ];
+    for (int q = 0; q < 64; ++q) tbit[q] = -1;
+    for (int k = 0; k < tp->m; ++k) tbit[pa.tile_pos[k]] = k;
+    for (int k = 0; k < kTileMaxQ; ++k) slot[k] = -1;
+    for (int r = 0; r < tp->rb; ++r) slot[sg.rpos[r]] = r;
+    std::vector<TileOp<float>> ops;
+    for (const std::vector<PGate> &group : groups) {
+        for (const PGate &g : group) {
+            TileOp<float> op{};
+            for (int q = 0; q < 64; ++q) {
+                if (!(g.cmask >> q & 1)) continue;
+                const uint64_t want = g.cval >> q & 1;
+                if (q >= kParamBit0) {
+                    op.pmask |= 1u << (q - kParamBit0);
+                    op.pval |= uint32_t(want) << (q - kParamBit0);
+                } else if (tbit[q] < 0) {
+                    op.gmask |= uint64_t(1) << q;
+                    op.gval |= want << q;
+                } else if (slot[tbit[q]] >= 0) {
+                    op.rmask |= 1u << slot[tbit[q]];
+                    op.rval |= uint32_t(want) << slot[tbit[q]];
+                } else {
+                    op.tmask |= 1u << tbit[q];
+                    op.tval |= uint32_t(want) << tbit[q];
+                }
+            }
+            const cd ph = toc(g.u[0]);
+            op.type = ph == cd(-1) ? TOP_NEG : TOP_PHASE;
+            op.a = reg_cond_id(op.rmask, op.rval);
+            op.u[0] = float(ph.real());
+            op.u[1] = float(ph.imag());
+            ops.push_back(op);
+        }
+        TileOp<float> flush{};
+        flush.type = TOP_FLUSH;
+        ops.push_back(flush);
+    }
+    const int add = int(ops.size());
+    tp->ops.insert(tp->ops.begin() + pa.op_begin + 1, ops.begin(), ops.end());
+    for (size_t i = 0; i < tp->passes.size(); ++i) {
+        if (i > 0) tp->passes[i].op_begin += add;
+        tp->passes[i].op_end += add;
+    }
+    return SV_OK;
+}
+
 template sv_status plan_tiles<float>(const std::vector<PGate> &, int, const TileConfig &, TilePlan<float> *);
 template sv_status plan_tiles<double>(const std::vector<PGate> &, int, const TileConfig &, TilePlan<double> *);
 

@@ -254,3 +254,29 @@ def test_prefix_sharing_matches_batched(S, monkeypatch, form):
         got, s1 = S.sv_cut_amplitudes(c, c.n, mask, z, form=form)
         assert s0 == s1
         close(got, ref)
+
+
+@pytest.mark.parametrize("rows,cols,m", [(6, 8, 1), (6, 8, 5000), (5, 8, 700)])
+def test_chunked_last_stage(S, monkeypatch, rows, cols, m):
+    """Partitions of more than 2^28 batched amplitudes run their last stage in
+    chunks of branches, on the tiles that hold a string where few are asked
+    for; the amplitudes are those of the whole vectors (more strings than
+    their kept amplitudes may take room, and every branch from the first gate
+    on with SV_CUT_PREFIX=0)."""
+    import torch
+
+    if torch.cuda.mem_get_info()[0] < (90 << 30):
+        pytest.skip("not enough device memory")
+    n = rows * cols
+    c = C.grid_circuit(rows, cols, 8, 3)
+    mask = C.grid_partition_mask(rows, cols, rows // 2)
+    z = C.random_bitstrings(600000, n, 11)
+    z[:3] = [0, (1 << n) - 1, 1]
+    got, s = S.sv_cut_amplitudes(c, n, mask, z[:m])
+    assert s == 8
+    whole, _ = S.sv_cut_amplitudes(c, n, mask, z)
+    tol = 1e-5 * np.max(np.abs(whole))  # (|<0..0|C|0>| itself is zero here)
+    assert np.max(np.abs(got - whole[:m])) <= tol
+    monkeypatch.setenv("SV_CUT_PREFIX", "0")
+    batched, _ = S.sv_cut_amplitudes(c, n, mask, z[:m])
+    assert np.max(np.abs(got - batched)) <= tol
