@@ -71,7 +71,8 @@ typedef enum {
 
 /* Circuit execution modes (sv_run_circuit, sv_plan_create). */
 typedef enum {
-    SV_MODE_PERGATE = 0,     /* one HBM pass per gate (Eq. 1 per gate) */
+    SV_MODE_PERGATE = 0,     /* one HBM pass per gate (Eq. 1 per gate); several
+                                gates per launch where the state stays in L2 */
     SV_MODE_TILED = 1,       /* many gates per HBM pass: 2^13-amplitude tiles in
                                 shared memory, one compiled kernel per pass */
     SV_MODE_FUSED = 2,       /* gates fused into dense k-qubit blocks (k = 3..6

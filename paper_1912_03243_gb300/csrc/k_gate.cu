@@ -12,6 +12,9 @@
 // the control set is read); a control inside the vector is a per-lane test.
 // Diagonal gates with u00 = 1 (T, S, Z, P, CZ, CP) read and write only the
 // amplitudes they change.
+#include <algorithm>
+#include <cmath>
+
 #include "sv_internal.h"
 
 namespace sv {
@@ -218,14 +221,21 @@ __global__ void __launch_bounds__(Shape1<float>::threads) k_gate_inner(float4 *_
 // another phase.
 enum PhaseForm { P_GENERAL = 0, P_NEG, P_I, P_MI };
 
+// -x as a flip of the sign bit: the compiler's own negation of a double that
+// is stored as it is goes through the FP64 pipe.
+__device__ __forceinline__ float neg(float x) { return -x; }
+__device__ __forceinline__ double neg(double x) {
+    return __hiloint2double(__double2hiint(x) ^ int(0x80000000u), __double2loint(x));
+}
+
 template <int F, typename R>
 __device__ __forceinline__ void phase1(R pr, R pi, R &x, R &y) {
     if constexpr (F == P_NEG) {
-        x = -x;
-        y = -y;
+        x = neg(x);
+        y = neg(y);
     } else if constexpr (F == P_I || F == P_MI) {
-        const R t = F == P_I ? x : -x;
-        x = F == P_I ? -y : y;
+        const R t = F == P_I ? x : neg(x);
+        x = F == P_I ? neg(y) : y;
         y = t;
     } else {
         const R r = x * pr - y * pi, i = x * pi + y * pr;
@@ -605,6 +615,219 @@ cudaError_t small_run(sv_state *h, const Gate1 *g, size_t count) {
     return cudaSuccess;
 }
 
+// ---------------------------------------------------------------- states in L2
+// A per-gate plan of a state that stays in L2 takes several gates per launch:
+// a thread holds the 2^S amplitudes of S chosen qubits in registers, applies
+// the run's gates and stores them back (plan_gate_runs chooses the runs).  One
+// launch per gate of such a state is bound by launches and L2 round trips, in
+// complex128 also by the FP64 pipe (two lanes per SM and clock), so the scalar
+// factors of H, SX, SY and their adjoints (powers of e^(i pi/4) and 2^(-1/2),
+// counted exactly on the host) are owed: those gates are then 4 additions per
+// pair instead of 6 to 10 operations, and a later launch pays the factors with
+// one multiplication per component.  20 qubits, 590 gates of the random family
+// in complex128: 4.00 ms with a launch per gate, 2.66 now; 236 gates in
+// complex64: 0.10 ms.
+// Few forms keep the code small (a launch starts with it uncached), and the
+// gates come as kernel parameters, so that branches and factors are uniform.
+enum RunKind : uint8_t { R_HAD, R_SX, R_SXD, R_SY, R_SYD, R_GENERAL, R_SWAP, R_NEG, R_TURN, R_PHASE };
+
+template <typename R>
+struct RunArgs {
+    uint32_t q[kRunSlots];   // the registers' qubits, ascending
+    int nops, odd, quarter;  // factor paid at the end: (1 + i)^odd i^quarter m
+    R m;
+    GateRunHead op[kRunMaxOps];
+    R u[8 * kRunMaxOps];
+};
+
+// Without their factors: H (a + b, a - b), SX (a - i b, b - i a), SY (a - b,
+// a + b) and the adjoints of the last two.
+template <int K, typename R>
+__device__ __forceinline__ void run_pair(C2<R> &a, C2<R> &b) {
+    const C2<R> x = a, y = b;
+    if constexpr (K == R_SX) {
+        a = C2<R>{x.re + y.im, x.im - y.re};
+        b = C2<R>{y.re + x.im, y.im - x.re};
+    } else if constexpr (K == R_SXD) {
+        a = C2<R>{x.re - y.im, x.im + y.re};
+        b = C2<R>{y.re - x.im, y.im + x.re};
+    } else {
+        const C2<R> s = {x.re + y.re, x.im + y.im};
+        const C2<R> d = K == R_SYD ? C2<R>{y.re - x.re, y.im - x.im} : C2<R>{x.re - y.re, x.im - y.im};
+        a = K == R_SY ? d : s;
+        b = K == R_SY ? s : d;
+    }
+}
+
+template <int K, int SLOT, int S, typename R>
+__device__ __forceinline__ void run_all(C2<R> (&x)[1 << S]) {
+#pragma unroll
+    for (int v = 0; v < (1 << S); ++v)
+        if (!(v >> SLOT & 1)) run_pair<K>(x[v], x[v | 1 << SLOT]);
+}
+
+template <int SLOT, int S, typename R>
+__device__ __forceinline__ void run_pairs(C2<R> (&x)[1 << S], const GateRunHead &op, const R *u) {
+    if constexpr (SLOT < S) {
+        const uint32_t mask = op.rmask;
+        switch (op.kind) {
+            case R_HAD: run_all<R_HAD, SLOT, S>(x); break;
+            case R_SX: run_all<R_SX, SLOT, S>(x); break;
+            case R_SXD: run_all<R_SXD, SLOT, S>(x); break;
+            case R_SY: run_all<R_SY, SLOT, S>(x); break;
+            case R_SYD: run_all<R_SYD, SLOT, S>(x); break;
+            case R_SWAP:
+#pragma unroll
+                for (int v = 0; v < (1 << S); ++v) {
+                    if (v >> SLOT & 1) continue;
+                    const int w = v | 1 << SLOT;
+                    if ((v & mask) == mask) apply2<G_SWAP>(u, x[v].re, x[v].im, x[w].re, x[w].im);
+                }
+                break;
+            default:
+#pragma unroll
+                for (int v = 0; v < (1 << S); ++v) {
+                    if (v >> SLOT & 1) continue;
+                    const int w = v | 1 << SLOT;
+                    if ((v & mask) == mask) apply2<G_GENERAL>(u, x[v].re, x[v].im, x[w].re, x[w].im);
+                }
+                break;
+        }
+    }
+}
+
+template <int F, int S, typename R>
+__device__ __forceinline__ void run_phase(C2<R> (&x)[1 << S], uint32_t mask, R pr, R pi) {
+#pragma unroll
+    for (int v = 0; v < (1 << S); ++v)
+        if ((v & mask) == mask) phase1<F>(pr, pi, x[v].re, x[v].im);
+}
+
+// The same for one mask known to the compiler: a test per register becomes a
+// predicate, and a predicated FP64 instruction takes its turn in the pipe also
+// where no lane executes it (20-qubit Fourier transform in complex128 1.78 ms, 0.96 so).
+template <uint32_t MASK, int S, typename R>
+__device__ __forceinline__ void run_phase_of(C2<R> (&x)[1 << S], R pr, R pi) {
+    if constexpr (MASK < (1u << S)) {
+#pragma unroll
+        for (uint32_t v = 0; v < (1u << S); ++v)
+            if ((v & MASK) == MASK) phase1<P_GENERAL>(pr, pi, x[v].re, x[v].im);
+    }
+}
+template <int S, typename R>
+__device__ __forceinline__ void run_phase_general(C2<R> (&x)[1 << S], uint32_t mask, R pr, R pi) {
+    switch (mask) {  // a diagonal gate has at most two qubits
+        case 0: run_phase_of<0, S>(x, pr, pi); break;
+        case 1: run_phase_of<1, S>(x, pr, pi); break;
+        case 2: run_phase_of<2, S>(x, pr, pi); break;
+        case 3: run_phase_of<3, S>(x, pr, pi); break;
+        case 4: run_phase_of<4, S>(x, pr, pi); break;
+        case 5: run_phase_of<5, S>(x, pr, pi); break;
+        case 6: run_phase_of<6, S>(x, pr, pi); break;
+        case 8: run_phase_of<8, S>(x, pr, pi); break;
+        case 9: run_phase_of<9, S>(x, pr, pi); break;
+        case 10: run_phase_of<10, S>(x, pr, pi); break;
+        default: run_phase_of<12, S>(x, pr, pi); break;
+    }
+}
+
+template <int S, typename R>
+__device__ __forceinline__ void run_gate(C2<R> (&x)[1 << S], const GateRunHead &op, const R *u) {
+    if (op.kind >= R_NEG) {
+        if (op.kind == R_NEG) run_phase<P_NEG, S>(x, op.rmask, R(0), R(0));
+        else if (op.kind == R_PHASE) run_phase_general<S>(x, op.rmask, u[0], u[1]);
+        else if (op.arg == 1) run_phase<P_I, S>(x, op.rmask, R(0), R(0));
+        else run_phase<P_MI, S>(x, op.rmask, R(0), R(0));
+        return;
+    }
+    switch (op.slot) {
+        case 0: run_pairs<0, S>(x, op, u); break;
+        case 1: run_pairs<1, S>(x, op, u); break;
+        case 2: run_pairs<2, S>(x, op, u); break;
+        default: run_pairs<3, S>(x, op, u); break;
+    }
+}
+
+template <typename R>
+struct Amp2;
+template <>
+struct Amp2<float> {
+    using T = float2;
+};
+template <>
+struct Amp2<double> {
+    using T = double2;
+};
+
+constexpr int kRunThreads = 64;  // small CTAs: even work per SM (20 qubits: 1024 CTAs, 6.7 per SM)
+
+template <typename R, int S>
+__global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *__restrict__ psi,
+                                                          const __grid_constant__ RunArgs<R> a) {
+    uint32_t i = blockIdx.x * kRunThreads + threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < S; ++k) i += i & ~((1u << a.q[k]) - 1u);  // a zero bit inserted at q[k]
+    C2<R> x[1 << S];
+    auto at = [&](int v) {
+        uint32_t j = i;
+#pragma unroll
+        for (int k = 0; k < S; ++k)
+            if (v >> k & 1) j |= 1u << a.q[k];
+        return psi + j;
+    };
+#pragma unroll
+    for (int v = 0; v < (1 << S); ++v) {
+        const auto z = *at(v);
+        x[v].re = z.x;
+        x[v].im = z.y;
+    }
+    for (int k = 0; k < a.nops; ++k)
+        if ((i & a.op[k].imask) == a.op[k].imask) run_gate<S>(x, a.op[k], a.u + 2 * a.op[k].arg);
+    if (a.odd) {
+#pragma unroll
+        for (int v = 0; v < (1 << S); ++v) {
+            const R r = x[v].re - x[v].im;
+            x[v].im = x[v].re + x[v].im;
+            x[v].re = r;
+        }
+    }
+    if (a.m != R(1)) {
+#pragma unroll
+        for (int v = 0; v < (1 << S); ++v) {
+            x[v].re *= a.m;
+            x[v].im *= a.m;
+        }
+    }
+    if (a.quarter & 1) run_phase<P_I, S>(x, 0u, R(0), R(0));
+    if (a.quarter & 2) run_phase<P_NEG, S>(x, 0u, R(0), R(0));
+#pragma unroll
+    for (int v = 0; v < (1 << S); ++v) {
+        typename Amp2<R>::T z;
+        z.x = x[v].re;
+        z.y = x[v].im;
+        *at(v) = z;
+    }
+}
+
+template <typename R, int S>
+cudaError_t gate_runs_impl(sv_state *h, const GateRuns &p) {
+    for (const GateRun &r : p.runs) {
+        RunArgs<R> a;
+        for (int k = 0; k < S; ++k) a.q[k] = uint32_t(r.q[k]);
+        a.nops = r.count;
+        std::copy_n(p.ops.begin() + long(r.first), r.count, a.op);
+        for (int k = 0; k < r.ucount; ++k) a.u[k] = R(p.u[r.ufirst + size_t(k)]);
+        a.odd = r.odd;
+        a.quarter = r.quarter;
+        a.m = R(r.m);
+        k_gate_run<R, S><<<1u << (h->n - S - 6), kRunThreads, 0, h->stream>>>(
+            static_cast<typename Amp2<R>::T *>(h->data), a);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // ---------------------------------------------------------------- set basis
 template <typename R>
 __global__ void k_set_one(C2<R> *psi, uint64_t idx) {
@@ -742,6 +965,147 @@ cudaError_t launch_small_run(sv_state *h, const Gate1 *g, size_t count) {
     // whose FP64 chains want many warps (8 qubits, 115 gates: 60 us against 86)
     if (h->dt == SV_C128) return small_run<double, 1>(h, g, count);
     return h->n < 12 ? small_run<float, 2>(h, g, count) : small_run<float, 3>(h, g, count);
+}
+
+// States of at most 64 MiB (half of L2): a gate's pass reads and writes L2.
+bool gate_runs_fit(sv_dtype dt, int n) {
+    return dt != SV_ENC2B && n > small_run_max_n(dt) && n <= (dt == SV_C64 ? 23 : 22);
+}
+
+// Runs of gates for k_gate_run.  A run's register qubits are the targets of
+// the first gates that can be applied next (at most `slots` distinct ones);
+// then every gate that commutes with all the skipped gates before it joins if
+// its target is one of them.  A diagonal gate that costs arithmetic waits for
+// a run that holds one of its qubits (on half of the registers, not of the
+// lanes) until no other gate is left; sign flips and quarter turns join at once.
+void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *out) {
+    constexpr size_t kWindow = 1024;  // gates looked at ahead of the first unplaced one
+    // Register qubits.  A small complex128 state is bound by the FP64 pipes of
+    // the few SMs that its threads fill (random circuits of depth 8: 11 qubits
+    // 73 us with two, 197 with four; 15 qubits 103 and 271), a larger one by the
+    // passes over L2 (22 qubits 4.70 ms with two, 4.48 with four); complex64 15
+    // qubits 45 us with three and 51 with four, 23 qubits 619 and 555.
+    const int slots = dt == SV_C128 ? (n <= 18 ? 2 : 4) : (n <= 17 ? 3 : 4);
+    out->slots = slots;
+    std::vector<char> placed(g.size(), 0);
+    std::vector<char> phase(g.size());
+    std::vector<GateRunHead> base(g.size());
+    auto factors = [&](size_t i, double u[8]) {
+        for (int k = 0; k < 4; ++k) {
+            u[2 * k] = g[i].u[k].re;
+            u[2 * k + 1] = g[i].u[k].im;
+        }
+    };
+    for (size_t i = 0; i < g.size(); ++i) {
+        phase[i] = is_phase(g[i]);
+        GateRunHead &o = base[i];
+        o = GateRunHead{};
+        double u[8];
+        factors(i, u);
+        const int pf = phase_form(u);
+        if (phase[i]) {
+            o.kind = pf == P_GENERAL ? R_PHASE : pf == P_NEG ? R_NEG : R_TURN;
+            o.arg = pf == P_I ? 1 : 3;
+            continue;
+        }
+        const int form = gate_form(u);
+        o.kind = form == G_SWAP ? R_SWAP : R_GENERAL;
+        if (g[i].control >= 0) continue;
+        switch (form) {
+            case G_HAD: o.kind = u[0] == std::sqrt(0.5) ? R_HAD : R_GENERAL; break;
+            case G_SX: o.kind = R_SX; break;
+            case G_SXD: o.kind = R_SXD; break;
+            case G_SY: o.kind = R_SY; break;
+            case G_SYD: o.kind = R_SYD; break;
+            default: break;
+        }
+    }
+    int eighths = 0, halves = 0;  // factor owed: e^(i pi eighths / 4) 2^(-halves / 2)
+    size_t start = 0;
+    while (true) {
+        while (start < g.size() && placed[start]) ++start;
+        if (start == g.size()) break;
+        const size_t end = std::min(g.size(), start + kWindow);
+        uint64_t qs = 0, wish = 0;  // register qubits; qubits of waiting diagonal gates
+        GateRun r;
+        r.first = out->ops.size();
+        r.ufirst = out->u.size();
+        for (int round = 0; round < 2; ++round) {  // 0: choose the qubits, 1: take the gates
+            uint64_t diag = 0, any = 0;            // qubits on which a skipped gate is diagonal / is not
+            const bool only_phases = qs == 0;      // (of round 1)
+            if (round == 1) {
+                for (uint64_t from : {wish, (uint64_t(1) << n) - 1})
+                    for (int q = n - 1; q >= 0; --q)
+                        if (__builtin_popcountll(qs) < slots && (from >> q & 1)) qs |= uint64_t(1) << q;
+                for (int q = 0, k = 0; q < n; ++q)
+                    if (qs >> q & 1) r.q[k++] = q;
+            }
+            for (size_t i = start; i < end && r.count < kRunMaxOps; ++i) {
+                if (placed[i]) continue;
+                const uint64_t t = uint64_t(1) << g[i].target;
+                const uint64_t c = g[i].control < 0 ? 0 : uint64_t(1) << g[i].control;
+                bool take = phase[i] ? !((t | c) & any) : !(t & (diag | any)) && !(c & any);
+                if (take && round == 0) {
+                    if (phase[i]) {
+                        if (base[i].kind == R_PHASE) wish |= t;
+                    } else if (!(qs & t) && __builtin_popcountll(qs) == slots) {
+                        take = false;
+                    } else {
+                        qs |= t;
+                    }
+                } else if (take) {
+                    take = phase[i] ? only_phases || base[i].kind != R_PHASE || ((t | c) & qs) : (qs & t) != 0;
+                }
+                if (!take) {
+                    (phase[i] ? diag : any) |= t;
+                    diag |= c;
+                    continue;
+                }
+                if (round == 0) continue;
+                placed[i] = 1;
+                ++r.count;
+                out->ops.push_back(base[i]);
+                GateRunHead &o = out->ops.back();
+                const uint64_t cond = phase[i] ? t | c : c;
+                for (int k = 0; k < slots; ++k) {
+                    if (cond >> r.q[k] & 1) o.rmask |= uint8_t(1u << k);
+                    if (r.q[k] == g[i].target) o.slot = uint8_t(k);
+                }
+                o.imask = uint32_t(cond & ~qs);
+                if (o.kind <= R_SYD) {  // SX, SY: e^(i pi/4) 2^(-1/2), H: 2^(-1/2)
+                    ++halves;
+                    eighths += o.kind == R_SX || o.kind == R_SY ? 1 : o.kind == R_SXD || o.kind == R_SYD ? -1 : 0;
+                } else if (o.kind == R_GENERAL || o.kind == R_PHASE) {
+                    double u[8];
+                    factors(i, u);
+                    const double *from = o.kind == R_GENERAL ? u : u + 6;
+                    const size_t len = o.kind == R_GENERAL ? 8 : 2;
+                    size_t at = r.ufirst;  // the same factors again (the T gates of a run) share their place
+                    while (at < out->u.size() && (at + len > out->u.size() || !std::equal(from, from + len, &out->u[at])))
+                        at += 2;
+                    if (at == out->u.size()) out->u.insert(out->u.end(), from, from + len);
+                    o.arg = uint8_t((at - r.ufirst) / 2);
+                }
+            }
+        }
+        r.ucount = int(out->u.size() - r.ufirst);
+        // the factor, once it exceeds 2^-12 or at the end
+        while (start < g.size() && placed[start]) ++start;
+        if (halves >= 24 || start == g.size()) {
+            const int k = eighths & 7;
+            r.odd = k & 1;
+            r.quarter = k >> 1;
+            halves += r.odd;  // e^(i pi / 4) = (1 + i) 2^(-1/2)
+            r.m = std::ldexp(halves & 1 ? std::sqrt(0.5) : 1.0, -(halves >> 1));
+            eighths = halves = 0;
+        }
+        out->runs.push_back(r);
+    }
+}
+
+cudaError_t launch_gate_runs(sv_state *h, const GateRuns &p) {
+    if (h->dt == SV_C128) return p.slots == 2 ? gate_runs_impl<double, 2>(h, p) : gate_runs_impl<double, 4>(h, p);
+    return p.slots == 3 ? gate_runs_impl<float, 3>(h, p) : gate_runs_impl<float, 4>(h, p);
 }
 
 cudaError_t launch_set_basis(sv_state *h, uint64_t idx) {

@@ -320,6 +320,7 @@ sv_status create_plan(sv_state *h, const char *text, const Circuit &c, const Str
                 p->launches.push_back(PlanLaunch{0, int(i), b});
                 p->bytes += b;
             }
+        if (!s && gate_runs_fit(h->dt, h->n) && p->launches.size() >= 2) plan_gate_runs(h->dt, h->n, p->pergate, &p->gruns);
     } else {
         s = build_tile_plan(h, c, p, st.cfg, st.pass_ctas);
         if (!s && !key.empty()) {
@@ -646,15 +647,16 @@ namespace sv {
 namespace {
 
 // A plan of two or more per-gate updates of a state of 2 to
-// small_run_max_n qubits runs in few launches (k_small_run); its launch list keeps one entry per gate, which is
-// what sv_plan_execute_timed and the statistics show.
+// small_run_max_n qubits runs in few launches (k_small_run), and so does one
+// of a larger state that stays in L2 (k_gate_run); its launch list keeps one
+// entry per gate, which is what sv_plan_execute_timed and the statistics show.
 bool small_plan(const sv_plan_s *p) {
     return p->h->n >= 2 && p->h->n <= small_run_max_n(p->h->dt) && p->launches.size() >= 2 &&
            p->launches.size() == p->pergate.size();
 }
 
 sv_status execute_direct(sv_plan_s *p) {
-    if (small_plan(p)) return check_launch(launch_small_run(p->h, p->pergate.data(), p->pergate.size()), "sv_plan_execute");
+    if (small_plan(p) || !p->gruns.runs.empty()) return check_launch(plan_launch_all(p), "sv_plan_execute");
     for (const PlanLaunch &l : p->launches) {
         sv_status s = check_launch(launch_one(p, l), "sv_plan_execute");
         if (s) return s;
@@ -667,6 +669,7 @@ sv_status execute_direct(sv_plan_s *p) {
 extern "C++" {
 cudaError_t plan_launch_all(sv_plan_s *p) {
     if (small_plan(p)) return launch_small_run(p->h, p->pergate.data(), p->pergate.size());
+    if (!p->gruns.runs.empty()) return launch_gate_runs(p->h, p->gruns);
     for (const PlanLaunch &l : p->launches) {
         const cudaError_t e = launch_one(p, l);
         if (e != cudaSuccess) return e;

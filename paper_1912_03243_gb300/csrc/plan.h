@@ -59,6 +59,7 @@ struct sv_plan_s {
     int mode = 0;
     int64_t gates = 0;                     // gates of the circuit text
     std::vector<sv::Gate1> pergate;        // per-gate updates
+    sv::GateRuns gruns;                    // the same in runs (states that stay in L2)
     struct EncRun {
         int first, count;                  // ops d_encops[first .. first + count)
         int nbits, pos[sv::kEncRunMaxBits];  // block-index bits of its tiles

@@ -118,6 +118,32 @@ cudaError_t launch_gate1(sv_state *h, const Gate1 &g);
 // one launch per about a hundred gates, the state in one CTA's shared memory.
 int small_run_max_n(sv_dtype dt);
 cudaError_t launch_small_run(sv_state *h, const Gate1 *g, size_t count);
+// Runs of gates on a state of more qubits than that which stays in L2, one
+// launch per run (k_gate_run): the run's gates and its registers' qubits.
+constexpr int kRunSlots = 4;    // most register qubits
+constexpr int kRunMaxOps = 48;  // gates per run: under 4 KB of kernel parameters
+struct GateRunHead {
+    uint8_t kind, slot;  // (RunKind; register slot of the target)
+    uint8_t rmask;       // register-index bits that must be 1
+    uint8_t arg;         // R_TURN: the power of i; else the place of its factors, in pairs
+    uint32_t imask;      // other amplitude-index bits that must be 1
+};
+struct GateRun {
+    int q[kRunSlots];             // ascending
+    size_t first = 0, ufirst = 0;  // ops[first .. first + count), factors u[ufirst .. ufirst + ucount)
+    int count = 0, ucount = 0;
+    int odd = 0, quarter = 0;     // factor paid after them: (1 + i)^odd i^quarter m
+    double m = 1.0;
+};
+struct GateRuns {
+    int slots = 0;
+    std::vector<GateRun> runs;
+    std::vector<GateRunHead> ops;
+    std::vector<double> u;
+};
+bool gate_runs_fit(sv_dtype dt, int n);
+void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *out);
+cudaError_t launch_gate_runs(sv_state *h, const GateRuns &p);
 cudaError_t launch_set_basis(sv_state *h, uint64_t idx);
 cudaError_t launch_norm(sv_state *h, double *d_out);  // d_out: device double
 cudaError_t launch_gather(sv_state *h, const uint64_t *d_idx, size_t m, double *d_out);

@@ -133,6 +133,31 @@ def test_small_states_run(S, orc, dtype, n):
         p.free()
 
 
+@pytest.mark.parametrize("dtype,n", [("c64", 15), ("c64", 18), ("c64", 23), ("c64", 24), ("c128", 11), ("c128", 12), ("c128", 17),
+                                     ("c128", 22), ("c128", 23)])
+def test_runs_of_gates(S, orc, dtype, n):
+    """Plans of states that stay in L2 run several gates per launch, from the
+    smallest to the largest such state and one qubit beyond: mixed circuits
+    (controlled and dense gates among them), the random family (complex128 owes
+    its scalar factors), a QFT and diagonal gates alone, direct and as a graph
+    replay, against the oracle."""
+    diag = C.Circuit(n)
+    for q in range(n):
+        diag.add("T", q)
+        diag.add("CZ" if q else "S", *((q, q - 1) if q else (q,)))
+    full = [C.random_unitary_gates(n, 300, n), C.random_circuit(n, 12, 3), C.qft_circuit(n, 1), diag]
+    for c in full if n <= 18 else [C.random_unitary_gates(n, 60, n), C.random_circuit(n, 3, 3)]:
+        psi0 = C.random_state(n, 90 + n)
+        ref = orc.run(c, psi=psi0)
+        s = S.StateVector(n, dtype)
+        p = s.plan(c, "pergate")
+        for _ in range(3):  # direct, capture, replay
+            s.from_numpy(psi0)
+            p.execute()
+            check(dtype, s.to_numpy(), ref)
+        p.free()
+
+
 @pytest.mark.parametrize("dtype", ["c64", "c128"])
 @pytest.mark.parametrize("seed", [1, 2, 3])
 def test_random_circuit_20q(S, orc, dtype, seed):
