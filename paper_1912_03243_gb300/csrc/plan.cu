@@ -182,7 +182,7 @@ sv_status build_tile_plan(sv_state *h, const Circuit &c, sv_plan_s *p, const Til
         return s ? s : upload_tile_plan(p, tp);
     }
     TilePlan<double> tp;
-    sv_status s = plan_tiles<double>(c, h->n, tile_config128(), &tp);
+    sv_status s = plan_tiles<double>(c, h->n, cfg, &tp);
     return s ? s : upload_tile_plan(p, tp);
 }
 
@@ -207,7 +207,7 @@ const char *launch_name(const sv_plan_s *p, const PlanLaunch &l) {
     if (l.kind == 2) return tc_kernel_name(p->tcargs[size_t(l.index)]);
     if (l.kind == 3) return p->h->dt == SV_C64 ? "k_fused_dense<f32>" : "k_fused_dense<f64>";
     if (l.kind == 4) return "k_enc_run_in";
-    return tile_kernel_name(p->h);
+    return tile_kernel_name(p->h->dt, p->cfg);
 }
 
 }  // namespace
@@ -270,12 +270,15 @@ std::string pass_ctas_key(const std::vector<int> &pc) {
     return k;
 }
 
-TileConfig default_config(const sv_state *h) { return h->dt == SV_C64 ? tile_config64() : tile_config128(); }
+TileConfig default_config(const sv_state *h) { return tile_config_for(h->dt, h->n); }
 
 // Build the plan of one strategy for the handle (text already parsed into c).
 sv_status create_plan(sv_state *h, const char *text, const Circuit &c, const Strategy &st, sv_plan_s **out) {
     *out = nullptr;
-    const int tile_m = st.mode == SV_MODE_TILED ? st.cfg.m : (h->dt == SV_C64 ? kTileM64 : kTileM128);
+    // smaller states than one full tile run gate by gate (also with a smaller tile)
+    const int tile_m = st.mode == SV_MODE_TILED && st.cfg.c64 && st.cfg.m == tile_m64() ? st.cfg.m
+                       : h->dt == SV_C64                                               ? kTileM64
+                                                                                       : kTileM128;
     const bool tiled = st.mode == SV_MODE_TILED && h->n >= tile_m;
     std::string key;
     if (tiled && text) {
@@ -286,6 +289,7 @@ sv_status create_plan(sv_state *h, const char *text, const Circuit &c, const Str
             sv_plan_s *p = new sv_plan_s;
             p->h = h;
             p->mode = st.mode;
+            p->cfg = st.cfg;
             p->gates = it->second.gates;
             p->tfns = it->second.fns;
             p->tile_rb = it->second.rb;
@@ -306,6 +310,7 @@ sv_status create_plan(sv_state *h, const char *text, const Circuit &c, const Str
     sv_plan_s *p = new sv_plan_s;
     p->h = h;
     p->mode = st.mode;
+    p->cfg = st.cfg;
     p->gates = int64_t(c.instrs.size());
     sv_status s = SV_OK;
     if (st.mode == SV_MODE_FUSED) {
@@ -356,16 +361,17 @@ std::vector<Strategy> candidates(const sv_state *h) {
         return v;
     }
     if (h->n >= tile_m) {
+        v.push_back(Strategy{SV_MODE_TILED, default_config(h), 0});
         if (h->dt == SV_C64) {
             // the generator's configurations: register bits, CTAs per SM,
             // direct HBM I/O, prefetching, tile bits
             const int opts[][5] = {{5, 2, 1, 0, 13}, {5, 2, 1, 1, 13}, {5, 2, 0, 0, 13},
                                    {4, 2, 1, 0, 13}, {5, 3, 1, 0, 13}, {5, 4, 1, 0, 12}};
             for (const auto &o : opts)
-                if (h->n >= o[4])
-                    v.push_back(Strategy{SV_MODE_TILED, tile_config64(o[0], o[1], o[2], o[3], o[4]), 0});
-        } else {
-            v.push_back(Strategy{SV_MODE_TILED, tile_config128(), 0});
+                if (h->n >= o[4]) {
+                    const Strategy c{SV_MODE_TILED, tile_config64(o[0], o[1], o[2], o[3], o[4]), 0};
+                    if (c.name() != v[0].name()) v.push_back(c);
+                }
         }
     } else {
         v.push_back(Strategy{SV_MODE_PERGATE, TileConfig{}, 0});
@@ -826,7 +832,7 @@ sv_status sv_plan_stats(const char *text, int n, sv_dtype dt, int compile, int64
             return SV_ERR_UNSUPPORTED;
         }
         TilePlan<float> tp;
-        s = plan_tiles<float>(c, n, tile_config64(), &tp);
+        s = plan_tiles<float>(c, n, tile_config_for(dt, n), &tp);
         return s ? s : count(tp);
     }
     if (n < kTileM128) {
@@ -834,7 +840,7 @@ sv_status sv_plan_stats(const char *text, int n, sv_dtype dt, int compile, int64
         return SV_ERR_UNSUPPORTED;
     }
     TilePlan<double> tp;
-    s = plan_tiles<double>(c, n, tile_config128(), &tp);
+    s = plan_tiles<double>(c, n, tile_config_for(dt, n), &tp);
     return s ? s : count(tp);
 }
 
@@ -878,7 +884,7 @@ sv_status sv_plan_pass_source(const char *text, int n, sv_dtype dt, int64_t pass
             return SV_ERR_UNSUPPORTED;
         }
         TilePlan<float> tp;
-        s = plan_tiles<float>(c, n, tile_config64(), &tp);
+        s = plan_tiles<float>(c, n, tile_config_for(dt, n), &tp);
         return s ? s : emit(tp);
     }
     if (n < kTileM128) {
@@ -886,7 +892,7 @@ sv_status sv_plan_pass_source(const char *text, int n, sv_dtype dt, int64_t pass
         return SV_ERR_UNSUPPORTED;
     }
     TilePlan<double> tp;
-    s = plan_tiles<double>(c, n, tile_config128(), &tp);
+    s = plan_tiles<double>(c, n, tile_config_for(dt, n), &tp);
     return s ? s : emit(tp);
 }
 

@@ -67,6 +67,7 @@ struct sv_plan_s {
     std::vector<EncRun> encruns;           // two-byte code: runs of gates, one pass each
     sv::EncRunOp *d_encops = nullptr;      // their ops (device)
     std::vector<void *> tfns;              // compiled tile passes
+    sv::TileConfig cfg{};                  // of the compiled passes
     int tile_rb = 0;                       // their register bits per thread
     std::vector<double> tile_lane_ops;     // their FP32 lane operations per amplitude
     std::vector<int> tile_nseg;            // their register segments

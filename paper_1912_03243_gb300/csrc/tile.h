@@ -173,6 +173,8 @@ TileConfig tile_config64(int rb = 0, int ctas = 0, int direct = -1, int prefetch
 // Tile bits of complex64 passes (SV_TILE_M overrides: 12 or 13).
 int tile_m64();
 TileConfig tile_config128();
+// The tiled mode's configuration for a state of n qubits.
+TileConfig tile_config_for(sv_dtype dt, int n);
 // Folder of the compiled-pass disk cache ("" when there is none).
 std::string jit_cache_dir();
 // A short text naming a configuration (plan keys, tuning reports).
@@ -198,7 +200,7 @@ struct RemapTiles {
     unsigned rot = 0;
 };
 cudaError_t launch_jit_remap(void *fn, int rb, const RemapTiles &t, uint64_t param, cudaStream_t st);
-const char *tile_kernel_name(const sv_state *h);
+const char *tile_kernel_name(sv_dtype dt, const TileConfig &cfg);
 // The code-generation switches (environment) that shape a compiled pass, as
 // part of a plan-cache key.
 std::string tile_codegen_key();

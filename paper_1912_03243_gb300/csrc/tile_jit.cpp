@@ -40,6 +40,7 @@
 #include <iterator>
 #include <map>
 #include <mutex>
+#include <set>
 #include <sstream>
 #include <string>
 #include <thread>
@@ -162,6 +163,8 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
              "__device__ __forceinline__ u64 sub2(u64 a, u64 b) { u64 d; asm(\"sub.rn.f32x2 %0, %1, %2;\" : \"=l\"(d) : \"l\"(a), \"l\"(b)); return d; }\n"
              "__device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) { u64 d; asm(\"fma.rn.f32x2 %0, %1, %2, %3;\" : \"=l\"(d) : \"l\"(a), \"l\"(b), \"l\"(c)); return d; }\n";
     }
+    if (sizeof(R) == 8)
+        o << "__device__ __forceinline__ double flip(double x, u32 s) { return __hiloint2double(__double2hiint(x) ^ (int)s, __double2loint(x)); }\n";
     o << "__device__ __forceinline__ void cpa16(void* s, const void* g) {\n"
          "  u32 sa = (u32)__cvta_generic_to_shared(s);\n"
          "  asm volatile(\"cp.async.cg.shared.global [%0], [%1], 16;\\n\" :: \"r\"(sa), \"l\"(g) : \"memory\");\n}\n";
@@ -364,6 +367,20 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
     };
     const bool packed = sizeof(R) == 4 && packed_adds_enabled();
     auto reg = [](const char *a, int v) { return std::string(a) + "[" + std::to_string(v) + "]"; };
+    // -x by itself (not an operand of an addition): complex128 flips the sign
+    // bit, which the FP64 pipe has no part in
+    auto neg = [](const std::string &x) { return sizeof(R) == 8 ? "flip(" + x + ", 0x80000000u)" : "-" + x; };
+    std::map<std::vector<int>, std::string> mask_name;
+    auto sign_mask = [&](const std::vector<int> &set) -> std::string {  // the sign bit of prod(set)
+        auto it = mask_name.find(set);
+        if (it != mask_name.end()) return it->second;
+        const std::string nm = "sb" + std::to_string(mask_name.size()) + "_" + std::to_string(cur_seg);
+        o << "  const u32 " << nm << " = ";
+        for (size_t i = 0; i < set.size(); ++i) o << (i ? " ^ " : "") << "(c" << set[i] << " ? 0x80000000u : 0u)";
+        o << ";\n";
+        mask_name.emplace(set, nm);
+        return nm;
+    };
     auto materialise = [&](int v) {
         if (!rph[v].empty()) {
             std::string f;  // real factor ("" for 1)
@@ -386,6 +403,11 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
             const std::string x = reg("xr", v), y = reg("xi", v);
             o << "  { const " << RT << " r = " << x << " * " << k.first << " - " << y << " * " << k.second << "; " << y
               << " = " << x << " * " << k.second << " + " << y << " * " << k.first << "; " << x << " = r; }\n";
+        } else if (!rsg[v].empty() && sizeof(R) == 8 && me[v] == 0) {
+            // signs alone: flips of the sign bits, no FP64 operations
+            const std::string f = sign_mask(rsg[v]) + (sgn[v] < 0 ? " ^ 0x80000000u" : "");
+            o << "  " << reg("xr", v) << " = flip(" << reg("xr", v) << ", " << f << "); " << reg("xi", v) << " = flip("
+              << reg("xi", v) << ", " << f << ");\n";
         } else if (!rsg[v].empty()) {
             const std::string f = scaled(prod(rsg[v]), -me[v]);
             const char *neg = sgn[v] < 0 ? "-" : "";
@@ -394,7 +416,8 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
             const std::string f = lit(R(sgn[v] * mag(-me[v])));
             o << "  " << reg("xr", v) << " *= " << f << "; " << reg("xi", v) << " *= " << f << ";\n";
         } else if (sgn[v] < 0) {
-            o << "  " << reg("xr", v) << " = -" << reg("xr", v) << "; " << reg("xi", v) << " = -" << reg("xi", v) << ";\n";
+            o << "  " << reg("xr", v) << " = " << neg(reg("xr", v)) << "; " << reg("xi", v) << " = " << neg(reg("xi", v))
+              << ";\n";
         }
         rsg[v].clear();
         rph[v].clear();
@@ -404,12 +427,13 @@ std::string gen_pass(const TilePlan<R> &tp, size_t pass) {
     auto scatter = [&]() {
         for (int v = 0; v < G.NR; ++v) {
             if (!rsg[v].empty() || !rph[v].empty() || me[v] != 0) materialise(v);
-            const char *neg = sgn[v] < 0 ? "-" : "";
-            o << "  sm[pj ^ " << pv[v] << "u] = make_" << C2T << "(" << neg << "xr[" << v << "], " << neg << "xi[" << v
-              << "]);\n";
+            const std::string x = reg("xr", v), y = reg("xi", v);
+            o << "  sm[pj ^ " << pv[v] << "u] = make_" << C2T << "(" << (sgn[v] < 0 ? neg(x) : x) << ", "
+              << (sgn[v] < 0 ? neg(y) : y) << ");\n";
             sgn[v] = 1;
         }
         prod_name.clear();
+        mask_name.clear();
         scaled_name.clear();
         cph.clear();
         kph.clear();
@@ -1117,6 +1141,40 @@ TileConfig tile_config128() {
     return c;
 }
 
+// Tiles of a state of n qubits.  A pass of few tiles takes as long as one CTA
+// takes for its tile, so a small state is cut into about 128 tiles, one per SM:
+// complex64 down to 2^11 amplitudes (random circuits of depth 12: 14 qubits
+// 20.8 -> 10.5 us, 17 qubits 26.9 -> 12.6, 19 qubits 30.9 -> 18.8), complex128,
+// bound by each SM's FP64 pipe, down to 2^9 (12 qubits 310 -> 49 us, 17 qubits
+// 443 -> 121, 18 qubits 474 -> 246).  Fewer register bits keep the threads of a
+// CTA.  Three waves and less of full complex64 tiles (21 and 22 qubits) leave
+// the last one part empty: there 2^11 amplitudes, 16 per thread (53.5 -> 47.4
+// and 92.5 -> 80.0 us); from 23 qubits on their additional passes cost more
+// (25-qubit Fourier transform 395 -> 567 us).
+TileConfig tile_config_for(sv_dtype dt, int n) {
+    const int m = n - 7;  // 2^7 tiles
+    if (dt != SV_C64) {
+        TileConfig c = tile_config128();
+        if (m < c.m) {
+            c.m = std::max(m, 9);
+            c.rb = c.m - 7;
+            c.ctas = 4;
+        }
+        return c;
+    }
+    TileConfig c = tile_config64();
+    if (std::getenv("SV_TILE_M") || std::getenv("SV_TILE_RB") || std::getenv("SV_TILE_CTAS")) return c;
+    if (m < c.m) {
+        c.m = std::max(m, 11);
+        c.rb = c.m - 8;
+        c.ctas = c.m == 12 ? 3 : 4;
+    } else if (n == 21 || n == 22) {
+        c.m = 11;
+        c.rb = 4;
+    }
+    return c;
+}
+
 std::string tile_config_name(const TileConfig &cfg) {
     return "m=" + std::to_string(cfg.m) + ",rb=" + std::to_string(cfg.rb) + ",low=" + std::to_string(cfg.low) +
            ",ctas=" + std::to_string(cfg.ctas) + ",direct=" + std::to_string(int(cfg.direct)) +
@@ -1137,9 +1195,12 @@ sv_status jit_tile_plan(const TilePlan<double> &tp, std::vector<void *> *fns) { 
 sv_status jit_compile_check(const TilePlan<float> &tp) { return compile_check_impl(tp); }
 sv_status jit_compile_check(const TilePlan<double> &tp) { return compile_check_impl(tp); }
 
-const char *tile_kernel_name(const sv_state *h) {
-    static const char *n64[] = {"svp<f32,13,4>", "svp<f32,13,5>", "svp<f32,13,6>"};
-    return h->dt == SV_C64 ? n64[tile_rb64() - 4] : "svp<f64,12,4>";
+const char *tile_kernel_name(sv_dtype dt, const TileConfig &cfg) {
+    static std::mutex mu;
+    static std::set<std::string> names;  // (its strings stay where they are)
+    std::lock_guard<std::mutex> lock(mu);
+    return names.insert(std::string(dt == SV_C64 ? "svp<f32," : "svp<f64,") + std::to_string(cfg.m) + "," +
+                        std::to_string(cfg.rb) + ">").first->c_str();
 }
 
 cudaError_t launch_jit_remap(void *fn, int rb, const RemapTiles &r, uint64_t param, cudaStream_t st) {

@@ -70,6 +70,29 @@ def test_every_gate_kind(S, orc, dtype, n, seed):
     check(dtype, s.to_numpy(), ref)
 
 
+@pytest.mark.parametrize("dtype,n", [("c64", 13), ("c64", 17), ("c64", 18), ("c64", 19), ("c64", 20), ("c64", 21), ("c64", 22),
+                                     ("c128", 12), ("c128", 15), ("c128", 16), ("c128", 17), ("c128", 18), ("c128", 19)])
+def test_small_tiles(S, orc, dtype, n):
+    """States of up to 22 qubits take smaller tiles, by size: each choice on
+    both sides of its borders, with every gate kind, the random family
+    (eighth turns and signs on qubits outside a tile) and a QFT, on a state
+    alone and as the member of a batch."""
+    for c in (C.random_unitary_gates(n, 150, n), C.random_circuit(n, 6, 2), C.qft_circuit(n, 1)):
+        psi0 = C.random_state(n, 300 + n)
+        ref = orc.run(c, psi=psi0)
+        s, t = S.StateVector(n, dtype), S.StateVector(n, dtype)
+        p, b = s.plan(c, "tiled"), S.Batch([t], [c])
+        for _ in range(2):
+            s.from_numpy(psi0)
+            t.from_numpy(psi0)
+            p.execute()
+            b.execute()
+            check(dtype, s.to_numpy(), ref)
+            check(dtype, t.to_numpy(), ref)
+        p.free()
+        b.free()
+
+
 @pytest.mark.parametrize("dtype", ["c64", "c128"])
 def test_ghz_qft_uniform(S, orc, dtype):
     n = 18
