@@ -27,6 +27,7 @@
 struct sv_batch_s {
     std::vector<sv_handle> handles;
     std::vector<sv_plan> plans;
+    std::vector<size_t> order;             // members, the longest first
     std::vector<cudaStream_t> branch;      // one private stream per member (capture branches)
     std::vector<cudaStream_t> user;        // the distinct streams of the member handles
     std::vector<cudaEvent_t> ev;           // fork, joins, user-side events
@@ -52,6 +53,17 @@ void destroy_batch(sv_batch_s *b) {
     delete b;
 }
 
+// Tiles of a batch's member.  Members run side by side, so a pass of few tiles
+// need not fill the chip by itself, as tile_config_for has it do: from 17 to 22
+// qubits whole 2^13 tiles (the fewest passes) with 16 amplitudes per thread,
+// whose CTAs of 512 threads finish their tile sooner (64 members of 13 to 22
+// qubits: 1.87 ms with 32 amplitudes per thread, 1.58 with the tiles of a
+// member run alone, 1.34 so; 8 to 16 qubits: 0.121 ms with those of a member
+// run alone, 0.135 with whole tiles).
+TileConfig member_config(const sv_state *h) {
+    return h->dt == SV_C64 && h->n >= 17 && h->n <= 22 ? tile_config64(4) : tile_config_for(h->dt, h->n);
+}
+
 // Run every member's launches on its branch stream, forked from and joined
 // to the main stream (direct launches, or recorded into the graph being
 // captured on the main stream).
@@ -59,7 +71,8 @@ cudaError_t launch_members(sv_batch_s *b) {
     const size_t n = b->plans.size();
     cudaEvent_t fork = b->ev[0];
     cudaError_t e = cudaEventRecord(fork, b->main);
-    for (size_t k = 0; k < n && e == cudaSuccess; ++k) {
+    for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+        const size_t k = b->order[i];
         sv_plan_s *p = b->plans[k];
         e = cudaStreamWaitEvent(b->branch[k], fork, 0);
         if (e != cudaSuccess) break;
@@ -127,7 +140,8 @@ extern "C" sv_status sv_batch_create(const sv_handle *handles, const char *const
     sv_status s = SV_OK;
     for (int k = 0; k < count && s == SV_OK; ++k) {
         sv_plan p = nullptr;
-        s = sv_plan_create(handles[k], texts[k], SV_MODE_TILED, &p);
+        const TileConfig cfg = member_config(handles[k]);
+        s = plan_create(handles[k], texts[k], SV_MODE_TILED, &cfg, &p);
         if (s) break;
         b->handles.push_back(handles[k]);
         b->plans.push_back(p);
@@ -143,9 +157,22 @@ extern "C" sv_status sv_batch_create(const sv_handle *handles, const char *const
             b->user.push_back(handles[k]->stream);
     }
     cudaError_t e = s == SV_OK ? cudaStreamCreateWithFlags(&b->main, cudaStreamNonBlocking) : cudaSuccess;
+    // A batch ends with its longest chain: members are launched longest first,
+    // and a branch's priority falls by a step for every halving of its
+    // member's traffic, so that the long chains' CTAs are not queued behind the
+    // short ones'.
+    double most = 0.0;
+    for (sv_plan p : b->plans) most = std::max(most, p->bytes);
+    for (size_t k = 0; k < b->plans.size(); ++k) b->order.push_back(k);
+    std::stable_sort(b->order.begin(), b->order.end(),
+                     [&](size_t x, size_t y) { return b->plans[x]->bytes > b->plans[y]->bytes; });
+    int least = 0, greatest = 0;
+    if (s == SV_OK && e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
     for (int k = 0; k < count && s == SV_OK && e == cudaSuccess; ++k) {
         cudaStream_t st = nullptr;
-        e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        int prio = greatest;
+        for (double bytes = 2.0 * b->plans[size_t(k)]->bytes; prio < least && bytes <= most; bytes *= 2.0) ++prio;
+        e = cudaStreamCreateWithPriority(&st, cudaStreamNonBlocking, prio);
         b->branch.push_back(st);
     }
     // events: the fork, one join per member, one per distinct user stream

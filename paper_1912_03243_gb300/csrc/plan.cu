@@ -599,6 +599,10 @@ sv_status create_auto_plan(sv_state *h, const char *text, const Circuit &c, sv_p
 }  // namespace sv
 
 sv_status sv_plan_create(sv_handle h, const char *text, int mode, sv_plan *out) {
+    return sv::plan_create(h, text, mode, nullptr, out);
+}
+
+extern "C++" sv_status sv::plan_create(sv_handle h, const char *text, int mode, const TileConfig *cfg, sv_plan *out) {
     if (!out) {
         set_error("out is NULL");
         return SV_ERR_ARG;
@@ -623,7 +627,7 @@ sv_status sv_plan_create(sv_handle h, const char *text, int mode, sv_plan *out) 
     Circuit c;
     sv_status s = SV_OK;
     // a cached tiled plan needs no parse (the text is part of its key)
-    const Strategy st{mode, default_config(h), 0};
+    const Strategy st{mode, cfg ? *cfg : default_config(h), 0};
     const bool maybe_cached = mode == SV_MODE_TILED;
     if (!maybe_cached) {
         s = parse_circuit(text, h->n, &c);

@@ -90,6 +90,8 @@ struct sv_plan_s {
 };
 
 namespace sv {
+// sv_plan_create with a tile configuration (null: the mode's own for the state).
+sv_status plan_create(sv_handle h, const char *text, int mode, const TileConfig *cfg, sv_plan *out);
 // Every launch of a plan, in order, on the stream of its handle (no graph).
 cudaError_t plan_launch_all(sv_plan_s *p);
 // Whether a plan's launches can be captured into a CUDA graph (no host-side
