@@ -435,9 +435,9 @@ cudaError_t gate1_impl(sv_state *h, const Gate1 &g) {
 // kernel parameter, so a launch needs no device memory of its own.
 template <typename R>
 struct SmallOp {
-    uint8_t code;    // pair updates: GateForm * 3 + slot; 24 + PhaseForm; a stage header: number of its gates
+    uint8_t code;    // pair updates: GateForm * 2 + slot; 16 + PhaseForm; a stage header: number of its gates
     uint8_t rmask;   // register-index bits that must be 1
-    uint8_t s[2];    // stage header: its first two qubits (the third in imask)
+    uint8_t s[2];    // stage header: its qubits
     uint32_t imask;  // other amplitude-index bits that must be 1
     R u[8];
 };
@@ -477,9 +477,8 @@ __device__ __forceinline__ void small_phase(C2<R> (&x)[1 << S], const SmallOp<R>
 template <int S, typename R>
 __device__ __forceinline__ void small_gate(C2<R> (&x)[1 << S], const SmallOp<R> &op) {
 #define SV_SMALL_FORM(F)                                        \
-    case 3 * F: small_pairs<F, 0, S>(x, op); break;             \
-    case 3 * F + 1: small_pairs<F, 1, S>(x, op); break;         \
-    case 3 * F + 2: small_pairs<F, 2, S>(x, op); break;
+    case 2 * F: small_pairs<F, 0, S>(x, op); break;             \
+    case 2 * F + 1: small_pairs<F, 1, S>(x, op); break;
     switch (op.code) {
         SV_SMALL_FORM(G_GENERAL)
         SV_SMALL_FORM(G_REAL)
@@ -489,9 +488,9 @@ __device__ __forceinline__ void small_gate(C2<R> (&x)[1 << S], const SmallOp<R> 
         SV_SMALL_FORM(G_SY)
         SV_SMALL_FORM(G_SYD)
         SV_SMALL_FORM(G_SWAP)
-        case 24 + P_NEG: small_phase<P_NEG, S>(x, op); break;
-        case 24 + P_I: small_phase<P_I, S>(x, op); break;
-        case 24 + P_MI: small_phase<P_MI, S>(x, op); break;
+        case 16 + P_NEG: small_phase<P_NEG, S>(x, op); break;
+        case 16 + P_I: small_phase<P_I, S>(x, op); break;
+        case 16 + P_MI: small_phase<P_MI, S>(x, op); break;
         default: small_phase<P_GENERAL, S>(x, op); break;
     }
 #undef SV_SMALL_FORM
@@ -512,24 +511,23 @@ __global__ void __launch_bounds__(kSmallThreads<R>) k_small_run(C2<R> *__restric
     __syncthreads();
     for (int k = 0; k < a.nops;) {
         const int cnt = ops[k].code;
-        const int s0 = ops[k].s[0], s1 = ops[k].s[1], s2 = int(ops[k].imask);
-        const uint32_t d0 = small_pos<R>(1u << s0), d1 = small_pos<R>(1u << s1), d2 = small_pos<R>(1u << s2);
+        const int s0 = ops[k].s[0], s1 = ops[k].s[1];
+        const uint32_t d0 = small_pos<R>(1u << s0), d1 = small_pos<R>(1u << s1);
         for (uint32_t w = threadIdx.x; w < namps >> S; w += blockDim.x) {
             uint32_t i = w + (w & ~((1u << s0) - 1));  // a zero bit inserted at s0
             if (S > 1) i += i & ~((1u << s1) - 1);
-            if (S > 2) i += i & ~((1u << s2) - 1);
             const uint32_t p = small_pos<R>(i);
             C2<R> x[1 << S];
 #pragma unroll
             for (int v = 0; v < (1 << S); ++v)
-                x[v] = sm[p ^ (v & 1 ? d0 : 0u) ^ (v & 2 ? d1 : 0u) ^ (v & 4 ? d2 : 0u)];
+                x[v] = sm[p ^ (v & 1 ? d0 : 0u) ^ (v & 2 ? d1 : 0u)];
             for (int j = k + 1; j <= k + cnt; ++j) {
                 const SmallOp<R> &op = ops[j];
                 if ((i & op.imask) == op.imask) small_gate<S>(x, op);
             }
 #pragma unroll
             for (int v = 0; v < (1 << S); ++v)
-                sm[p ^ (v & 1 ? d0 : 0u) ^ (v & 2 ? d1 : 0u) ^ (v & 4 ? d2 : 0u)] = x[v];
+                sm[p ^ (v & 1 ? d0 : 0u) ^ (v & 2 ? d1 : 0u)] = x[v];
         }
         __syncthreads();
         k += cnt + 1;
@@ -551,7 +549,7 @@ size_t small_stage(int n, const Gate1 *g, size_t i, size_t count, SmallRun<R> *a
         qs |= b;
     }
     for (int q = n - 1; q >= 0 && __builtin_popcount(qs) < S; --q) qs |= 1u << q;  // high ones: no bank conflicts
-    int slot[32], s[3] = {0, 0, 0}, ns = 0;
+    int slot[32], s[2] = {0, 0}, ns = 0;
     for (int q = 0; q < n; ++q) {
         slot[q] = -1;
         if (qs >> q & 1u) {
@@ -564,7 +562,6 @@ size_t small_stage(int n, const Gate1 *g, size_t i, size_t count, SmallRun<R> *a
     hd.code = uint8_t(e - i);
     hd.s[0] = uint8_t(s[0]);
     hd.s[1] = uint8_t(s[1]);
-    hd.imask = uint32_t(s[2]);
     for (; i < e; ++i) {
         SmallOp<R> &op = a->op[a->nops++];
         op = SmallOp<R>{};
@@ -575,9 +572,9 @@ size_t small_stage(int n, const Gate1 *g, size_t i, size_t count, SmallRun<R> *a
         uint32_t cond = g[i].control < 0 ? 0u : 1u << g[i].control;
         if (is_phase(g[i])) {
             cond |= 1u << g[i].target;
-            op.code = uint8_t(24 + phase_form(op.u));
+            op.code = uint8_t(16 + phase_form(op.u));
         } else {
-            op.code = uint8_t(3 * gate_form(op.u) + slot[g[i].target]);
+            op.code = uint8_t(2 * gate_form(op.u) + slot[g[i].target]);
         }
         for (int q = 0; q < n; ++q)
             if (cond >> q & 1u) {
@@ -594,15 +591,6 @@ cudaError_t small_run(sv_state *h, const Gate1 *g, size_t count) {
     const int tlog = n - S;
     const int threads = tlog < 5 ? 32 : (1 << tlog) > kSmallThreads<R> ? kSmallThreads<R> : 1 << tlog;
     const int smem = int(sizeof(C2<R>)) << n;
-    if (smem > 32 * 1024) {
-        static std::atomic<uint64_t> configured{0};
-        if (attrs_needed(configured, h->device)) {
-            const cudaError_t e = cudaFuncSetAttribute(k_small_run<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                       int(sizeof(C2<R>)) << small_run_max_n(h->dt));
-            if (e != cudaSuccess) return e;
-            attrs_set(configured, h->device);
-        }
-    }
     for (size_t i = 0; i < count;) {
         SmallRun<R> a;
         a.n = n;
@@ -625,7 +613,7 @@ cudaError_t small_run(sv_state *h, const Gate1 *g, size_t count) {
 // counted exactly on the host) are owed: those gates are then 4 additions per
 // pair instead of 6 to 10 operations, and a later launch pays the factors with
 // one multiplication per component.  20 qubits, 590 gates of the random family
-// in complex128: 4.00 ms with a launch per gate, 2.66 now; 236 gates in
+// in complex128: 4.00 ms with a launch per gate, 2.77 now; 236 gates in
 // complex64: 0.10 ms.
 // Few forms keep the code small (a launch starts with it uncached), and the
 // gates come as kernel parameters, so that branches and factors are uniform.
@@ -952,19 +940,17 @@ cudaError_t launch_gate1(sv_state *h, const Gate1 &g) {
     return launch_enc_gate1(h, g);
 }
 
-// Largest small state: complex64 up to 128 KB of shared memory (14 qubits, 205
-// gates: 174 us against 370 with one launch per gate); complex128 while one
-// SM's FP64 pipe beats a launch on all of them (10 qubits, 145 gates: 166
-// against 195 us; 11 qubits, 160 gates: 336 against 215).
-int small_run_max_n(sv_dtype dt) { return dt == SV_C64 ? 14 : dt == SV_C128 ? 10 : 0; }
+// Largest small state: beyond it one CTA is slower than runs of gates on many
+// (k_gate_run).  Random circuits of depth 10, one CTA against runs: complex64 10
+// qubits 35 and 35 us, 11 qubits 43 and 39, 14 qubits 173 and 51; complex128 8
+// qubits 56 and 62, 9 qubits 82 and 72, 10 qubits 153 and 74.
+int small_run_max_n(sv_dtype dt) { return dt == SV_C64 ? 10 : dt == SV_C128 ? 8 : 0; }
 
 cudaError_t launch_small_run(sv_state *h, const Gate1 *g, size_t count) {
-    // amplitudes per thread: two target bits up to 11 qubits, where threads are
-    // few (10 qubits, 145 gates: 35 us; 41 with one bit, 39 with three), three
-    // from 12 on (13 qubits, 190 gates: 93 us against 121); one for complex128,
-    // whose FP64 chains want many warps (8 qubits, 115 gates: 60 us against 86)
-    if (h->dt == SV_C128) return small_run<double, 1>(h, g, count);
-    return h->n < 12 ? small_run<float, 2>(h, g, count) : small_run<float, 3>(h, g, count);
+    // amplitudes per thread: two target bits in complex64 (10 qubits, 145 gates:
+    // 35 us; 41 with one bit, 39 with three); one in complex128, whose FP64
+    // chains want many warps (8 qubits, 115 gates: 60 us against 86)
+    return h->dt == SV_C128 ? small_run<double, 1>(h, g, count) : small_run<float, 2>(h, g, count);
 }
 
 // States of at most 64 MiB (half of L2): a gate's pass reads and writes L2.
