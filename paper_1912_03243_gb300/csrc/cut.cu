@@ -243,10 +243,10 @@ std::mutex g_sched_mu;
 std::unordered_map<std::string, Schedule> g_sched;
 constexpr size_t kSchedCacheMax = 256;
 
-std::string schedule_key(const Half &h, int S) {
+std::string schedule_key(const Half &h, int S, bool remap) {
     std::string k = std::to_string(h.nlocal) + "," + std::to_string(h.nq) + "," + std::to_string(S) + "," +
-                    std::to_string(int(prefix_sharing())) + "," + tile_config_name(tile_config64()) + "," +
-                    tile_codegen_key() + "," + std::to_string(plan_lookahead_width()) + "|";
+                    std::to_string(int(prefix_sharing())) + "," + std::to_string(int(remap)) + "," +
+                    tile_config_name(tile_config64()) + "," + tile_codegen_key() + "," + std::to_string(plan_lookahead_width()) + "|";
     int dev = 0;
     cudaGetDevice(&dev);
     k += std::to_string(dev) + "|";
@@ -261,12 +261,14 @@ std::string schedule_key(const Half &h, int S) {
     return k;
 }
 
-sv_status plan_half_uncached(Half &h, int S);
+sv_status plan_half_uncached(Half &h, int S, bool remap);
 
 // The schedule of a partition: planned and compiled once, then run for every
 // branch part (the fixed branch bits of a part are launch parameters).
-sv_status plan_half(Half &h, int S) {
-    const std::string key = schedule_key(h, S);
+// remap: stages may read the previous stage's vector; else copies in place,
+// which need no memory besides the vector.
+sv_status plan_half(Half &h, int S, bool remap) {
+    const std::string key = schedule_key(h, S, remap);
     {
         std::lock_guard<std::mutex> lock(g_sched_mu);
         auto it = g_sched.find(key);
@@ -277,7 +279,7 @@ sv_status plan_half(Half &h, int S) {
             return SV_OK;
         }
     }
-    const sv_status s = plan_half_uncached(h, S);
+    const sv_status s = plan_half_uncached(h, S, remap);
     if (s) return s;
     std::lock_guard<std::mutex> lock(g_sched_mu);
     if (g_sched.size() >= kSchedCacheMax) g_sched.clear();
@@ -285,10 +287,10 @@ sv_status plan_half(Half &h, int S) {
     return SV_OK;
 }
 
-sv_status plan_half_uncached(Half &h, int S) {
+sv_status plan_half_uncached(Half &h, int S, bool remap_ok) {
     h.stages.clear();
     h.init_all = !prefix_sharing();
-    h.remap = !h.init_all && h.nlocal >= tile_config64().m;
+    h.remap = remap_ok && !h.init_all && h.nlocal >= tile_config64().m;
     if (h.init_all) {
         HalfStage st;
         st.level = S;
@@ -372,13 +374,26 @@ void choose_tiles(Half &h, size_t m, const uint64_t *z, int nwords) {
 
 size_t align256(size_t b) { return (b + 255) & ~size_t(255); }
 
-// Bytes of the stage vectors a partition needs besides h.d: every stage but
-// the last, and the chunk buffer of a chunked one.
-size_t work_bytes(const Half &h) {
-    if (!h.remap) return 0;
+// Where the stages' vectors are: two areas, by turns, because a stage reads
+// the previous one's vector only.  The last stage's area is the chunk buffer,
+// or h.d itself where the last stage runs whole (the stages before it that
+// share the area are smaller); the other is workspace.
+int stage_area(const Half &h, size_t i) { return int((h.stages.size() - 1 - i) & 1); }
+bool area_in_work(const Half &h, int area) { return area == 1 || h.chunk < h.nbits; }
+size_t area_bytes(const Half &h, int area) {
     size_t b = 0;
-    for (size_t i = 0; i + 1 < h.stages.size(); ++i) b += align256(sizeof(float2) << (h.nlocal + h.stages[i].level));
-    if (h.chunk < h.nbits) b += align256(sizeof(float2) << (h.nlocal + h.chunk));
+    for (size_t i = 0; i < h.stages.size(); ++i) {
+        const int live = i + 1 == h.stages.size() ? h.chunk : h.stages[i].level;
+        if (stage_area(h, i) == area) b = std::max(b, sizeof(float2) << (h.nlocal + live));
+    }
+    return align256(b);
+}
+
+// Bytes of the areas in the workspace.
+size_t work_bytes(const Half &h) {
+    size_t b = 0;
+    for (int area = 0; area < 2; ++area)
+        if (h.remap && area_in_work(h, area)) b += area_bytes(h, area);
     return b;
 }
 
@@ -423,17 +438,18 @@ sv_status exec_half(Half &h, cudaStream_t st, int S, uint64_t param, char *work,
     }
     const int tile = tile_config64().m;
     auto tiles = [&](int level) { return uint64_t(1) << (h.nlocal + level - tile); };
+    float2 *area[2];
+    for (int k = 0; k < 2; ++k) {
+        area[k] = area_in_work(h, k) ? reinterpret_cast<float2 *>(work) : h.d;
+        if (area_in_work(h, k)) work += area_bytes(h, k);
+    }
     const float2 *src = nullptr;
     int src_level = 0;
     for (size_t i = 0; i < h.stages.size(); ++i) {
         const HalfStage &stage = h.stages[i];
         const bool last = i + 1 == h.stages.size();
         const int live = last ? h.chunk : stage.level;  // branch bits of this stage's vector
-        float2 *dst = h.d;
-        if (!last || h.chunk < h.nbits) {
-            dst = reinterpret_cast<float2 *>(work);
-            work += align256(sizeof(float2) << (h.nlocal + live));
-        }
+        float2 *dst = area[stage_area(h, i)];
         if (i == 0) {  // |0...0> of branch 0
             SV_CUDA_TRY(cudaMemsetAsync(dst, 0, sizeof(float2) << h.nlocal, st));
             k_branch_init<<<1, 32, 0, st>>>(dst, h.nlocal, 0);
@@ -632,31 +648,50 @@ static sv_status cut_impl(const char *text, int n, const uint8_t *part_of, int P
     if (m == 0) return SV_OK;
 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    for (int p = 0; p < P && s == SV_OK; ++p) s = plan_half(parts[p], parts[p].nbits);
-    if (s) return s;
+    // device memory: the vectors (or kept amplitudes), one workspace for the
+    // partitions, which run one after another, bit strings, indices, results
+    size_t bytesV = 0, bytesW = 0, bytesI = 0, total = 0;
+    const size_t bytesZ = align256(m * size_t(nwords) * sizeof(uint64_t)), bytesO = align256(m * sizeof(double2));
+    size_t free_b = 0, total_b = 0, least = 0;
     for (int p = 0; p < P; ++p) {
+        s = plan_half(parts[p], parts[p].nbits, true);
+        if (s) return s;
         choose_chunk(parts[p], m);
         choose_tiles(parts[p], m, z, nwords);
     }
-
-    // device memory: the vectors (or kept amplitudes), one workspace for the
-    // partitions, which run one after another, bit strings, indices, results
-    size_t bytesV = 0, bytesW = 0;
-    bool kept = false;
-    for (int p = 0; p < P; ++p) {
-        bytesV += align256(result_bytes(parts[p], m));
-        bytesV += align256(parts[p].want.size() * sizeof(unsigned));
-        bytesW = std::max(bytesW, work_bytes(parts[p]));
-        kept = kept || parts[p].chunk < parts[p].nbits;
-    }
-    const size_t bytesZ = align256(m * size_t(nwords) * sizeof(uint64_t)), bytesO = align256(m * sizeof(double2));
-    const size_t bytesI = kept ? align256(m * sizeof(uint64_t)) : 0;
-    const size_t total = bytesV + bytesW + bytesZ + bytesO + bytesI;
-    size_t free_b = 0, total_b = 0;
-    SV_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-    if (total + (size_t(256) << 20) > free_b) {
-        set_error("decomposition needs %zu bytes of device memory, %zu free", total, free_b);
-        return SV_ERR_OOM;
+    // Where the stages' own vectors do not fit beside the results, partitions
+    // whose last stage runs whole take the schedule in place (no vector but
+    // the result), and where that does not fit either, every partition.
+    for (int attempt = 0;; ++attempt) {
+        auto in_place = [&](const Half &h) { return attempt == 2 || (attempt == 1 && h.chunk == h.nbits); };
+        bytesV = bytesW = bytesI = 0;
+        for (int p = 0; p < P; ++p) {
+            const Half &h = parts[p];
+            if (in_place(h)) {
+                bytesV += align256(sizeof(float2) << h.nq);
+                continue;
+            }
+            bytesV += align256(result_bytes(h, m)) + align256(h.want.size() * sizeof(unsigned));
+            bytesW = std::max(bytesW, work_bytes(h));
+            if (h.chunk < h.nbits) bytesI = align256(m * sizeof(uint64_t));
+        }
+        total = bytesV + bytesW + bytesZ + bytesO + bytesI;
+        least = attempt == 0 ? total : std::min(least, total);
+        SV_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+        if (total + (size_t(256) << 20) <= free_b) {
+            for (int p = 0; p < P; ++p) {
+                if (!in_place(parts[p]) || !parts[p].remap) continue;
+                s = plan_half(parts[p], parts[p].nbits, false);
+                if (s) return s;
+                choose_chunk(parts[p], m);
+                choose_tiles(parts[p], m, z, nwords);
+            }
+            break;
+        }
+        if (attempt == 2) {
+            set_error("decomposition needs %zu bytes of device memory, %zu free", least, free_b);
+            return SV_ERR_OOM;
+        }
     }
     if (fault_injected("alloc")) {
         set_error("injected allocation failure");

@@ -280,3 +280,28 @@ def test_chunked_last_stage(S, monkeypatch, rows, cols, m):
     monkeypatch.setenv("SV_CUT_PREFIX", "0")
     batched, _ = S.sv_cut_amplitudes(c, n, mask, z[:m])
     assert np.max(np.abs(got - batched)) <= tol
+
+
+def test_fits_where_the_results_fit(S):
+    """A decomposition whose branch vectors fit the free memory runs there: the
+    stages' own vectors are extra and must not make it fail.  48-qubit grid with
+    more strings than kept amplitudes may take room for (whole vectors, 64 GiB),
+    with memory left for them and 1 GiB; the amplitudes are those of the
+    schedule that had room."""
+    import torch
+
+    result = (2 << 32) * 8
+    if torch.cuda.mem_get_info()[0] < result + (8 << 30):
+        pytest.skip("not enough device memory")
+    c = C.grid_circuit(6, 8, 8, 3)
+    mask = C.grid_partition_mask(6, 8, 3)
+    z = C.random_bitstrings(600000, 48, 11)
+    ref, s0 = S.sv_cut_amplitudes(c, 48, mask, z)
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - result - (1 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        got, s1 = S.sv_cut_amplitudes(c, 48, mask, z)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    assert s0 == s1 == 8
+    close(got, ref)
