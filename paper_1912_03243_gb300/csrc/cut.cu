@@ -355,8 +355,8 @@ void choose_chunk(Half &h, size_t m) {
 // 1024 strings name 39% of the 2048 tiles of 24 qubits.
 void choose_tiles(Half &h, size_t m, const uint64_t *z, int nwords) {
     h.want.clear();
-    const uint64_t ntiles = uint64_t(1) << (h.nlocal - tile_config64().m);
-    if (h.chunk >= h.nbits || m > ntiles) return;
+    if (h.chunk >= h.nbits) return;  // (a chunked partition has at least a tile's qubits)
+    if (m > uint64_t(1) << (h.nlocal - tile_config64().m)) return;
     const uint64_t tile = h.stages.back().last_tile;
     for (size_t j = 0; j < m; ++j) {
         uint64_t t = 0;
