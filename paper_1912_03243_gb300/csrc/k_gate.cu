@@ -613,8 +613,8 @@ cudaError_t small_run(sv_state *h, const Gate1 *g, size_t count) {
 // counted exactly on the host) are owed: those gates are then 4 additions per
 // pair instead of 6 to 10 operations, and a later launch pays the factors with
 // one multiplication per component.  20 qubits, 590 gates of the random family
-// in complex128: 4.00 ms with a launch per gate, 2.77 now; 236 gates in
-// complex64: 0.10 ms.
+// in complex128: 4.00 ms with a launch per gate, 2.77 in runs that multiply for
+// every H, 1.86 now; 236 gates in complex64: 0.094 ms.
 // Few forms keep the code small (a launch starts with it uncached), and the
 // gates come as kernel parameters, so that branches and factors are uniform.
 enum RunKind : uint8_t { R_HAD, R_SX, R_SXD, R_SY, R_SYD, R_GENERAL, R_SWAP, R_NEG, R_TURN, R_PHASE };
@@ -693,7 +693,8 @@ __device__ __forceinline__ void run_phase(C2<R> (&x)[1 << S], uint32_t mask, R p
 
 // The same for one mask known to the compiler: a test per register becomes a
 // predicate, and a predicated FP64 instruction takes its turn in the pipe also
-// where no lane executes it (20-qubit Fourier transform in complex128 1.78 ms, 0.96 so).
+// where no lane executes it (20-qubit Fourier transform in complex128 1.78 ms with
+// tests, 0.96 so; 0.74 now that H owes its factor too).
 template <uint32_t MASK, int S, typename R>
 __device__ __forceinline__ void run_phase_of(C2<R> (&x)[1 << S], R pr, R pi) {
     if constexpr (MASK < (1u << S)) {
@@ -968,9 +969,10 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
     constexpr size_t kWindow = 1024;  // gates looked at ahead of the first unplaced one
     // Register qubits.  A small complex128 state is bound by the FP64 pipes of
     // the few SMs that its threads fill (random circuits of depth 8: 11 qubits
-    // 73 us with two, 197 with four; 15 qubits 103 and 271), a larger one by the
-    // passes over L2 (22 qubits 4.70 ms with two, 4.48 with four); complex64 15
-    // qubits 45 us with three and 51 with four, 23 qubits 619 and 555.
+    // 58 us with two, 131 with four; 15 qubits 82 and 183), a larger one by the
+    // passes over L2 (22 qubits 3.08 ms with two, 3.04 with four; its Fourier
+    // transform 3.17 and 2.97); complex64 15 qubits 41 us with three and 47 with
+    // four, 23 qubits 545 and 495.
     const int slots = dt == SV_C128 ? (n <= 18 ? 2 : 4) : (n <= 17 ? 3 : 4);
     out->slots = slots;
     std::vector<char> placed(g.size(), 0);
@@ -998,7 +1000,9 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
         o.kind = form == G_SWAP ? R_SWAP : R_GENERAL;
         if (g[i].control >= 0) continue;
         switch (form) {
-            case G_HAD: o.kind = u[0] == std::sqrt(0.5) ? R_HAD : R_GENERAL; break;
+            case G_HAD:  // the gate table's 1 / sqrt(2) is one place below the rounded sqrt(1/2)
+                o.kind = std::fabs(u[0] - std::sqrt(0.5)) <= 1.2e-16 ? R_HAD : R_GENERAL;
+                break;
             case G_SX: o.kind = R_SX; break;
             case G_SXD: o.kind = R_SXD; break;
             case G_SY: o.kind = R_SY; break;

@@ -287,3 +287,23 @@ def test_basis_and_norm(S):
         a = s.amplitudes([1234, 0])
         assert a[0] == 1 and a[1] == 0
         assert s.norm() == 1.0
+
+
+@pytest.mark.parametrize("dtype,n", [("c64", 11), ("c64", 19), ("c128", 9), ("c128", 20)])
+def test_hadamard_factors_are_owed(S, dtype, n):
+    """Runs of gates owe the factor of the library's H: two layers of it on a
+    basis state are additions of whole numbers and one power of two, so the
+    basis state comes back exactly (with a multiplication per gate 2 c c is one
+    place off 1 in both precisions)."""
+    c = C.Circuit(n)
+    for _ in range(2):
+        for q in range(n):
+            c.add("H", q)
+    s = S.StateVector(n, dtype)
+    p = s.plan(c, "pergate")
+    for _ in range(3):  # direct, capture, replay
+        s.set_basis(5)
+        p.execute()
+        got = s.to_numpy()
+        assert got[5] == 1 and np.count_nonzero(got) == 1
+    p.free()
