@@ -17,6 +17,11 @@
  *               scales (one per 256 consecutive amplitudes; one scale when
  *               n < 8).  Amplitude x = sign(q) * scale * fl(|q|/127).
  *   sv_bytes_required() gives the exact device footprint of each layout.
+ *   States are meant to have norm about 1.  Between the gates of one launch
+ *   values may exceed the state's norm where factors of 2^(-1/2) are applied
+ *   late: by up to 2^4 (SV_C128: 2^12) in SV_MODE_PERGATE and about 2^80 in
+ *   SV_MODE_TILED, which an unnormalised state near the type's range must
+ *   leave room for.
  * Matrices.  Complex matrices are row-major, each entry (re, im) as two
  *   doubles.  A 2x2 gate is 8 doubles: u00 u01 u10 u11.
  * Ownership.  Handles belong to the library until sv_free().  Every array a

@@ -611,13 +611,23 @@ cudaError_t small_run(sv_state *h, const Gate1 *g, size_t count) {
 // complex128 also by the FP64 pipe (two lanes per SM and clock), so the scalar
 // factors of H, SX, SY and their adjoints (powers of e^(i pi/4) and 2^(-1/2),
 // counted exactly on the host) are owed: those gates are then 4 additions per
-// pair instead of 6 to 10 operations, and a later launch pays the factors with
-// one multiplication per component.  20 qubits, 590 gates of the random family
+// pair instead of 6 to 10 operations, and a multiplication per component pays
+// 2^-4 (complex128: 2^-12) whenever as much is owed, the last launch the rest.
+// The powers of two are exact, and no value in between exceeds the state's norm
+// by more than that factor.  20 qubits, 590 gates of the random family
 // in complex128: 4.00 ms with a launch per gate, 2.77 in runs that multiply for
-// every H, 1.86 now; 236 gates in complex64: 0.094 ms.
+// every H, 1.85 now; 236 gates in complex64: 0.097 ms.
 // Few forms keep the code small (a launch starts with it uncached), and the
 // gates come as kernel parameters, so that branches and factors are uniform.
-enum RunKind : uint8_t { R_HAD, R_SX, R_SXD, R_SY, R_SYD, R_GENERAL, R_SWAP, R_NEG, R_TURN, R_PHASE };
+enum RunKind : uint8_t { R_HAD, R_SX, R_SXD, R_SY, R_SYD, R_GENERAL, R_SWAP, R_NEG, R_TURN, R_PHASE, R_SCALE };
+
+// Factors 2^(-1/2) owed at most, and what R_SCALE multiplies by to pay them.
+// complex64 pays early, for the range of its exponent: a 32nd of a run's
+// operations, under its launches.
+template <typename R>
+constexpr int kRunOwed = sizeof(R) == 4 ? 8 : 24;
+template <typename R>
+constexpr R kRunScale = R(1) / R(1 << kRunOwed<R> / 2);
 
 template <typename R>
 struct RunArgs {
@@ -725,6 +735,13 @@ __device__ __forceinline__ void run_gate(C2<R> (&x)[1 << S], const GateRunHead &
     if (op.kind >= R_NEG) {
         if (op.kind == R_NEG) run_phase<P_NEG, S>(x, op.rmask, R(0), R(0));
         else if (op.kind == R_PHASE) run_phase_general<S>(x, op.rmask, u[0], u[1]);
+        else if (op.kind == R_SCALE) {
+#pragma unroll
+            for (int v = 0; v < (1 << S); ++v) {
+                x[v].re *= kRunScale<R>;
+                x[v].im *= kRunScale<R>;
+            }
+        }
         else if (op.arg == 1) run_phase<P_I, S>(x, op.rmask, R(0), R(0));
         else run_phase<P_MI, S>(x, op.rmask, R(0), R(0));
         return;
@@ -943,8 +960,8 @@ cudaError_t launch_gate1(sv_state *h, const Gate1 &g) {
 
 // Largest small state: beyond it one CTA is slower than runs of gates on many
 // (k_gate_run).  Random circuits of depth 10, one CTA against runs: complex64 10
-// qubits 35 and 35 us, 11 qubits 43 and 39, 14 qubits 173 and 51; complex128 8
-// qubits 56 and 62, 9 qubits 82 and 72, 10 qubits 153 and 74.
+// qubits 33 and 33 us, 11 qubits 42 and 37, 12 qubits 66 and 40; complex128 9
+// qubits 82 and 58, 10 qubits 152 and 60.
 int small_run_max_n(sv_dtype dt) { return dt == SV_C64 ? 10 : dt == SV_C128 ? 8 : 0; }
 
 cudaError_t launch_small_run(sv_state *h, const Gate1 *g, size_t count) {
@@ -1010,6 +1027,7 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
             default: break;
         }
     }
+    const int owed = dt == SV_C128 ? kRunOwed<double> : kRunOwed<float>;
     int eighths = 0, halves = 0;  // factor owed: e^(i pi eighths / 4) 2^(-halves / 2)
     size_t start = 0;
     while (true) {
@@ -1030,7 +1048,7 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
                 for (int q = 0, k = 0; q < n; ++q)
                     if (qs >> q & 1) r.q[k++] = q;
             }
-            for (size_t i = start; i < end && r.count < kRunMaxOps; ++i) {
+            for (size_t i = start; i < end && r.count + 1 < kRunMaxOps; ++i) {  // (room for a gate and R_SCALE)
                 if (placed[i]) continue;
                 const uint64_t t = uint64_t(1) << g[i].target;
                 const uint64_t c = g[i].control < 0 ? 0 : uint64_t(1) << g[i].control;
@@ -1063,8 +1081,14 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
                 }
                 o.imask = uint32_t(cond & ~qs);
                 if (o.kind <= R_SYD) {  // SX, SY: e^(i pi/4) 2^(-1/2), H: 2^(-1/2)
-                    ++halves;
                     eighths += o.kind == R_SX || o.kind == R_SY ? 1 : o.kind == R_SXD || o.kind == R_SYD ? -1 : 0;
+                    if (++halves == owed) {
+                        GateRunHead pay{};
+                        pay.kind = R_SCALE;
+                        out->ops.push_back(pay);  // (o is no longer valid)
+                        ++r.count;
+                        halves = 0;
+                    }
                 } else if (o.kind == R_GENERAL || o.kind == R_PHASE) {
                     double u[8];
                     factors(i, u);
@@ -1079,15 +1103,13 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
             }
         }
         r.ucount = int(out->u.size() - r.ufirst);
-        // the factor, once it exceeds 2^-12 or at the end
         while (start < g.size() && placed[start]) ++start;
-        if (halves >= 24 || start == g.size()) {
+        if (start == g.size()) {  // the rest of the factor
             const int k = eighths & 7;
             r.odd = k & 1;
             r.quarter = k >> 1;
             halves += r.odd;  // e^(i pi / 4) = (1 + i) 2^(-1/2)
             r.m = std::ldexp(halves & 1 ? std::sqrt(0.5) : 1.0, -(halves >> 1));
-            eighths = halves = 0;
         }
         out->runs.push_back(r);
     }

@@ -307,3 +307,29 @@ def test_hadamard_factors_are_owed(S, dtype, n):
         got = s.to_numpy()
         assert got[5] == 1 and np.count_nonzero(got) == 1
     p.free()
+
+
+@pytest.mark.parametrize("dtype,n,e", [("c64", 11, 120), ("c64", 18, 120), ("c64", 18, -100), ("c128", 9, 1008), ("c128", 19, 1008),
+                                       ("c128", 19, -900)])
+def test_unnormalised_states(S, orc, dtype, n, e):
+    """Per-gate plans keep room for states far from norm 1: norm 2^120
+    (complex128: 2^1008), where a factor owed over many gates would leave the
+    type's range, and the smallest ones.  Powers of two are exact, so the
+    results are those of the normalised state times 2^e.  Many gates on few
+    qubits, so that runs are long."""
+    c = C.Circuit(n)
+    rng = np.random.default_rng(n)
+    for _ in range(100):
+        for q in (0, n - 1):
+            c.add(str(rng.choice(["H", "SX", "SY", "SXDG", "SYDG", "T"])), q)
+    for q in range(n):
+        c.add("H", q)
+    psi = C.random_state(n, 33)
+    ref = orc.run(c, psi=psi)
+    s = S.StateVector(n, dtype)
+    p = s.plan(c, "pergate")
+    for _ in range(3):  # direct, capture, replay
+        s.from_numpy(psi * 2.0**e)
+        p.execute()
+        check(dtype, s.to_numpy().astype(np.complex128) * 2.0**-e, ref)
+    p.free()
