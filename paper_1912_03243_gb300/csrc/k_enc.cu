@@ -380,17 +380,25 @@ __device__ __forceinline__ uint32_t amp_ctl(int c, int lane) {
     return c == 0 ? 0xAAu : c == 1 ? 0xCCu : 0xF0u;
 }
 
-template <int SHAPE, bool CTL>
+// How an in-block control is met: none; every word computed and the words'
+// halves selected (runs of gates, whose few warps want instructions without
+// branches in between); words left out (one gate per pass, whole words only).
+enum EncCtl { CTL_NONE = 0, CTL_SELECT, CTL_SKIP };
+
+template <int SHAPE, int CTL>
 __device__ __forceinline__ void gate2_sel(const Mat2<SHAPE> &m, Amp2 &a, Amp2 &b, uint32_t bits) {
-    if constexpr (CTL)
+    if constexpr (CTL == CTL_SELECT) {
         gate2_ctl<SHAPE>(m, a, b, bits);
-    else
+    } else if constexpr (CTL == CTL_SKIP) {
+        if (bits & 1u) gate2<SHAPE>(m, a, b);
+    } else {
         gate2<SHAPE>(m, a, b);
+    }
 }
 
 // The rearranged words of a block, decoded and updated; returns the lane's
 // absolute maximum.  cm: pair_ctl.
-template <int SHAPE, bool CTL>
+template <int SHAPE, int CTL>
 __device__ __forceinline__ float update_in(const DecTable &dec, const Mat2<SHAPE> &m, uint32_t cm, const uint4 &v,
                                            float s, Amp2 (&x)[4]) {
     const F2 s2 = dup2(s);
@@ -408,9 +416,20 @@ __device__ __forceinline__ float update_in(const DecTable &dec, const Mat2<SHAPE
 __device__ __forceinline__ uint4 as_u4(const int4 &v) {
     return make_uint4(uint32_t(v.x), uint32_t(v.y), uint32_t(v.z), uint32_t(v.w));
 }
+__device__ __forceinline__ int4 as_i4(const uint4 &v) { return make_int4(int(v.x), int(v.y), int(v.z), int(v.w)); }
+__device__ __forceinline__ int4 arranged(const int4 &v, int t, int lane) {
+    uint4 u = as_u4(v);
+    arrange(u, t, lane);
+    return as_i4(u);
+}
+__device__ __forceinline__ int4 arranged_back(const int4 &v, int t, int lane) {
+    uint4 u = as_u4(v);
+    arrange_back(u, t, lane);
+    return as_i4(u);
+}
 
 // One in-block gate on a block: codes v, scale s.
-template <int SHAPE, bool CTL>
+template <int SHAPE, int CTL>
 __device__ __forceinline__ void block_gate_in(const DecTable &dec, const Mat2<SHAPE> &m, int t, uint32_t cm, int lane, uint4 &v, float &s) {
     arrange(v, t, lane);
     Lane8 x;
@@ -420,7 +439,7 @@ __device__ __forceinline__ void block_gate_in(const DecTable &dec, const Mat2<SH
 }
 
 // The same on two blocks at once (independent instructions to issue).
-template <int SHAPE, bool CTL>
+template <int SHAPE, int CTL>
 __device__ __forceinline__ void block_gate_in2(const DecTable &dec, const Mat2<SHAPE> &m, int t, uint32_t cm, int lane, uint4 &v0, float &s0,
                                                uint4 &v1, float &s1) {
     arrange(v0, t, lane);
@@ -439,7 +458,7 @@ __device__ __forceinline__ void block_gate_in2(const DecTable &dec, const Mat2<S
 
 // One gate on a pair of blocks that differ in the target bit.  ENC_DIAG1
 // leaves the lower block as it is: its codes are not needed.
-template <int SHAPE, bool CTL>
+template <int SHAPE, int CTL>
 __device__ __forceinline__ void block_gate_pair(const DecTable &dec, const Mat2<SHAPE> &m, uint32_t cm, int lane, int4 &v0, float &s0,
                                                 int4 &v1, float &s1) {
     Lane8 x, y;
@@ -479,9 +498,9 @@ __global__ void __launch_bounds__(32 * kGateWarps, 3) k_enc_gate_in(uint4 *__res
         uint4 v = codes[b * 32 + lane];
         float s = scales[b];
         if (ctl)
-            block_gate_in<SHAPE, true>(dec, m, a.t, cm, lane, v, s);
+            block_gate_in<SHAPE, CTL_SELECT>(dec, m, a.t, cm, lane, v, s);
         else
-            block_gate_in<SHAPE, false>(dec, m, a.t, cm, lane, v, s);
+            block_gate_in<SHAPE, CTL_NONE>(dec, m, a.t, cm, lane, v, s);
         codes[b * 32 + lane] = v;
         if (lane == 0) scales[b] = s;
     }
@@ -507,8 +526,13 @@ __global__ void __launch_bounds__(32 * kGateWarps, kAcrossCtas[SHAPE]) k_enc_gat
     const uint64_t wid = uint64_t(blockIdx.x) * kGateWarps + (threadIdx.x >> 5);
     const uint64_t nw = uint64_t(gridDim.x) * kGateWarps;
     const Mat2<SHAPE> m(a.u);
+    // An in-block control selects whole words of a lane: a control on qubit 0
+    // once the words are rearranged as for a target there (their upper
+    // amplitudes in words 2, 3).  Words without it are left out (27 qubits, SX
+    // with a control inside the blocks: 137 to 144 us; 157 with every word
+    // computed and its halves selected).
     const bool ctl = a.c >= 0 && a.c < kEncBlockLog2;
-    const uint32_t cm = amp_ctl(ctl ? a.c : -1, lane);
+    const uint32_t cm = amp_ctl(ctl ? (a.c == 0 ? 2 : a.c) : -1, lane);
     for (uint64_t w = wid; w < a.nwork; w += nw) {
         const uint64_t b0 = insert_zeros(w, a.nins, a.ins[0], a.ins[1]) | a.set_mask;
         const uint64_t b1 = b0 | a.tbit;
@@ -518,10 +542,19 @@ __global__ void __launch_bounds__(32 * kGateWarps, kAcrossCtas[SHAPE]) k_enc_gat
             v0 = codes[b0 * 32 + lane];
             s0 = scales[b0];
         }
-        if (ctl)
-            block_gate_pair<SHAPE, true>(dec, m, cm, lane, v0, s0, v1, s1);
-        else
-            block_gate_pair<SHAPE, false>(dec, m, cm, lane, v0, s0, v1, s1);
+        if (ctl) {
+            if (a.c == 0) {
+                v0 = arranged(v0, 0, lane);
+                v1 = arranged(v1, 0, lane);
+            }
+            block_gate_pair<SHAPE, CTL_SKIP>(dec, m, cm, lane, v0, s0, v1, s1);
+            if (a.c == 0) {
+                v0 = arranged_back(v0, 0, lane);
+                v1 = arranged_back(v1, 0, lane);
+            }
+        } else {
+            block_gate_pair<SHAPE, CTL_NONE>(dec, m, cm, lane, v0, s0, v1, s1);
+        }
         if constexpr (SHAPE != ENC_DIAG1) {
             codes[b0 * 32 + lane] = v0;
             if (lane == 0) scales[b0] = s0;
@@ -786,7 +819,7 @@ __device__ __forceinline__ uint4 flip_codes(uint4 v, uint32_t m) {
 // The gate `op` on every block (or pair of blocks) of the tile that meets its
 // block-level condition.  base: block index of the tile; tile block k is
 // base | spread[k].  In-block gates take two blocks at a time.
-template <int SHAPE, bool CTL>
+template <int SHAPE, int CTL>
 __device__ __forceinline__ void run_gate(const DecTable &dec, const EncRunOp &op, uint4 *tile, float &sc, uint32_t base,
                                          const uint32_t *spread, int nblk, int lane) {
     const Mat2<SHAPE> m(op.u);
@@ -906,27 +939,27 @@ __global__ void __launch_bounds__(32 * kRunWarps, 1) k_enc_run_in(uint4 *__restr
             switch (op.shape) {
                 case ENC_REAL:
                     if (op.c >= 0)
-                        run_gate<ENC_REAL, true>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_REAL, CTL_SELECT>(dec, op, tile, sc, base, spread, nblk, lane);
                     else
-                        run_gate<ENC_REAL, false>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_REAL, CTL_NONE>(dec, op, tile, sc, base, spread, nblk, lane);
                     break;
                 case ENC_DIAG:
                     if (op.c >= 0)
-                        run_gate<ENC_DIAG, true>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_DIAG, CTL_SELECT>(dec, op, tile, sc, base, spread, nblk, lane);
                     else
-                        run_gate<ENC_DIAG, false>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_DIAG, CTL_NONE>(dec, op, tile, sc, base, spread, nblk, lane);
                     break;
                 case ENC_DIAG1:
                     if (op.c >= 0)
-                        run_gate<ENC_DIAG1, true>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_DIAG1, CTL_SELECT>(dec, op, tile, sc, base, spread, nblk, lane);
                     else
-                        run_gate<ENC_DIAG1, false>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_DIAG1, CTL_NONE>(dec, op, tile, sc, base, spread, nblk, lane);
                     break;
                 default:
                     if (op.c >= 0)
-                        run_gate<ENC_GENERAL, true>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_GENERAL, CTL_SELECT>(dec, op, tile, sc, base, spread, nblk, lane);
                     else
-                        run_gate<ENC_GENERAL, false>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_GENERAL, CTL_NONE>(dec, op, tile, sc, base, spread, nblk, lane);
                     break;
             }
         }
