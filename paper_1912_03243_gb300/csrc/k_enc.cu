@@ -795,8 +795,14 @@ __global__ void __launch_bounds__(256) k_enc_xblocks(uint4 *__restrict__ codes, 
 // and the 64 KB table leave 16 warps on an SM at 128 registers.  (Decoding by
 // arithmetic instead of the table: 11.7 against 11.0 ms on 27 qubits and 160
 // gates; 24 warps at 80 registers: spills, 11.9 against 11.7.)
+//
+// A run inside the blocks takes one block per warp, its codes in registers
+// (57 of them), so that 32 warps share an SM: 64 gates at 25 qubits 1393 us,
+// 2057 in tiles of 16 blocks, 1454 with one pass each; 12 to 18 qubits 33 us
+// for any of them.
 
 constexpr int kRunWarps = 16;
+constexpr int kRunCtas0 = 2;  // CTAs per SM of runs inside single blocks
 
 struct EncRunArgs {
     uint64_t ntiles;
@@ -819,17 +825,22 @@ __device__ __forceinline__ uint4 flip_codes(uint4 v, uint32_t m) {
 // The gate `op` on every block (or pair of blocks) of the tile that meets its
 // block-level condition.  base: block index of the tile; tile block k is
 // base | spread[k].  In-block gates take two blocks at a time.
-template <int SHAPE, int CTL>
+template <int SHAPE, int CTL, int NB>
 __device__ __forceinline__ void run_gate(const DecTable &dec, const EncRunOp &op, uint4 *tile, float &sc, uint32_t base,
                                          const uint32_t *spread, int nblk, int lane) {
     const Mat2<SHAPE> m(op.u);
     const uint32_t hm = uint32_t(op.hi_mask), hv = uint32_t(op.hi_val);
     const int t = op.t;
-    uint4 *mine = tile + lane;
-    if (op.kind == ENC_OP_IN) {
+    uint4 *mine = NB == 0 ? tile : tile + lane;
+    if constexpr (NB == 0) {
+        if ((base & hm) != hv) return;
+        uint4 v = mine[0];
+        block_gate_in<SHAPE, CTL>(dec, m, t, pair_ctl(t, op.c, lane), lane, v, sc);  // (every lane holds the scale)
+        mine[0] = v;
+    } else if (op.kind == ENC_OP_IN) {
         const uint32_t cm = pair_ctl(t, op.c, lane);
         for (int k0 = 0; k0 < nblk; k0 += 2) {
-            const int k1 = nblk > 1 ? k0 + 1 : 0;
+            const int k1 = k0 + 1;
             const bool on0 = ((base | spread[k0]) & hm) == hv, on1 = ((base | spread[k1]) & hm) == hv;
             if (!on0 && !on1) continue;
             uint4 v0 = mine[k0 * 32], v1 = mine[k1 * 32];
@@ -868,7 +879,7 @@ __device__ __forceinline__ void run_gate(const DecTable &dec, const EncRunOp &op
 }
 
 template <int NB>  // tile bits, or -1: a.nbits
-__global__ void __launch_bounds__(32 * kRunWarps, 1) k_enc_run_in(uint4 *__restrict__ codes,
+__global__ void __launch_bounds__(32 * kRunWarps, NB == 0 ? kRunCtas0 : 1) k_enc_run_in(uint4 *__restrict__ codes,
                                                                      float *__restrict__ scales,
                                                                      const EncRunOp *__restrict__ gops,
                                                                      const EncRunArgs a) {
@@ -888,20 +899,23 @@ __global__ void __launch_bounds__(32 * kRunWarps, 1) k_enc_run_in(uint4 *__restr
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const DecTable dec{smem, uint32_t(lane) * 4u};
-    uint4 *tile = reinterpret_cast<uint4 *>(smem + kTabBytes) + (threadIdx.x >> 5) * (nblk * 32);
-    const uint64_t wid = uint64_t(blockIdx.x) * kRunWarps + (threadIdx.x >> 5);
-    const uint64_t nw = uint64_t(gridDim.x) * kRunWarps;
+    uint4 held;  // a single block's codes
+    uint4 *tile = &held;
+    if constexpr (NB != 0) tile = reinterpret_cast<uint4 *>(smem + kTabBytes) + (threadIdx.x >> 5) * (nblk * 32);
+    const int ml = NB == 0 ? 0 : lane;  // this lane's place in a block of the tile
+    const uint64_t wid = uint64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const uint64_t nw = uint64_t(gridDim.x) * (blockDim.x >> 5);
     for (uint64_t w = wid; w < a.ntiles; w += nw) {
         uint64_t b64 = w;
 #pragma unroll
         for (int j = 0; j < kEncRunMaxBits; ++j)
             if (NB == kEncRunMaxBits || j < a.nbits) b64 = insert_zero(b64, a.pos[j]);
         const uint32_t base = uint32_t(b64);  // at most 2^32 blocks (n <= 40)
-        const uint32_t mine = base | spread[lane & (nblk - 1)];
-        float sc = scales[mine];
+        const uint32_t own = base | spread[lane & (nblk - 1)];
+        float sc = scales[own];
 #pragma unroll
         for (int k = 0; k < nblk; ++k) {
-            tile[k * 32 + lane] = codes[uint64_t(base | spread[k]) * 32 + lane];
+            tile[k * 32 + ml] = codes[uint64_t(base | spread[k]) * 32 + lane];
         }
         for (int i = 0; i < a.nops; ++i) {
             const EncRunOp &op = ops[i];
@@ -918,19 +932,19 @@ __global__ void __launch_bounds__(32 * kRunWarps, 1) k_enc_run_in(uint4 *__restr
                                         (uint32_t(lane * 8) & g.lo_mask & 0xF8u) == (g.lo_val & 0xF8u);
                         m ^= on ? g.amps : 0u;
                     }
-                    if (__any_sync(0xffffffffu, m != 0)) tile[k * 32 + lane] = flip_codes(tile[k * 32 + lane], m);
+                    if (__any_sync(0xffffffffu, m != 0)) tile[k * 32 + ml] = flip_codes(tile[k * 32 + ml], m);
                 }
                 i = e - 1;
                 continue;
             }
-            if (op.kind == ENC_OP_SWAP) {  // X on a tile bit: the blocks change places
+            if (NB != 0 && op.kind == ENC_OP_SWAP) {  // X on a tile bit: the blocks change places
                 const uint32_t hm = uint32_t(op.hi_mask), hv = uint32_t(op.hi_val);
                 for (int k = 0; k < nblk; ++k) {
                     const int k1 = k | (1 << op.t);
                     if (k == k1 || ((base | spread[k]) & hm) != hv) continue;
-                    const uint4 v = tile[k * 32 + lane];
-                    tile[k * 32 + lane] = tile[k1 * 32 + lane];
-                    tile[k1 * 32 + lane] = v;
+                    const uint4 v = tile[k * 32 + ml];
+                    tile[k * 32 + ml] = tile[k1 * 32 + ml];
+                    tile[k1 * 32 + ml] = v;
                     const float s0 = __shfl_sync(0xffffffffu, sc, k), s1 = __shfl_sync(0xffffffffu, sc, k1);
                     sc = lane == k ? s1 : lane == k1 ? s0 : sc;
                 }
@@ -939,33 +953,33 @@ __global__ void __launch_bounds__(32 * kRunWarps, 1) k_enc_run_in(uint4 *__restr
             switch (op.shape) {
                 case ENC_REAL:
                     if (op.c >= 0)
-                        run_gate<ENC_REAL, CTL_SELECT>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_REAL, CTL_SELECT, NB>(dec, op, tile, sc, base, spread, nblk, lane);
                     else
-                        run_gate<ENC_REAL, CTL_NONE>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_REAL, CTL_NONE, NB>(dec, op, tile, sc, base, spread, nblk, lane);
                     break;
                 case ENC_DIAG:
                     if (op.c >= 0)
-                        run_gate<ENC_DIAG, CTL_SELECT>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_DIAG, CTL_SELECT, NB>(dec, op, tile, sc, base, spread, nblk, lane);
                     else
-                        run_gate<ENC_DIAG, CTL_NONE>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_DIAG, CTL_NONE, NB>(dec, op, tile, sc, base, spread, nblk, lane);
                     break;
                 case ENC_DIAG1:
                     if (op.c >= 0)
-                        run_gate<ENC_DIAG1, CTL_SELECT>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_DIAG1, CTL_SELECT, NB>(dec, op, tile, sc, base, spread, nblk, lane);
                     else
-                        run_gate<ENC_DIAG1, CTL_NONE>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_DIAG1, CTL_NONE, NB>(dec, op, tile, sc, base, spread, nblk, lane);
                     break;
                 default:
                     if (op.c >= 0)
-                        run_gate<ENC_GENERAL, CTL_SELECT>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_GENERAL, CTL_SELECT, NB>(dec, op, tile, sc, base, spread, nblk, lane);
                     else
-                        run_gate<ENC_GENERAL, CTL_NONE>(dec, op, tile, sc, base, spread, nblk, lane);
+                        run_gate<ENC_GENERAL, CTL_NONE, NB>(dec, op, tile, sc, base, spread, nblk, lane);
                     break;
             }
         }
 #pragma unroll
-        for (int k = 0; k < nblk; ++k) codes[uint64_t(base | spread[k]) * 32 + lane] = tile[k * 32 + lane];
-        if (lane < nblk) scales[mine] = sc;
+        for (int k = 0; k < nblk; ++k) codes[uint64_t(base | spread[k]) * 32 + lane] = tile[k * 32 + ml];
+        if (lane < nblk) scales[own] = sc;
     }
 }
 
@@ -982,7 +996,7 @@ cudaError_t enc_attrs(int device) {
           set(k_enc_gate_in<ENC_DIAG>, kTabBytes), set(k_enc_gate_in<ENC_DIAG1>, kTabBytes),
           set(k_enc_gate_across<ENC_GENERAL>, kTabBytes), set(k_enc_gate_across<ENC_REAL>, kTabBytes),
           set(k_enc_gate_across<ENC_DIAG>, kTabBytes), set(k_enc_gate_across<ENC_DIAG1>, kTabBytes),
-          set(k_enc_run_in<kEncRunMaxBits>, run), set(k_enc_run_in<-1>, run)})
+          set(k_enc_run_in<kEncRunMaxBits>, run), set(k_enc_run_in<-1>, run), set(k_enc_run_in<0>, run)})
         if (e != cudaSuccess) return e;
     attrs_set(configured, device);
     return cudaSuccess;
@@ -1150,14 +1164,21 @@ cudaError_t launch_enc_run(sv_state *h, const EncRunOp *d_ops, int nops, int nbi
     a.nbits = nbits;
     for (int j = 0; j < nbits; ++j) a.pos[j] = pos[j];
     uint4 *codes = static_cast<uint4 *>(h->data);
-    const unsigned block = 32 * kRunWarps;
-    const int smem = kTabBytes + kRunWarps * (512 << nbits);
     const cudaError_t e = enc_attrs(h->device);
     if (e != cudaSuccess) return e;
-    const uint64_t want = (a.ntiles + kRunWarps - 1) / kRunWarps;
-    const unsigned grid = unsigned(want < 152 ? want : 152);
+    // few tiles spread over the SMs, on CTAs of at least 8 warps (4 take 2 us
+    // longer to fill the decode table)
+    const uint64_t share = (a.ntiles + 151) / 152;
+    const unsigned warps = unsigned(share < 8 ? 8 : share > kRunWarps ? kRunWarps : share);
+    const unsigned block = 32 * warps;
+    const uint64_t want = (a.ntiles + warps - 1) / warps;
+    const uint64_t cap = 152 * (nbits == 0 ? kRunCtas0 : 1);
+    const unsigned grid = unsigned(want < cap ? want : cap);
+    const int smem = kTabBytes + (nbits == 0 ? 0 : int(warps) * (512 << nbits));
     if (nbits == kEncRunMaxBits)
         k_enc_run_in<kEncRunMaxBits><<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a);
+    else if (nbits == 0)
+        k_enc_run_in<0><<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a);
     else
         k_enc_run_in<-1><<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a);
     return cudaGetLastError();

@@ -118,6 +118,13 @@ sv_status build_enc_runs(sv_state *h, sv_plan_s *p) {
             alone += gate1_bytes(h, p->pergate[j]);
             ++j;
         }
+        // From 23 qubits on a run with fewer bits takes other ones of the block
+        // index (any will do): tiles of 16 blocks are the kernel's own form, and
+        // there are enough of them (runs of 2 or 3 SX across blocks: 27 qubits 268
+        // us instead of 352, 23 qubits 24.8 and 29.0, but 22 qubits 18.7 and 16.8).
+        // Runs inside the blocks have none and take one block per warp.
+        for (int b = 0; nb_log >= 15 && !bits.empty() && int(bits.size()) < bmax; ++b)
+            if (!std::binary_search(bits.begin(), bits.end(), b)) bits.insert(std::lower_bound(bits.begin(), bits.end(), b), b);
         if (j - i >= 2 && alone > pass_bytes) {
             PlanLaunch l{4, int(p->encruns.size()), pass_bytes};
             sv_plan_s::EncRun run{int(ops.size()), int(j - i), int(bits.size()), {0, 0, 0, 0}};

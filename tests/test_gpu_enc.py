@@ -210,3 +210,57 @@ def test_runs_across_blocks_bit_exact(S, orc, monkeypatch, n, blockq):
             rc, rs = orc.enc_run(circ, None, *orc.enc_encode(psi))
             assert np.array_equal(out[0][0], rc)
             assert np.array_equal(out[0][1].view(np.uint32), rs.view(np.uint32))
+
+
+@pytest.mark.parametrize("n,blockq", [(8, []), (9, []), (16, []), (23, []), (23, [12]), (24, [9, 20])])
+def test_runs_with_few_block_bits(S, monkeypatch, n, blockq):
+    """Runs inside single blocks (controls outside them too) and runs whose
+    tiles are made whole by block bits that no gate targets write the codes of
+    one pass per gate."""
+    circ = _mixed_on(n, [0, 1, 2, 5, 7] + blockq, 200, n)
+    if n > 8:
+        for q in (0, 3, 7):
+            circ.add("CX", n - 1, q)
+            circ.add("H", q)
+    psi = rand_c64(n, 6)
+    src = S.StateVector(n, "c64")
+    src.from_numpy(psi)
+    out = []
+    for runs in ("1", "0"):
+        monkeypatch.setenv("SV_ENC_RUNS", runs)
+        enc = S.StateVector(n, "enc2b")
+        enc.encode_from(src)
+        enc.run(circ, "pergate")
+        out.append(enc.codes())
+        enc.free()
+    assert np.array_equal(out[0][0], out[1][0])
+    assert np.array_equal(out[0][1].view(np.uint32), out[1][1].view(np.uint32))
+
+
+def test_runs_inside_blocks_do_their_work_once(S, monkeypatch):
+    """A run of gates inside the blocks exists to save passes: at 24 qubits it
+    takes no longer than one and a half times those passes (it took almost
+    three times as long when every block was computed twice)."""
+    import torch
+
+    n = 24
+    circ = C.Circuit(n)
+    for k in range(48):
+        circ.add(("H", "SX", "T", "SY")[k % 4], k % 8)
+    ms = {}
+    for runs in ("1", "0"):
+        monkeypatch.setenv("SV_ENC_RUNS", runs)
+        enc = S.StateVector(n, "enc2b")
+        p = enc.plan(circ, "pergate")
+        ms[runs] = 1e9
+        for _ in range(6):
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            ev[0].record()
+            for _ in range(3):
+                p.execute()
+            ev[1].record()
+            torch.cuda.synchronize()
+            ms[runs] = min(ms[runs], ev[0].elapsed_time(ev[1]))
+        p.free()
+        enc.free()
+    assert ms["1"] <= 1.5 * ms["0"], ms
