@@ -238,6 +238,7 @@ struct TileCacheEntry {
     int64_t gates = 0;
     std::vector<double> lane_ops;
     std::vector<int> nseg;
+    TileConfig cfg{};
 };
 std::mutex g_tile_cache_mu;
 std::unordered_map<std::string, TileCacheEntry> g_tile_cache;
@@ -257,6 +258,7 @@ struct Strategy {
     TileConfig cfg{};
     int k = 0;
     std::vector<int> pass_ctas;
+    bool by_circuit = false;  // tiled: cfg is the size's, the circuit may change it
     std::string name() const {
         if (mode == SV_MODE_TILED) {
             std::string nm = "tiled " + tile_config_name(cfg);
@@ -289,14 +291,14 @@ sv_status create_plan(sv_state *h, const char *text, const Circuit &c, const Str
     const bool tiled = st.mode == SV_MODE_TILED && h->n >= tile_m;
     std::string key;
     if (tiled && text) {
-        key = tile_cache_key(h, st.cfg, text) + "|" + pass_ctas_key(st.pass_ctas);
+        key = tile_cache_key(h, st.cfg, text) + "|" + pass_ctas_key(st.pass_ctas) + (st.by_circuit ? "|c" : "");
         std::lock_guard<std::mutex> lock(g_tile_cache_mu);
         auto it = g_tile_cache.find(key);
         if (it != g_tile_cache.end()) {
             sv_plan_s *p = new sv_plan_s;
             p->h = h;
             p->mode = st.mode;
-            p->cfg = st.cfg;
+            p->cfg = it->second.cfg;
             p->gates = it->second.gates;
             p->tfns = it->second.fns;
             p->tile_rb = it->second.rb;
@@ -334,11 +336,12 @@ sv_status create_plan(sv_state *h, const char *text, const Circuit &c, const Str
             }
         if (!s && gate_runs_fit(h->dt, h->n) && p->launches.size() >= 2) plan_gate_runs(h->dt, h->n, p->pergate, &p->gruns);
     } else {
-        s = build_tile_plan(h, c, p, st.cfg, st.pass_ctas);
+        if (st.by_circuit) p->cfg = tile_config_for(h->dt, h->n, c);
+        s = build_tile_plan(h, c, p, p->cfg, st.pass_ctas);
         if (!s && !key.empty()) {
             std::lock_guard<std::mutex> lock(g_tile_cache_mu);
             if (g_tile_cache.size() >= kTileCacheMax) g_tile_cache.clear();
-            g_tile_cache[key] = TileCacheEntry{p->tfns, p->tile_rb, p->gates, p->tile_lane_ops, p->tile_nseg};
+            g_tile_cache[key] = TileCacheEntry{p->tfns, p->tile_rb, p->gates, p->tile_lane_ops, p->tile_nseg, p->cfg};
         }
     }
     if (s) {
@@ -591,6 +594,7 @@ sv_status create_auto_plan(sv_state *h, const char *text, const Circuit &c, sv_p
     if (s == SV_ERR_OOM) {
         // no room to time: the planner's own choice
         Strategy st{h->dt == SV_ENC2B ? SV_MODE_PERGATE : SV_MODE_TILED, default_config(h), 0};
+        st.by_circuit = true;
         s = create_plan(h, text, c, st, out);
         if (!s) (*out)->tuning = report;
         return s;
@@ -634,7 +638,8 @@ extern "C++" sv_status sv::plan_create(sv_handle h, const char *text, int mode, 
     Circuit c;
     sv_status s = SV_OK;
     // a cached tiled plan needs no parse (the text is part of its key)
-    const Strategy st{mode, cfg ? *cfg : default_config(h), 0};
+    Strategy st{mode, cfg ? *cfg : default_config(h), 0};
+    st.by_circuit = !cfg;
     const bool maybe_cached = mode == SV_MODE_TILED;
     if (!maybe_cached) {
         s = parse_circuit(text, h->n, &c);
@@ -843,7 +848,7 @@ sv_status sv_plan_stats(const char *text, int n, sv_dtype dt, int compile, int64
             return SV_ERR_UNSUPPORTED;
         }
         TilePlan<float> tp;
-        s = plan_tiles<float>(c, n, tile_config_for(dt, n), &tp);
+        s = plan_tiles<float>(c, n, tile_config_for(dt, n, c), &tp);
         return s ? s : count(tp);
     }
     if (n < kTileM128) {
@@ -851,7 +856,7 @@ sv_status sv_plan_stats(const char *text, int n, sv_dtype dt, int compile, int64
         return SV_ERR_UNSUPPORTED;
     }
     TilePlan<double> tp;
-    s = plan_tiles<double>(c, n, tile_config_for(dt, n), &tp);
+    s = plan_tiles<double>(c, n, tile_config_for(dt, n, c), &tp);
     return s ? s : count(tp);
 }
 
@@ -895,7 +900,7 @@ sv_status sv_plan_pass_source(const char *text, int n, sv_dtype dt, int64_t pass
             return SV_ERR_UNSUPPORTED;
         }
         TilePlan<float> tp;
-        s = plan_tiles<float>(c, n, tile_config_for(dt, n), &tp);
+        s = plan_tiles<float>(c, n, tile_config_for(dt, n, c), &tp);
         return s ? s : emit(tp);
     }
     if (n < kTileM128) {
@@ -903,7 +908,7 @@ sv_status sv_plan_pass_source(const char *text, int n, sv_dtype dt, int64_t pass
         return SV_ERR_UNSUPPORTED;
     }
     TilePlan<double> tp;
-    s = plan_tiles<double>(c, n, tile_config_for(dt, n), &tp);
+    s = plan_tiles<double>(c, n, tile_config_for(dt, n, c), &tp);
     return s ? s : emit(tp);
 }
 

@@ -175,6 +175,8 @@ int tile_m64();
 TileConfig tile_config128();
 // The tiled mode's configuration for a state of n qubits.
 TileConfig tile_config_for(sv_dtype dt, int n);
+// The same for a circuit (sizes at which it decides).
+TileConfig tile_config_for(sv_dtype dt, int n, const Circuit &c);
 // Folder of the compiled-pass disk cache ("" when there is none).
 std::string jit_cache_dir();
 // A short text naming a configuration (plan keys, tuning reports).

@@ -1150,7 +1150,7 @@ TileConfig tile_config128() {
 // CTA.  Three waves and less of full complex64 tiles (21 and 22 qubits) leave
 // the last one part empty: there 2^11 amplitudes, 16 per thread (53.5 -> 47.4
 // and 92.5 -> 80.0 us); from 23 qubits on their additional passes cost more
-// (25-qubit Fourier transform 395 -> 567 us).
+// (25-qubit Fourier transform 395 -> 567 us).  All in replays of a graph.
 TileConfig tile_config_for(sv_dtype dt, int n) {
     const int m = n - 7;  // 2^7 tiles
     if (dt != SV_C64) {
@@ -1173,6 +1173,20 @@ TileConfig tile_config_for(sv_dtype dt, int n) {
         c.rb = 4;
     }
     return c;
+}
+
+// The same for a circuit.  At 21 and 22 qubits full tiles are faster where two
+// passes do and smaller ones need a third: the passes are light then, and a
+// launch and its traffic cost more than the last wave (22 qubits: GHZ 24.6 us
+// against 26.8, uniform 26.8 and 30.8, random of depth 2 26.8 and 28.9; depth 4,
+// three passes each, 41.1 and 32.8; depth 12, 4 passes against 5, 92.3 and 80.0).
+TileConfig tile_config_for(sv_dtype dt, int n, const Circuit &c) {
+    const TileConfig small = tile_config_for(dt, n), full = tile_config64();
+    if (dt != SV_C64 || n < 21 || n > 22 || small.m >= full.m) return small;
+    TilePlan<float> a, b;
+    const bool take = plan_tiles<float>(c, n, full, &a) == SV_OK && a.passes.size() <= 2 &&
+                      plan_tiles<float>(c, n, small, &b) == SV_OK && b.passes.size() > a.passes.size();
+    return take ? full : small;
 }
 
 std::string tile_config_name(const TileConfig &cfg) {

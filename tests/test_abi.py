@@ -193,3 +193,17 @@ def test_direct_hbm_segments_cover_whole_sectors(L):
             assert {0, 1, 2} <= lanes, (i, sorted(lanes))
             direct += 1
     assert direct >= passes  # most passes load and store directly
+
+
+@pytest.mark.parametrize("n", [21, 22])
+def test_light_circuits_keep_full_tiles(L, n):
+    """Host only: at 21 and 22 qubits a circuit that two passes of full tiles
+    can hold takes no third pass; deeper ones keep the smaller tiles (more,
+    lighter passes)."""
+    for c in (C.ghz_circuit(n), C.uniform_circuit(n), C.random_circuit(n, 2, 1), C.random_circuit(n, 1, 1)):
+        assert sv.sv_plan_stats(c, n, "c64")[1] <= 2
+    assert sv.sv_plan_stats(C.random_circuit(n, 12, 1), n, "c64")[1] >= 5
+    one = C.Circuit(n)
+    one.add("H", 0)
+    one.add("CX", 0, n - 1)
+    assert sv.sv_plan_stats(one, n, "c64")[1] == 1
