@@ -19,6 +19,7 @@
 // stream to it before and after, so work already queued on those streams is
 // ordered with the batch.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <vector>
 
@@ -53,15 +54,19 @@ void destroy_batch(sv_batch_s *b) {
     delete b;
 }
 
-// Tiles of a batch's member.  Members run side by side, so a pass of few tiles
-// need not fill the chip by itself, as tile_config_for has it do: from 17 to 22
-// qubits whole 2^13 tiles (the fewest passes) with 16 amplitudes per thread,
-// whose CTAs of 512 threads finish their tile sooner (64 members of 13 to 22
-// qubits: 1.87 ms with 32 amplitudes per thread, 1.58 with the tiles of a
-// member run alone, 1.34 so; 8 to 16 qubits: 0.121 ms with those of a member
-// run alone, 0.135 with whole tiles).
-TileConfig member_config(const sv_state *h) {
-    return h->dt == SV_C64 && h->n >= 17 && h->n <= 22 ? tile_config64(4) : tile_config_for(h->dt, h->n);
+// Tiles of a batch's members.  Members run side by side: once their passes
+// together fill the chip, a member's need not fill it alone, as
+// tile_config_for has it do, and complex64 members of 17 to 22 qubits take
+// whole 2^13 tiles (the fewest passes) with 16 amplitudes per thread, whose
+// CTAs of 512 threads finish their tile sooner.  tiles: whole tiles of all
+// members.  Up to 20 qubits the line is what the SMs hold at once (2 CTAs each;
+// with other work between executions 16 members of 17 qubits 83 us whole and 78
+// alone, 3 of 20 qubits 62 and 67, 16 of 19 qubits 154 and 163); members of 21
+// and 22 qubits fill the chip alone for longer (2 of 22 qubits 142 and 129, 4 of
+// 21 qubits 135 and 125; 8 of 21 qubits 326 and 405, 8 of 22 qubits 636 and 747).
+bool whole_tiles(const sv_state *h, double tiles) {
+    if (h->dt != SV_C64 || h->n < 17 || h->n > 22) return false;
+    return tiles > (h->n <= 20 ? 2.0 * 152.0 : 1024.0);
 }
 
 // Run every member's launches on its branch stream, forked from and joined
@@ -138,10 +143,13 @@ extern "C" sv_status sv_batch_create(const sv_handle *handles, const char *const
     }
     sv_batch_s *b = new sv_batch_s;
     sv_status s = SV_OK;
+    double tiles = 0.0;
+    for (int k = 0; k < count; ++k)
+        tiles += std::ldexp(1.0, handles[k]->n - (handles[k]->dt == SV_C64 ? kTileM64 : kTileM128));
+    const TileConfig whole = tile_config64(4);
     for (int k = 0; k < count && s == SV_OK; ++k) {
         sv_plan p = nullptr;
-        const TileConfig cfg = member_config(handles[k]);
-        s = plan_create(handles[k], texts[k], SV_MODE_TILED, &cfg, &p);
+        s = plan_create(handles[k], texts[k], SV_MODE_TILED, whole_tiles(handles[k], tiles) ? &whole : nullptr, &p);
         if (s) break;
         b->handles.push_back(handles[k]);
         b->plans.push_back(p);

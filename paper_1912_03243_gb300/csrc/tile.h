@@ -173,6 +173,8 @@ TileConfig tile_config64(int rb = 0, int ctas = 0, int direct = -1, int prefetch
 // Tile bits of complex64 passes (SV_TILE_M overrides: 12 or 13).
 int tile_m64();
 TileConfig tile_config128();
+// Whether the environment names a configuration (which then is everyone's).
+bool tile_config_set();
 // The tiled mode's configuration for a state of n qubits.
 TileConfig tile_config_for(sv_dtype dt, int n);
 // The same for a circuit (sizes at which it decides).

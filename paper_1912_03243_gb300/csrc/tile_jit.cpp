@@ -1141,6 +1141,8 @@ TileConfig tile_config128() {
     return c;
 }
 
+bool tile_config_set() { return std::getenv("SV_TILE_M") || std::getenv("SV_TILE_RB") || std::getenv("SV_TILE_CTAS"); }
+
 // Tiles of a state of n qubits.  A pass of few tiles takes as long as one CTA
 // takes for its tile, so a small state is cut into about 128 tiles, one per SM:
 // complex64 down to 2^11 amplitudes (random circuits of depth 12: 14 qubits
@@ -1163,7 +1165,7 @@ TileConfig tile_config_for(sv_dtype dt, int n) {
         return c;
     }
     TileConfig c = tile_config64();
-    if (std::getenv("SV_TILE_M") || std::getenv("SV_TILE_RB") || std::getenv("SV_TILE_CTAS")) return c;
+    if (tile_config_set()) return c;
     if (m < c.m) {
         c.m = std::max(m, 11);
         c.rb = c.m - 8;

@@ -67,3 +67,23 @@ def test_batch_rejects_shared_states_and_codes(S):
         S.Batch([a, e], [c, c])
     with pytest.raises(S.SVError):  # a qubit outside member 0's state
         S.Batch([a, b], [C.random_circuit(14, 2, 1), C.random_circuit(14, 2, 1)])
+
+
+@pytest.mark.parametrize("n,count,env", [(17, 2, None), (22, 1, None)])
+def test_members_take_the_tiles_of_a_state_alone(S, monkeypatch, tmp_path, n, count, env):
+    """Members that do not fill the chip together are tiled as each would be
+    alone:
+    a batch of circuits that are planned already compiles no further pass."""
+    if env:
+        monkeypatch.setenv("SV_TILE_RB", env)
+    monkeypatch.setenv("SV_JIT_CACHE", str(tmp_path))
+    circs = [C.random_circuit(n, 5, 900 + n + k) for k in range(count)]
+    states = [S.StateVector(n, "c64") for _ in circs]
+    for s, c in zip(states, circs):
+        s.plan(c, "tiled").free()
+    alone = sorted(f.name for f in tmp_path.iterdir())
+    assert alone
+    b = S.Batch(states, circs)
+    b.execute()
+    assert sorted(f.name for f in tmp_path.iterdir()) == alone
+    b.free()
