@@ -65,7 +65,7 @@ void destroy_batch(sv_batch_s *b) {
 // and 22 qubits fill the chip alone for longer (2 of 22 qubits 142 and 129, 4 of
 // 21 qubits 135 and 125; 8 of 21 qubits 326 and 405, 8 of 22 qubits 636 and 747).
 bool whole_tiles(const sv_state *h, double tiles) {
-    if (h->dt != SV_C64 || h->n < 17 || h->n > 22) return false;
+    if (h->dt != SV_C64 || h->n < 17 || h->n > 22 || tile_config_set()) return false;
     return tiles > (h->n <= 20 ? 2.0 * 152.0 : 1024.0);
 }
 

@@ -69,10 +69,10 @@ def test_batch_rejects_shared_states_and_codes(S):
         S.Batch([a, b], [C.random_circuit(14, 2, 1), C.random_circuit(14, 2, 1)])
 
 
-@pytest.mark.parametrize("n,count,env", [(17, 2, None), (22, 1, None)])
+@pytest.mark.parametrize("n,count,env", [(17, 2, None), (22, 1, None), (20, 3, "5")])
 def test_members_take_the_tiles_of_a_state_alone(S, monkeypatch, tmp_path, n, count, env):
     """Members that do not fill the chip together are tiled as each would be
-    alone:
+    alone, and so is every member where the environment names a configuration:
     a batch of circuits that are planned already compiles no further pass."""
     if env:
         monkeypatch.setenv("SV_TILE_RB", env)
