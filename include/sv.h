@@ -174,20 +174,28 @@ sv_status sv_run_circuit(sv_handle h, const char *text, int mode);
 sv_status sv_plan_create(sv_handle h, const char *text, int mode, sv_plan *out);
 /* Execute a plan on the handle's stream (asynchronous).  The first execution
  * launches the kernels one by one; the second captures them into a CUDA graph
- * on a stream the plan owns, and every later one replays that graph; the
- * plan's stream waits for the handle's stream before the graph and the
- * handle's stream waits for the graph after it, so the order of work on the
- * handle's stream is unchanged.  Plans with CUDA-core dense blocks (host
+ * on a stream the plan owns, and every later one replays that graph on the
+ * handle's stream.  Plans with CUDA-core dense blocks (host
  * matrix copies per launch), single-launch plans and runs with SV_GRAPH=0
- * always launch directly; so does a plan whose capture failed. */
+ * always launch directly; so does a plan whose capture failed.
+ * Plans of two or more per-gate updates on a small SV_C64 or SV_C128 state
+ * (2 to 23 qubits, SV_C128 2 to 22) are listed gate by gate but executed in
+ * fewer launches of several gates each: the statistics and the timing hook
+ * below describe the list, not those launches. */
 sv_status sv_plan_execute(sv_plan p);
 /* *out = 1 if the plan's executions now replay a CUDA graph, else 0. */
 sv_status sv_plan_uses_graph(sv_plan p, int *out);
-/* Statistics of a plan: number of gates, HBM passes (kernel launches) and
- * the algorithmic bytes all passes move. */
+/* Statistics of a plan: number of gates, HBM passes (entries of its launch
+ * list) and the algorithmic bytes all passes move.  The list is what
+ * sv_plan_execute launches, except for per-gate plans of small states (see
+ * there): theirs has one entry per gate, and an execution makes fewer
+ * launches that move fewer bytes. */
 sv_status sv_plan_info(sv_plan p, int64_t *gates, int64_t *passes, double *bytes);
-/* Per-launch timing hook: execute the plan and record event[i] (caller-
- * created cudaEvent_t) before launch i and event[passes] after the last. */
+/* Per-launch timing hook: execute the plan's launch list and record event[i]
+ * (caller-created cudaEvent_t) before launch i and event[passes] after the
+ * last.  A per-gate plan of a small state runs one launch per gate here (the
+ * times of its gates alone, not shares of sv_plan_execute's time), and rounds
+ * in another order than sv_plan_execute does. */
 sv_status sv_plan_execute_timed(sv_plan p, void *const *events, int64_t n_events);
 /* The autotuner's record of an SV_MODE_AUTO plan as JSON text: each
  * candidate strategy with its measured ms per execution and the chosen one
@@ -197,8 +205,9 @@ sv_status sv_plan_execute_timed(sv_plan p, void *const *events, int64_t n_events
  * NUL-terminated, may be NULL), *len = the full length. */
 sv_status sv_plan_tuning(sv_plan p, char *buf, size_t cap, size_t *len);
 sv_status sv_plan_free(sv_plan p);
-/* Launch i of a plan (0 <= i < passes): the name of the kernel it runs and
- * the algorithmic bytes it moves.  *kernel points to a static string. */
+/* Entry i of a plan's launch list (0 <= i < passes): the name of the kernel
+ * that the timing hook runs for it and the algorithmic bytes it moves.
+ * *kernel points to a static string. */
 sv_status sv_plan_launch_info(sv_plan p, int64_t i, const char **kernel, double *bytes);
 
 /* Launch i of a plan: for a compiled tile pass, the FP32 lane operations per
@@ -265,8 +274,9 @@ sv_status sv_fused_tc_layout(int n, int k, const int *qubits, char *kernel, size
 sv_status sv_batch_create(const sv_handle *handles, const char *const *texts, int count, sv_batch *out);
 /* Run every member's circuit once on its current state (asynchronous). */
 sv_status sv_batch_execute(sv_batch b);
-/* Gates of all members, their launches per execution, algorithmic bytes,
- * and whether executions now replay the graph (any pointer may be NULL). */
+/* Gates of all members, the entries of their launch lists and the
+ * algorithmic bytes of those (as sv_plan_info), and whether executions now
+ * replay the graph (any pointer may be NULL). */
 sv_status sv_batch_info(sv_batch b, int64_t *gates, int64_t *launches, double *bytes, int *uses_graph);
 sv_status sv_batch_free(sv_batch b);
 /* Create, execute once and free. */

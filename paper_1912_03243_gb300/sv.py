@@ -320,7 +320,9 @@ class Plan:
         return bool(v.value)
 
     def execute_timed(self, events) -> None:
-        """events: list of torch.cuda.Event (passes + 1), recorded around each launch."""
+        """Run the plan's launch list with events (a list of torch.cuda.Event,
+        passes + 1) recorded around each entry: per-gate plans of small states
+        run gate by gate here, several gates per launch in execute."""
         arr = (_vp * len(events))(*[_vp(e.cuda_event) for e in events])
         _check(lib().sv_plan_execute_timed(self.handle, arr, len(events)), "sv_plan_execute_timed")
 
@@ -346,7 +348,8 @@ class Plan:
         return out
 
     def launch_info(self):
-        """[(kernel name, algorithmic bytes)] for every launch of one execution."""
+        """[(kernel name, algorithmic bytes)] for every entry of the launch list
+        (what execute_timed runs; see there)."""
         out = []
         name, b = ctypes.c_char_p(), ctypes.c_double()
         for i in range(self.passes):

@@ -333,3 +333,35 @@ def test_unnormalised_states(S, orc, dtype, n, e):
         p.execute()
         check(dtype, s.to_numpy().astype(np.complex128) * 2.0**-e, ref)
     p.free()
+
+
+@pytest.mark.parametrize("dtype,n", [("c64", 9), ("c64", 16), ("c64", 23), ("c64", 24), ("c128", 8), ("c128", 18), ("c128", 23)])
+def test_statistics_describe_the_launch_list(S, dtype, n):
+    """A per-gate plan's statistics and timing hook describe its list of one
+    entry per gate, at every size, however many gates its launches take: the
+    entries' bytes add up to the plan's and are those of the gates planned
+    alone, and the hook wants one event more than entries."""
+    import torch
+
+    c = C.random_circuit(n, 2, 5)
+    s = S.StateVector(n, dtype)
+    p = s.plan(c, "pergate")
+    info = p.launch_info()
+    assert p.passes == p.gates == len(info) == len(c)
+    assert sum(b for _, b in info) == pytest.approx(p.bytes, rel=1e-12)
+    for k in (0, len(c) - 1):
+        one = C.Circuit(n)
+        one.gates = [c.gates[k]]
+        q = s.plan(one, "pergate")
+        assert q.launch_info() == [info[k]]
+        q.free()
+    with pytest.raises(S.SVError):
+        p.execute_timed([torch.cuda.Event(enable_timing=True)])
+    p.free()
+
+
+@pytest.mark.parametrize("dtype,n", [("c64", 11), ("c64", 17), ("c128", 9), ("c128", 18), ("c128", 19)])
+def test_runs_of_gates_at_the_borders(S, orc, dtype, n):
+    """The smallest states that run several gates per launch over many CTAs,
+    and both sides of the size at which a thread takes more qubits."""
+    test_runs_of_gates(S, orc, dtype, n)
