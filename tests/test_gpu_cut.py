@@ -305,3 +305,86 @@ def test_fits_where_the_results_fit(S):
         torch.cuda.empty_cache()
     assert s0 == s1 == 8
     close(got, ref)
+
+
+def _cut_first(rows, cols, depth, seed, qa, qb):
+    """A grid circuit after a cut gate on |+>|+>: the first fork precedes every
+    other gate of both partitions but these."""
+    g = C.grid_circuit(rows, cols, depth, seed)
+    c = C.Circuit(g.n)
+    for q in (qa, qb):
+        c.add("H", q)
+    c.add("CZ", qa, qb)
+    c.gates += g.gates
+    return c
+
+
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("first", [False, True])
+def test_parts_of_partitions_above_a_tile(S, monkeypatch, form, first):
+    """Branch parts where a partition has more qubits than a tile (4x7 grid,
+    14 + 14 qubits: forks inside the passes, fixed branch bits as launch
+    parameters): every part equals the fully batched form's, and their sum the
+    amplitudes of the 28-qubit state."""
+    c = _cut_first(4, 7, 6, 2, 0, 27) if first else C.grid_circuit(4, 7, 6, 2)
+    mask = C.grid_partition_mask(4, 7, 2)
+    z = C.random_bitstrings(1500, 28, 5)
+    s = S.StateVector(28, "c64")
+    s.run(c, "tiled")
+    full = s.amplitudes(z)
+    s.free()
+    whole, cuts = S.sv_cut_amplitudes(c, 28, mask, z, form=form)
+    assert cuts == 7 + first
+    close(whole, full)
+    for log2 in (1, 3):
+        total = 0
+        for k in range(1 << log2):
+            part, _ = S.sv_cut_amplitudes_part(c, 28, mask, z, k, log2, form=form)
+            monkeypatch.setenv("SV_CUT_PREFIX", "0")
+            ref, _ = S.sv_cut_amplitudes_part(c, 28, mask, z, k, log2, form=form)
+            monkeypatch.delenv("SV_CUT_PREFIX")
+            assert np.max(np.abs(part - ref)) <= 1e-5 * np.max(np.abs(full))
+            total = total + part
+        close(total, full)
+    parts, _ = S.sv_cut_amplitudes_parts(c, 28, mask, z, 3, range(8), form=form)
+    close(parts, full)
+
+
+@pytest.mark.parametrize("form", [0, 1])
+def test_three_partitions_above_a_tile(S, monkeypatch, form):
+    """Three partitions of 14 qubits (6x7 grid; the middle one holds the branch
+    bits of both borders), whole and in branch parts, against the fully batched
+    form."""
+    c = C.grid_circuit(6, 7, 5, 4)
+    part_of = [q // 14 for q in range(42)]
+    z = C.random_bitstrings(700, 42, 6)
+    lists = [(0, [0]), (2, [0, 1, 2, 3]), (2, [2]), (3, [1, 4, 6])]
+    got = [S.sv_cut_amplitudes_multi_parts(c, 42, part_of, z, log2, parts, form=form) for log2, parts in lists]
+    monkeypatch.setenv("SV_CUT_PREFIX", "0")
+    ref = [S.sv_cut_amplitudes_multi_parts(c, 42, part_of, z, log2, parts, form=form) for log2, parts in lists]
+    scale = np.max(np.abs(ref[0][0]))
+    assert scale > 0 and np.max(np.abs(got[1][0] - got[0][0])) <= 1e-5 * scale
+    for (a, sa), (b, sb) in zip(got, ref):
+        assert sa == sb == 8
+        assert np.max(np.abs(a - b)) <= 1e-5 * scale
+
+
+@pytest.mark.parametrize("form,m", [(0, 1500), (1, 900), (0, 3000)])
+def test_chunked_parts(S, monkeypatch, form, m):
+    """Branch parts of partitions whose last stage runs in chunks (6x8 grid, one
+    branch bit fixed: 2^31 batched amplitudes), on the wanted tiles where the
+    strings are fewer than the tiles, against the fully batched form."""
+    import torch
+
+    if torch.cuda.mem_get_info()[0] < (40 << 30):
+        pytest.skip("not enough device memory")
+    c = C.grid_circuit(6, 8, 8, 3)
+    mask = C.grid_partition_mask(6, 8, 3)
+    z = C.random_bitstrings(m, 48, 12)
+    got = [S.sv_cut_amplitudes_part(c, 48, mask, z, k, 1, form=form)[0] for k in (0, 1)]
+    monkeypatch.setenv("SV_CUT_PREFIX", "0")
+    ref = [S.sv_cut_amplitudes_part(c, 48, mask, z, k, 1, form=form)[0] for k in (0, 1)]
+    scale = np.max(np.abs(ref[0] + ref[1]))
+    assert scale > 0
+    for a, b in zip(got, ref):
+        assert np.max(np.abs(a - b)) <= 1e-5 * max(scale, np.max(np.abs(b)))
