@@ -632,6 +632,7 @@ constexpr R kRunScale = R(1) / R(1 << kRunOwed<R> / 2);
 template <typename R>
 struct RunArgs {
     uint32_t q[kRunSlots];   // the registers' qubits, ascending
+    uint32_t far[kRunSlots], rank[kRunSlots];  // (LOW) a warp's other qubits than 0..4; places of q among its qubits
     int nops, odd, quarter;  // factor paid at the end: (1 + i)^odd i^quarter m
     R m;
     GateRunHead op[kRunMaxOps];
@@ -767,13 +768,45 @@ struct Amp2<double> {
 
 constexpr int kRunThreads = 64;  // small CTAs: even work per SM (20 qubits: 1024 CTAs, 6.7 per SM)
 
-template <typename R, int S>
+template <typename R, int S, bool LOW>
 __global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *__restrict__ psi,
                                                           const __grid_constant__ RunArgs<R> a) {
+    using V = typename Amp2<R>::T;
     uint32_t i = blockIdx.x * kRunThreads + threadIdx.x;
 #pragma unroll
     for (int k = 0; k < S; ++k) i += i & ~((1u << a.q[k]) - 1u);  // a zero bit inserted at q[k]
     C2<R> x[1 << S];
+    // LOW: a warp's amplitudes (its S + 5 qubits always contain 0..4) are moved
+    // in rows of 32 consecutive ones, and change hands in shared memory.  A
+    // thread that holds several of qubits 0..3 itself makes every 8-byte access
+    // of its warp touch up to 32 lines instead of 2 (complex64, 4 H: on qubits
+    // 0..3 at 23 qubits 67.8 us direct, 23.3 by rows, 16.4 on high qubits; on 0, 1
+    // and two high ones 36.9 and 23.5; at 20 qubits 12.3 and 6.3).  With one low
+    // qubit, or two but 0 and 1, rows gain nothing (23 qubits 18.6 and 22.9, 20.6
+    // and 26.8), nor for states up to 17 qubits.
+    __shared__ V rows[LOW ? kRunThreads << S : 1];
+    const uint32_t lane = threadIdx.x & 31u;
+    V *const warp = rows + (LOW ? (threadIdx.x & ~31u) << S : 0u);
+    auto row = [&](int v) {
+        uint32_t j = __shfl_sync(0xffffffffu, i, 0) | lane;
+#pragma unroll
+        for (int k = 0; k < S; ++k)
+            if (v >> k & 1) j |= 1u << a.far[k];
+        return psi + j;
+    };
+    uint32_t own = lane;  // this thread's amplitudes in the warp's order
+    if constexpr (LOW) {
+#pragma unroll
+        for (int k = 0; k < S; ++k) own += own & ~((1u << a.rank[k]) - 1u);
+        own = small_pos<R>(own);
+    }
+    auto held = [&](int v) {
+        uint32_t j = own;
+#pragma unroll
+        for (int k = 0; k < S; ++k)
+            if (v >> k & 1) j ^= small_pos<R>(1u << a.rank[k]);
+        return warp + j;
+    };
     auto at = [&](int v) {
         uint32_t j = i;
 #pragma unroll
@@ -781,9 +814,14 @@ __global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *_
             if (v >> k & 1) j |= 1u << a.q[k];
         return psi + j;
     };
+    if constexpr (LOW) {
+#pragma unroll
+        for (int v = 0; v < (1 << S); ++v) warp[small_pos<R>(uint32_t(v) << 5 | lane)] = *row(v);
+        __syncwarp();
+    }
 #pragma unroll
     for (int v = 0; v < (1 << S); ++v) {
-        const auto z = *at(v);
+        const V z = LOW ? *held(v) : *at(v);
         x[v].re = z.x;
         x[v].im = z.y;
     }
@@ -808,10 +846,15 @@ __global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *_
     if (a.quarter & 2) run_phase<P_NEG, S>(x, 0u, R(0), R(0));
 #pragma unroll
     for (int v = 0; v < (1 << S); ++v) {
-        typename Amp2<R>::T z;
+        V z;
         z.x = x[v].re;
         z.y = x[v].im;
-        *at(v) = z;
+        *(LOW ? held(v) : at(v)) = z;
+    }
+    if constexpr (LOW) {
+        __syncwarp();
+#pragma unroll
+        for (int v = 0; v < (1 << S); ++v) *row(v) = warp[small_pos<R>(uint32_t(v) << 5 | lane)];
     }
 }
 
@@ -826,8 +869,28 @@ cudaError_t gate_runs_impl(sv_state *h, const GateRuns &p) {
         a.odd = r.odd;
         a.quarter = r.quarter;
         a.m = R(r.m);
-        k_gate_run<R, S><<<1u << (h->n - S - 6), kRunThreads, 0, h->stream>>>(
-            static_cast<typename Amp2<R>::T *>(h->data), a);
+        auto *psi = static_cast<typename Amp2<R>::T *>(h->data);
+        const unsigned grid = 1u << (h->n - S - 6);
+        bool rows = false;
+        if constexpr (sizeof(R) == 4 && S == 4) {
+            rows = r.q[1] == 1 || r.q[2] < 4;
+            if (rows) {
+                // the warp's qubits, ascending: the registers' and the lowest 5 others
+                int all[S + 5], na = 0, lanes = 0;
+                for (int q = 0; na < S + 5; ++q) {
+                    const bool reg = std::find(r.q, r.q + S, q) != r.q + S;
+                    if (!reg && lanes == 5) continue;
+                    lanes += !reg;
+                    all[na++] = q;
+                }
+                for (int k = 0; k < S; ++k) {
+                    a.far[k] = uint32_t(all[5 + k]);
+                    a.rank[k] = uint32_t(std::find(all, all + S + 5, r.q[k]) - all);
+                }
+                k_gate_run<R, S, true><<<grid, kRunThreads, 0, h->stream>>>(psi, a);
+            }
+        }
+        if (!rows) k_gate_run<R, S, false><<<grid, kRunThreads, 0, h->stream>>>(psi, a);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }

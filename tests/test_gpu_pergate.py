@@ -365,3 +365,60 @@ def test_runs_of_gates_at_the_borders(S, orc, dtype, n):
     """The smallest states that run several gates per launch over many CTAs,
     and both sides of the size at which a thread takes more qubits."""
     test_runs_of_gates(S, orc, dtype, n)
+
+
+@pytest.mark.parametrize("n", [18, 21])
+def test_runs_on_low_qubits(S, orc, n):
+    """Runs whose threads hold several of the lowest qubits move their
+    amplitudes in rows through shared memory: every combination of two to four
+    of qubits 0..5 with high ones, controls in all places, against the oracle."""
+    import itertools
+
+    rng = np.random.default_rng(n)
+    psi = C.random_state(n, 12).astype(np.complex64).astype(np.complex128)
+    s = S.StateVector(n, "c64")
+    for k in (2, 3, 4):
+        for low in itertools.combinations(range(6), k):
+            if n > 18 and (sum(low) + k) % 4:
+                continue
+            regs = list(low) + [n - 1, 9][: 4 - k]
+            c = C.Circuit(n)
+            for q in regs:  # (the first gates choose the run's qubits)
+                c.add(str(rng.choice(["H", "SX", "SYDG"])), q)
+            for q in regs:
+                ctl = int(rng.choice([x for x in range(n) if x != q]))
+                c.add("T", q)
+                c.add("CX", ctl, q)
+                c.add("CP", q, (q + 5) % n, 0.3 + q)
+            ref = orc.run(c, psi=psi)
+            p = s.plan(c, "pergate")
+            s.from_numpy(psi)
+            p.execute()
+            check("c64", s.to_numpy(), ref)
+            p.free()
+
+
+def test_runs_on_low_qubits_are_coalesced(S):
+    """Four H on the lowest qubits of a 23-qubit state take no more than two and
+    a half times four on the highest (more than four times when every access
+    touched a line of its own)."""
+    import torch
+
+    n, us = 23, {}
+    s = S.StateVector(n, "c64")
+    for name, qs in (("low", range(4)), ("high", range(n - 4, n))):
+        c = C.Circuit(n)
+        for q in qs:
+            c.add("H", q)
+        p = s.plan(c, "pergate")
+        us[name] = 1e9
+        for _ in range(8):
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            ev[0].record()
+            for _ in range(10):
+                p.execute()
+            ev[1].record()
+            torch.cuda.synchronize()
+            us[name] = min(us[name], ev[0].elapsed_time(ev[1]) * 100)
+        p.free()
+    assert us["low"] <= 2.5 * us["high"], us
