@@ -14,6 +14,7 @@
 // amplitudes they change.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "sv_internal.h"
 
@@ -632,12 +633,17 @@ constexpr R kRunScale = R(1) / R(1 << kRunOwed<R> / 2);
 template <typename R>
 struct RunArgs {
     uint32_t q[kRunSlots];   // the registers' qubits, ascending
-    uint32_t far[kRunSlots], rank[kRunSlots];  // (LOW) a warp's other qubits than 0..4; places of q among its qubits
     int nops, odd, quarter;  // factor paid at the end: (1 + i)^odd i^quarter m
     R m;
     GateRunHead op[kRunMaxOps];
     R u[8 * kRunMaxOps];
 };
+
+// A warp's qubits other than 0..4, and the places of the registers' among all.
+struct RunRows {
+    uint32_t far[kRunSlots], rank[kRunSlots];
+};
+struct NoRows {};
 
 // Without their factors: H (a + b, a - b), SX (a - i b, b - i a), SY (a - b,
 // a + b) and the adjoints of the last two.
@@ -736,15 +742,15 @@ __device__ __forceinline__ void run_gate(C2<R> (&x)[1 << S], const GateRunHead &
     if (op.kind >= R_NEG) {
         if (op.kind == R_NEG) run_phase<P_NEG, S>(x, op.rmask, R(0), R(0));
         else if (op.kind == R_PHASE) run_phase_general<S>(x, op.rmask, u[0], u[1]);
-        else if (op.kind == R_SCALE) {
+        else if (op.arg == 1) run_phase<P_I, S>(x, op.rmask, R(0), R(0));
+        else if (op.arg == 3) run_phase<P_MI, S>(x, op.rmask, R(0), R(0));
+        else {  // R_SCALE
 #pragma unroll
             for (int v = 0; v < (1 << S); ++v) {
                 x[v].re *= kRunScale<R>;
                 x[v].im *= kRunScale<R>;
             }
         }
-        else if (op.arg == 1) run_phase<P_I, S>(x, op.rmask, R(0), R(0));
-        else run_phase<P_MI, S>(x, op.rmask, R(0), R(0));
         return;
     }
     switch (op.slot) {
@@ -770,7 +776,8 @@ constexpr int kRunThreads = 64;  // small CTAs: even work per SM (20 qubits: 102
 
 template <typename R, int S, bool LOW>
 __global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *__restrict__ psi,
-                                                          const __grid_constant__ RunArgs<R> a) {
+                                                          const __grid_constant__ RunArgs<R> a,
+                                                          const __grid_constant__ std::conditional_t<LOW, RunRows, NoRows> w) {
     using V = typename Amp2<R>::T;
     uint32_t i = blockIdx.x * kRunThreads + threadIdx.x;
 #pragma unroll
@@ -787,24 +794,24 @@ __global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *_
     __shared__ V rows[LOW ? kRunThreads << S : 1];
     const uint32_t lane = threadIdx.x & 31u;
     V *const warp = rows + (LOW ? (threadIdx.x & ~31u) << S : 0u);
-    auto row = [&](int v) {
+    [[maybe_unused]] auto row = [&](int v) {
         uint32_t j = __shfl_sync(0xffffffffu, i, 0) | lane;
 #pragma unroll
         for (int k = 0; k < S; ++k)
-            if (v >> k & 1) j |= 1u << a.far[k];
+            if constexpr (LOW) j |= (v >> k & 1) << w.far[k];
         return psi + j;
     };
     uint32_t own = lane;  // this thread's amplitudes in the warp's order
     if constexpr (LOW) {
 #pragma unroll
-        for (int k = 0; k < S; ++k) own += own & ~((1u << a.rank[k]) - 1u);
+        for (int k = 0; k < S; ++k) own += own & ~((1u << w.rank[k]) - 1u);
         own = small_pos<R>(own);
     }
-    auto held = [&](int v) {
+    [[maybe_unused]] auto held = [&](int v) {
         uint32_t j = own;
 #pragma unroll
         for (int k = 0; k < S; ++k)
-            if (v >> k & 1) j ^= small_pos<R>(1u << a.rank[k]);
+            if constexpr (LOW) j ^= v >> k & 1 ? small_pos<R>(1u << w.rank[k]) : 0u;
         return warp + j;
     };
     auto at = [&](int v) {
@@ -821,7 +828,9 @@ __global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *_
     }
 #pragma unroll
     for (int v = 0; v < (1 << S); ++v) {
-        const V z = LOW ? *held(v) : *at(v);
+        V z;
+        if constexpr (LOW) z = *held(v);
+        else z = *at(v);
         x[v].re = z.x;
         x[v].im = z.y;
     }
@@ -849,7 +858,8 @@ __global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *_
         V z;
         z.x = x[v].re;
         z.y = x[v].im;
-        *(LOW ? held(v) : at(v)) = z;
+        if constexpr (LOW) *held(v) = z;
+        else *at(v) = z;
     }
     if constexpr (LOW) {
         __syncwarp();
@@ -873,6 +883,7 @@ cudaError_t gate_runs_impl(sv_state *h, const GateRuns &p) {
         const unsigned grid = 1u << (h->n - S - 6);
         bool rows = false;
         if constexpr (sizeof(R) == 4 && S == 4) {
+            RunRows w;
             rows = r.q[1] == 1 || r.q[2] < 4;
             if (rows) {
                 // the warp's qubits, ascending: the registers' and the lowest 5 others
@@ -884,13 +895,13 @@ cudaError_t gate_runs_impl(sv_state *h, const GateRuns &p) {
                     all[na++] = q;
                 }
                 for (int k = 0; k < S; ++k) {
-                    a.far[k] = uint32_t(all[5 + k]);
-                    a.rank[k] = uint32_t(std::find(all, all + S + 5, r.q[k]) - all);
+                    w.far[k] = uint32_t(all[5 + k]);
+                    w.rank[k] = uint32_t(std::find(all, all + S + 5, r.q[k]) - all);
                 }
-                k_gate_run<R, S, true><<<grid, kRunThreads, 0, h->stream>>>(psi, a);
+                k_gate_run<R, S, true><<<grid, kRunThreads, 0, h->stream>>>(psi, a, w);
             }
         }
-        if (!rows) k_gate_run<R, S, false><<<grid, kRunThreads, 0, h->stream>>>(psi, a);
+        if (!rows) k_gate_run<R, S, false><<<grid, kRunThreads, 0, h->stream>>>(psi, a, NoRows{});
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
