@@ -869,8 +869,13 @@ __global__ void __launch_bounds__(kRunThreads) k_gate_run(typename Amp2<R>::T *_
 }
 
 template <typename R, int S>
-cudaError_t gate_runs_impl(sv_state *h, const GateRuns &p) {
+cudaError_t gate_runs_impl(sv_state *h, const GateRuns &p, const std::vector<Gate1> &g) {
     for (const GateRun &r : p.runs) {
+        for (int i : r.alone) {
+            const cudaError_t e = launch_gate1(h, g[size_t(i)]);
+            if (e != cudaSuccess) return e;
+        }
+        if (r.count == 0) continue;
         RunArgs<R> a;
         for (int k = 0; k < S; ++k) a.q[k] = uint32_t(r.q[k]);
         a.nops = r.count;
@@ -1050,12 +1055,45 @@ bool gate_runs_fit(sv_dtype dt, int n) {
     return dt != SV_ENC2B && n > small_run_max_n(dt) && n <= (dt == SV_C64 ? 23 : 22);
 }
 
+// Time of a gate in a launch of its own, and of a run of gates, in us: a
+// launch, the bytes over L2 and in complex128 the FP64 operations (a run's
+// FP64 work overlaps half of its traffic).  Of the diagonal gates a launch
+// visits only the amplitudes that change; a run computes where a lane of the
+// warp has the condition met (lanes: the state's qubits inside a warp).
+double launch_us(sv_dtype dt, int n, const Gate1 &g, int kind) {
+    const double amps = std::ldexp(1.0, n);
+    const int first = dt == SV_C64 ? 1 : 0;  // (qubit 0 lies inside complex64's vectors)
+    double part = 1.0;
+    if (g.control >= first) part /= 2;
+    if (is_phase(g) && g.target >= first) part /= 2;
+    const double ops = kind == R_PHASE ? 4 : kind == R_GENERAL ? 8 : kind == R_HAD ? 3 : kind <= R_SYD ? 5 : 0;
+    const double fp64 = dt == SV_C128 ? part * amps * ops / 0.52e6 : 0.0;
+    return 1.6 + std::max(part * amps * (dt == SV_C64 ? 16 : 32) / 12e6, fp64);
+}
+double run_us(sv_dtype dt, int n, const GateRunHead *op, int count, uint32_t lanes) {
+    // (complex64 of 23 qubits, half of L2, runs at 11 TB/s)
+    const double amps = std::ldexp(1.0, n), l2 = amps * (dt == SV_C64 ? 16 : 32) / (dt == SV_C64 && n > 22 ? 11e6 : 15e6);
+    double fp64 = 0.0;
+    for (int k = 0; k < count && dt == SV_C128; ++k) {
+        const int kind = op[k].kind;
+        const int conds = __builtin_popcount(op[k].imask & ~lanes) + (kind == R_PHASE ? __builtin_popcount(op[k].rmask) : 0);
+        const double ops = kind == R_PHASE ? 4 : kind == R_GENERAL ? 8 : kind <= R_SYD || kind == R_SCALE ? 2 : 0;
+        fp64 += std::ldexp(ops, -conds) * amps / 0.52e6 + (kind == R_PHASE ? 0.8 : 0.0);  // (0.8: its branches)
+    }
+    return 2.1 + std::max(l2, l2 / 2 + fp64);
+}
+
 // Runs of gates for k_gate_run.  A run's register qubits are the targets of
 // the first gates that can be applied next (at most `slots` distinct ones);
 // then every gate that commutes with all the skipped gates before it joins if
 // its target is one of them.  A diagonal gate that costs arithmetic waits for
 // a run that holds one of its qubits (on half of the registers, not of the
 // lanes) until no other gate is left; sign flips and quarter turns join at once.
+// A run that its gates beat in launches of their own by a seventh is left to
+// them: a few diagonal gates on a large state, which visit a quarter of it each
+// (23 qubits complex64, two CZ 14.4 us in a run and 12.9 so; 22 qubits
+// complex128, 21 controlled phases on neighbours 294 and 199, 20 qubits 94 and 66;
+// states below 8 MiB are all launches: 15 qubits, two phases 4.2 and 6.2).
 void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *out) {
     constexpr size_t kWindow = 1024;  // gates looked at ahead of the first unplaced one
     // Register qubits.  A small complex128 state is bound by the FP64 pipes of
@@ -1112,6 +1150,9 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
         GateRun r;
         r.first = out->ops.size();
         r.ufirst = out->u.size();
+        const int eighths0 = eighths, halves0 = halves;
+        std::vector<int> taken;
+        double alone = 0.0;
         for (int round = 0; round < 2; ++round) {  // 0: choose the qubits, 1: take the gates
             uint64_t diag = 0, any = 0;            // qubits on which a skipped gate is diagonal / is not
             const bool only_phases = qs == 0;      // (of round 1)
@@ -1145,6 +1186,8 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
                 }
                 if (round == 0) continue;
                 placed[i] = 1;
+                taken.push_back(int(i));
+                alone += launch_us(dt, n, g[i], base[i].kind);
                 ++r.count;
                 out->ops.push_back(base[i]);
                 GateRunHead &o = out->ops.back();
@@ -1178,7 +1221,22 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
         }
         r.ucount = int(out->u.size() - r.ufirst);
         while (start < g.size() && placed[start]) ++start;
-        if (start == g.size()) {  // the rest of the factor
+        uint32_t lanes = 0;  // the five lowest qubits outside the registers
+        for (int q = 0; __builtin_popcount(lanes) < 5; ++q)
+            if (!(qs >> q & 1)) lanes |= 1u << q;
+        const bool last = start == g.size(), big = n >= (dt == SV_C64 ? 20 : 19);
+        if (big && !(last && (halves0 || eighths0 & 7)) &&
+            alone < 0.85 * run_us(dt, n, &out->ops[r.first], r.count, lanes)) {
+            out->ops.resize(r.first);
+            out->u.resize(r.ufirst);
+            eighths = eighths0;
+            halves = halves0;
+            r.count = r.ucount = 0;
+            r.alone = std::move(taken);
+            out->runs.push_back(r);
+            continue;
+        }
+        if (last) {  // the rest of the factor
             const int k = eighths & 7;
             r.odd = k & 1;
             r.quarter = k >> 1;
@@ -1189,9 +1247,9 @@ void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *o
     }
 }
 
-cudaError_t launch_gate_runs(sv_state *h, const GateRuns &p) {
-    if (h->dt == SV_C128) return p.slots == 2 ? gate_runs_impl<double, 2>(h, p) : gate_runs_impl<double, 4>(h, p);
-    return p.slots == 3 ? gate_runs_impl<float, 3>(h, p) : gate_runs_impl<float, 4>(h, p);
+cudaError_t launch_gate_runs(sv_state *h, const GateRuns &p, const std::vector<Gate1> &g) {
+    if (h->dt == SV_C128) return p.slots == 2 ? gate_runs_impl<double, 2>(h, p, g) : gate_runs_impl<double, 4>(h, p, g);
+    return p.slots == 3 ? gate_runs_impl<float, 3>(h, p, g) : gate_runs_impl<float, 4>(h, p, g);
 }
 
 cudaError_t launch_set_basis(sv_state *h, uint64_t idx) {

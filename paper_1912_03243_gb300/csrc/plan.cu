@@ -691,7 +691,7 @@ sv_status execute_direct(sv_plan_s *p) {
 extern "C++" {
 cudaError_t plan_launch_all(sv_plan_s *p) {
     if (small_plan(p)) return launch_small_run(p->h, p->pergate.data(), p->pergate.size());
-    if (!p->gruns.runs.empty()) return launch_gate_runs(p->h, p->gruns);
+    if (!p->gruns.runs.empty()) return launch_gate_runs(p->h, p->gruns, p->pergate);
     for (const PlanLaunch &l : p->launches) {
         const cudaError_t e = launch_one(p, l);
         if (e != cudaSuccess) return e;

@@ -134,6 +134,7 @@ struct GateRun {
     int count = 0, ucount = 0;
     int odd = 0, quarter = 0;     // factor paid after them: (1 + i)^odd i^quarter m
     double m = 1.0;
+    std::vector<int> alone;       // instead (count 0): gates that are faster in launches of their own
 };
 struct GateRuns {
     int slots = 0;
@@ -143,7 +144,7 @@ struct GateRuns {
 };
 bool gate_runs_fit(sv_dtype dt, int n);
 void plan_gate_runs(sv_dtype dt, int n, const std::vector<Gate1> &g, GateRuns *out);
-cudaError_t launch_gate_runs(sv_state *h, const GateRuns &p);
+cudaError_t launch_gate_runs(sv_state *h, const GateRuns &p, const std::vector<Gate1> &g);
 cudaError_t launch_set_basis(sv_state *h, uint64_t idx);
 cudaError_t launch_norm(sv_state *h, double *d_out);  // d_out: device double
 cudaError_t launch_gather(sv_state *h, const uint64_t *d_idx, size_t m, double *d_out);

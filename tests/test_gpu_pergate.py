@@ -422,3 +422,65 @@ def test_runs_on_low_qubits_are_coalesced(S):
             us[name] = min(us[name], ev[0].elapsed_time(ev[1]) * 100)
         p.free()
     assert us["low"] <= 2.5 * us["high"], us
+
+
+@pytest.mark.parametrize("dtype,n", [("c64", 23), ("c128", 19), ("c128", 20), ("c128", 22)])
+def test_runs_and_launches_of_their_own(S, orc, dtype, n):
+    """Plans in which runs of gates that owe factors alternate with diagonal
+    gates that keep their own launches, these first, between and last: the
+    factors are paid all the same."""
+    c = C.Circuit(n)
+
+    def phases():
+        for q in (0, 4, 9, n - 2):
+            c.add("CP", q, q + 1, 0.2 + 0.1 * q)
+        c.add("CZ", 0, n - 1)
+
+    phases()
+    for name in ("SX", "H", "SYDG"):
+        for q in (0, 3, n - 1):
+            c.add(name, q)
+        phases()
+    psi0 = C.random_state(n, 90 + n)
+    ref = orc.run(c, psi=psi0)
+    s = S.StateVector(n, dtype)
+    p = s.plan(c, "pergate")
+    for _ in range(3):  # direct, capture, replay
+        s.from_numpy(psi0)
+        p.execute()
+        check(dtype, s.to_numpy(), ref)
+    p.free()
+
+
+@pytest.mark.parametrize("dtype,n", [("c64", 23), ("c128", 22), ("c128", 20)])
+def test_diagonal_gates_are_not_slower_together(S, dtype, n):
+    """Controlled phases on a large state, each of which visits a quarter of it,
+    take no longer in one plan than in a plan each (and a fifth)."""
+    import torch
+
+    c = C.Circuit(n)
+    for q in range(n - 1):
+        c.add("CP", q, q + 1, 0.1 + 0.1 * q)
+    if dtype == "c64":
+        c.gates = c.gates[-2:]
+    s = S.StateVector(n, dtype)
+    alone = []
+    for g in c.gates:
+        one = C.Circuit(n)
+        one.gates = [g]
+        alone.append(s.plan(one, "pergate"))
+    us = {}
+    for name, plans in (("together", [s.plan(c, "pergate")]), ("alone", alone)):
+        us[name] = 1e9
+        for _ in range(8):
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            ev[0].record()
+            for _ in range(10):
+                for p in plans:
+                    p.execute()
+            ev[1].record()
+            torch.cuda.synchronize()
+            us[name] = min(us[name], ev[0].elapsed_time(ev[1]) * 100)
+        for p in plans:
+            p.free()
+    assert us["together"] <= 1.2 * us["alone"], us
