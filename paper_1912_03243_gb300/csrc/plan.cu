@@ -81,10 +81,40 @@ sv_status build_fused_plan(sv_state *h, const Circuit &c, sv_plan_s *p, int kfix
     return SV_OK;
 }
 
+// Time of a gate of the two-byte code in a pass of its own and in a run, in
+// us: full passes over the code at HBM's rate (see enc_pass_us), and what a
+// launch takes on the smallest states.  A pass of its own computes longer than
+// it moves the code (H inside the blocks 1.7 full passes) except where it only
+// moves or negates codes; a run's traffic comes on top of its gates' (two
+// block loads in flight per warp), and an X inside the blocks computes there.
+double enc_pass_us(int n) { return std::ldexp(4.0, n) / 6.8e6; }
+double enc_alone_us(const sv_state *h, const Gate1 &g) {
+    const std::string k = gate1_kernel_name(h, g);
+    const double pass = enc_pass_us(h->n), part = g.control >= kEncBlockLog2 ? 0.5 : 1.0;
+    const auto one = [](const Cplx &z, double re) { return z.re == re && z.im == 0.0; };
+    const bool both = one(g.u[0], -1) && one(g.u[3], -1);
+    if (k == "k_enc_flip") return 2.1 + 1.07 * pass * part * (!both && g.target >= kEncBlockLog2 ? 0.5 : 1.0);
+    if (k == "k_enc_xin") return 2.1 + 1.07 * pass * part;
+    // (exchange of blocks: 2.6 passes once the code leaves L2)
+    if (k == "k_enc_xblocks") return 2.1 + (h->n <= 25 ? 1.07 : 2.6) * pass * part;
+    return 4.2 + (k == "k_enc_gate_across<diag1>" ? 0.95 : 1.65) * pass * part;
+}
+double enc_in_run_us(int n, const EncRunOp &op) {
+    const double pass = enc_pass_us(n), part = op.hi_mask ? 0.5 : 1.0;
+    if (op.kind == ENC_OP_FLIP) return 0.05 * pass;
+    if (op.kind == ENC_OP_SWAP) return 0.1 + 0.15 * pass * part;
+    const bool diag1 = op.shape == 3;
+    if (op.kind == ENC_OP_PAIR && diag1) return 0.5 + 0.45 * pass * part;
+    return 0.5 + (diag1 ? 0.95 : op.shape == 1 ? 1.0 : 1.15) * pass * part;
+}
+
 // Two-byte code: a run of consecutive gates whose targets are in-block qubits
 // or at most B block bits, and sign flips, becomes one pass (k_enc_run_in)
-// where its gates, one pass each, would move more bytes than one pass over
-// the code; the other gates keep their own passes.  A warp takes a tile of
+// where its gates, one pass each, would take longer; the other gates keep
+// their own passes.  (By bytes alone, runs of a few X and CX were slower than
+// their passes: X on two qubits 12 qubits 6.4 us against 4.4 and 23 qubits 17.1
+// and 13.1; CX both ways between a low and the highest qubit, 27 qubits, 209 and
+// 177.)  A warp takes a tile of
 // 2^B blocks through the whole run, so B is the largest that still leaves
 // about 2^10 tiles (7 warps per SM): B = 4 from 22 qubits on, 1 up to 19.
 // SV_ENC_RUNS=0 keeps one pass per gate.
@@ -105,7 +135,7 @@ sv_status build_enc_runs(sv_state *h, sv_plan_s *p) {
     while (i < ng) {
         EncRunOp op;
         size_t j = i;
-        double alone = 0.0;
+        double alone = 0.0, together = 4.2 + enc_pass_us(h->n);
         std::vector<int> bits;  // block bits of the run's tiles, ascending
         while (j < ng && j - i < size_t(kEncRunMaxOps) && enc_run_op(h->n, p->pergate[j], &op)) {
             if (op.kind == ENC_OP_PAIR || op.kind == ENC_OP_SWAP) {
@@ -115,7 +145,8 @@ sv_status build_enc_runs(sv_state *h, sv_plan_s *p) {
                     bits.insert(it, op.t);
                 }
             }
-            alone += gate1_bytes(h, p->pergate[j]);
+            alone += enc_alone_us(h, p->pergate[j]);
+            together += enc_in_run_us(h->n, op);
             ++j;
         }
         // From 23 qubits on a run with fewer bits takes other ones of the block
@@ -125,7 +156,7 @@ sv_status build_enc_runs(sv_state *h, sv_plan_s *p) {
         // Runs inside the blocks have none and take one block per warp.
         for (int b = 0; nb_log >= 15 && !bits.empty() && int(bits.size()) < bmax; ++b)
             if (!std::binary_search(bits.begin(), bits.end(), b)) bits.insert(std::lower_bound(bits.begin(), bits.end(), b), b);
-        if (j - i >= 2 && alone > pass_bytes) {
+        if (j - i >= 2 && alone > together) {
             PlanLaunch l{4, int(p->encruns.size()), pass_bytes};
             sv_plan_s::EncRun run{int(ops.size()), int(j - i), int(bits.size()), {0, 0, 0, 0}};
             for (size_t k = 0; k < bits.size(); ++k) run.pos[k] = bits[k];

@@ -264,3 +264,28 @@ def test_runs_inside_blocks_do_their_work_once(S, monkeypatch):
         p.free()
         enc.free()
     assert ms["1"] <= 1.5 * ms["0"], ms
+
+
+@pytest.mark.parametrize("n", [9, 12, 23, 27])
+def test_runs_where_they_are_faster(S, n):
+    """A few gates that only move or negate codes keep passes of their own (a
+    run decodes the code and computes in its tiles); gates that compute, and
+    many of any kind, go together."""
+    s = S.StateVector(n, "enc2b")
+
+    def kernels(gates):
+        c = C.Circuit(n)
+        for g in gates:
+            c.add(*g)
+        p = s.plan(c, "pergate")
+        names = [k for k, _ in p.launch_info()]
+        p.free()
+        return names
+
+    h = n - 1
+    assert "k_enc_run_in" not in kernels([("CX", h, 0), ("CX", h, 3)])
+    assert "k_enc_run_in" not in kernels([("CZ", 0, h), ("CZ", 1, h)])
+    if n <= 25:
+        assert "k_enc_run_in" not in kernels([("X", 0), ("X", h)])
+    assert kernels([("H", 0), ("SX", 3), ("H", h)]) == ["k_enc_run_in"]
+    assert kernels([("X", k % 8) for k in range(24)] + [("Z", k % 8) for k in range(24)]) == ["k_enc_run_in"]
