@@ -13,6 +13,9 @@ namespace sv {
 constexpr int kEncRunMaxOps = 64;  // ops of one run (one pass)
 constexpr int kEncRunMaxBits = 4;  // block bits of a run's tiles
 
+// Shape of a gate's matrix, from its exact zeros.
+enum EncShape { ENC_GENERAL = 0, ENC_REAL = 1, ENC_DIAG = 2, ENC_DIAG1 = 3 };  // (DIAG1: u00 = 1)
+
 enum EncOpKind : int {
     ENC_OP_IN = 0,    // 2x2 update on in-block target t
     ENC_OP_FLIP = 1,  // sign flip of the codes
@@ -23,7 +26,7 @@ enum EncOpKind : int {
 struct EncRunOp {
     int kind;
     int t, c;                  // target, in-block control (-1: none)
-    int shape;                 // matrix shape (exact zeros), as the single-gate kernels use it
+    int shape;                 // EncShape, as the single-gate kernels use it
     uint32_t lo_mask, lo_val;  // flip: in-block index bits of the condition
     uint32_t amps;             // flip: which of a lane's 8 amplitudes meet bits 0..2 of the condition
     uint32_t pad;

@@ -30,9 +30,9 @@
 // half the issue slots.  The decode table is addressed with one byte permute,
 // the block maximum is 3-input absolute maxima and one warp reduction (REDUX
 // on the bits: non-negative floats order as integers), and in-block pairs are
-// formed by exchanging packed codes.  28 qubits, one gate per pass: H inside
-// the blocks 255-274 us (319-385 before), H across them 240 (268), SX across
-// 244 (298), T across 129 (155); 27 qubits, 160 gates in runs: 11.0 ms
+// formed by exchanging packed codes.  27 qubits, one gate per pass: H inside
+// the blocks 138 us (172 before), H across them 128 (144), SX across 134 (159),
+// T across 76 (91); 27 qubits, 160 gates in runs: 11.0 ms
 // (17.5 with runs of in-block gates only).
 #include "sv_internal.h"
 
@@ -256,8 +256,7 @@ __device__ __forceinline__ void encode_two(const Amp2 (&x)[4], float s0, const A
 // fixed-order update (gate_pair), or the same update with the terms of zero
 // coefficients left out.  A left-out term contributes fmaf(0, x, y) = y up to
 // the sign of a zero, and a zero (of either sign) encodes to code 0 and does
-// not change a block maximum, so the codes are those of the general form.
-enum EncShape { ENC_GENERAL = 0, ENC_REAL = 1, ENC_DIAG = 2, ENC_DIAG1 = 3 };
+// not change a block maximum, so the codes are those of the general form (EncShape).
 
 // The matrix as packed operands; -u for the products the update subtracts
 // (a product with a negated factor is the negated product).
@@ -789,10 +788,12 @@ __global__ void __launch_bounds__(256) k_enc_xblocks(uint4 *__restrict__ codes, 
 // The tile's codes sit in shared memory, 16 bytes per lane and block, and are
 // only ever touched by their own lane (gates across blocks keep the lane,
 // in-block ones exchange codes by shuffles), so no gate needs a barrier; lane
-// k holds the scale of block k.  Bound: instruction issue (66-69% active, FMA
-// pipe 59%, ALU pipe 51%) on about 150 instructions per block and gate; the
-// HBM traffic, 1 KB per block and run, hides behind it.  B = 4: 8 KB per warp
-// and the 64 KB table leave 16 warps on an SM at 128 registers.  (Decoding by
+// k holds the scale of block k.  Bound: instruction issue (67% active, ALU
+// pipe 50%, FMA pipe 41%, under a profiler) on about 170 instructions per block
+// and gate; the HBM traffic, 1 KB per block and run, is 6% of a run of 12 gates,
+// but with 16 warps on an SM little of it overlaps in a run of two (plan.cu
+// weighs it).  B = 4: 8 KB per warp and the 64 KB table leave 16 warps on an SM
+// at 128 registers.  (Decoding by
 // arithmetic instead of the table: 11.7 against 11.0 ms on 27 qubits and 160
 // gates; 24 warps at 80 registers: spills, 11.9 against 11.7.)
 //
@@ -878,7 +879,7 @@ __device__ __forceinline__ void run_gate(const DecTable &dec, const EncRunOp &op
     }
 }
 
-template <int NB>  // tile bits, or -1: a.nbits
+template <int NB, bool FULL = false>  // tile bits, or -1: a.nbits; CTAs of kRunWarps warps
 __global__ void __launch_bounds__(32 * kRunWarps, NB == 0 ? kRunCtas0 : 1) k_enc_run_in(uint4 *__restrict__ codes,
                                                                      float *__restrict__ scales,
                                                                      const EncRunOp *__restrict__ gops,
@@ -903,8 +904,9 @@ __global__ void __launch_bounds__(32 * kRunWarps, NB == 0 ? kRunCtas0 : 1) k_enc
     uint4 *tile = &held;
     if constexpr (NB != 0) tile = reinterpret_cast<uint4 *>(smem + kTabBytes) + (threadIdx.x >> 5) * (nblk * 32);
     const int ml = NB == 0 ? 0 : lane;  // this lane's place in a block of the tile
-    const uint64_t wid = uint64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const uint64_t nw = uint64_t(gridDim.x) * (blockDim.x >> 5);
+    const unsigned warps = FULL ? unsigned(kRunWarps) : blockDim.x >> 5;
+    const uint64_t wid = uint64_t(blockIdx.x) * warps + (threadIdx.x >> 5);
+    const uint64_t nw = uint64_t(gridDim.x) * warps;
     for (uint64_t w = wid; w < a.ntiles; w += nw) {
         uint64_t b64 = w;
 #pragma unroll
@@ -996,7 +998,9 @@ cudaError_t enc_attrs(int device) {
           set(k_enc_gate_in<ENC_DIAG>, kTabBytes), set(k_enc_gate_in<ENC_DIAG1>, kTabBytes),
           set(k_enc_gate_across<ENC_GENERAL>, kTabBytes), set(k_enc_gate_across<ENC_REAL>, kTabBytes),
           set(k_enc_gate_across<ENC_DIAG>, kTabBytes), set(k_enc_gate_across<ENC_DIAG1>, kTabBytes),
-          set(k_enc_run_in<kEncRunMaxBits>, run), set(k_enc_run_in<-1>, run), set(k_enc_run_in<0>, run)})
+          set(k_enc_run_in<kEncRunMaxBits, true>, run), set(k_enc_run_in<kEncRunMaxBits>, run),
+          set(k_enc_run_in<-1, true>, run), set(k_enc_run_in<-1>, run),
+          set(k_enc_run_in<0>, run)})
         if (e != cudaSuccess) return e;
     attrs_set(configured, device);
     return cudaSuccess;
@@ -1167,7 +1171,9 @@ cudaError_t launch_enc_run(sv_state *h, const EncRunOp *d_ops, int nops, int nbi
     const cudaError_t e = enc_attrs(h->device);
     if (e != cudaSuccess) return e;
     // few tiles spread over the SMs, on CTAs of at least 8 warps (4 take 2 us
-    // longer to fill the decode table)
+    // longer to fill the decode table): 22 qubits, random circuit of depth 3, 485
+    // us on 64 CTAs of 16 warps, 355 on 128 of 8.  Full CTAs have the number of
+    // warps as a constant (27 qubits, 160 gates 11.02 ms, 11.04 without).
     const uint64_t share = (a.ntiles + 151) / 152;
     const unsigned warps = unsigned(share < 8 ? 8 : share > kRunWarps ? kRunWarps : share);
     const unsigned block = 32 * warps;
@@ -1175,12 +1181,14 @@ cudaError_t launch_enc_run(sv_state *h, const EncRunOp *d_ops, int nops, int nbi
     const uint64_t cap = 152 * (nbits == 0 ? kRunCtas0 : 1);
     const unsigned grid = unsigned(want < cap ? want : cap);
     const int smem = kTabBytes + (nbits == 0 ? 0 : int(warps) * (512 << nbits));
-    if (nbits == kEncRunMaxBits)
-        k_enc_run_in<kEncRunMaxBits><<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a);
-    else if (nbits == 0)
-        k_enc_run_in<0><<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a);
+    auto go = [&](auto *fn) { fn<<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a); };
+    const bool full = warps == kRunWarps;
+    if (nbits == 0)
+        go(k_enc_run_in<0>);
+    else if (nbits == kEncRunMaxBits)
+        full ? go(k_enc_run_in<kEncRunMaxBits, true>) : go(k_enc_run_in<kEncRunMaxBits>);
     else
-        k_enc_run_in<-1><<<grid, block, smem, h->stream>>>(codes, h->scales, d_ops, a);
+        full ? go(k_enc_run_in<-1, true>) : go(k_enc_run_in<-1>);
     return cudaGetLastError();
 }
 

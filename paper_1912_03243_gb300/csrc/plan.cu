@@ -1,5 +1,6 @@
 // Plan creation and replay.
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <string>
 
@@ -81,12 +82,15 @@ sv_status build_fused_plan(sv_state *h, const Circuit &c, sv_plan_s *p, int kfix
     return SV_OK;
 }
 
-// Time of a gate of the two-byte code in a pass of its own and in a run, in
-// us: full passes over the code at HBM's rate (see enc_pass_us), and what a
-// launch takes on the smallest states.  A pass of its own computes longer than
-// it moves the code (H inside the blocks 1.7 full passes) except where it only
-// moves or negates codes; a run's traffic comes on top of its gates' (two
-// block loads in flight per warp), and an X inside the blocks computes there.
+// Time of a gate of the two-byte code in a pass of its own and in a run, in us:
+// in passes over the code at HBM's rate (enc_pass_us), plus what a launch takes
+// on the smallest states.  A pass of its own computes longer than it moves the
+// code (H inside the blocks 1.7 passes) except where it only moves or negates
+// codes.  A run's traffic comes on top of its gates' work, and an X inside the
+// blocks computes there.  Fitted to single gates and pairs of gates at 9 to 27
+// qubits (27 qubits, us: H inside 138, across 128, SX 143 and 134, T 135 and 76,
+// X inside 84, across 210, with half the blocks 45; in runs H H 240, SX SX 267,
+// T T 187, X X 172).
 double enc_pass_us(int n) { return std::ldexp(4.0, n) / 6.8e6; }
 double enc_alone_us(const sv_state *h, const Gate1 &g) {
     const std::string k = gate1_kernel_name(h, g);
@@ -103,9 +107,9 @@ double enc_in_run_us(int n, const EncRunOp &op) {
     const double pass = enc_pass_us(n), part = op.hi_mask ? 0.5 : 1.0;
     if (op.kind == ENC_OP_FLIP) return 0.05 * pass;
     if (op.kind == ENC_OP_SWAP) return 0.1 + 0.15 * pass * part;
-    const bool diag1 = op.shape == 3;
+    const bool diag1 = op.shape == ENC_DIAG1;
     if (op.kind == ENC_OP_PAIR && diag1) return 0.5 + 0.45 * pass * part;
-    return 0.5 + (diag1 ? 0.95 : op.shape == 1 ? 1.0 : 1.15) * pass * part;
+    return 0.5 + (diag1 ? 0.95 : op.shape == ENC_REAL ? 1.0 : 1.15) * pass * part;
 }
 
 // Two-byte code: a run of consecutive gates whose targets are in-block qubits
