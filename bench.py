@@ -67,6 +67,8 @@ PROFILE_CASES = {
     "tiled24": "28 qubits, random circuit depth 24 (passes as full as at 32 qubits)",
     "pergate": "28 qubits, random circuit depth 1, one launch per gate",
     "enc": "28 qubits, two-byte code, random circuit depth 1",
+    "encruns": "27 qubits, two-byte code, random circuit depth 4 (runs of gates)",
+    "gateruns": "20 qubits, complex128, random circuit depth 20, and 10 qubits, complex64, depth 10: per-gate plans in runs",
     "fused": "26 qubits, three dense 6-qubit blocks on the tensor cores (low, high and mixed qubits)",
     "cut": "6x4 grid (24 qubits), depth 12, 8 cut CZs: 256 branches x 2 batched halves of 2^12 amplitudes each",
     "expect": "28 qubits, uniform superposition, <sigma^alpha_i> of every qubit (complex64, then the two-byte code)",
@@ -88,6 +90,14 @@ def run_profile_case(case: str) -> None:
     elif case == "enc":
         s = sv.StateVector(28, "enc2b")
         s.run(C.random_circuit(28, 1, 1), "pergate")
+    elif case == "encruns":
+        s = sv.StateVector(27, "enc2b")
+        s.run(C.random_circuit(27, 4, 1), "pergate")
+    elif case == "gateruns":
+        t = sv.StateVector(10, "c64")
+        t.run(C.random_circuit(10, 10, 1), "pergate")
+        s = sv.StateVector(20, "c128")
+        s.run(C.random_circuit(20, 20, 1), "pergate")
     elif case == "fused":
         s = sv.StateVector(26, "c64")
         rng = np.random.default_rng(0)

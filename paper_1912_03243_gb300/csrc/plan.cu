@@ -160,7 +160,7 @@ sv_status build_enc_runs(sv_state *h, sv_plan_s *p) {
         // Runs inside the blocks have none and take one block per warp.
         for (int b = 0; nb_log >= 15 && !bits.empty() && int(bits.size()) < bmax; ++b)
             if (!std::binary_search(bits.begin(), bits.end(), b)) bits.insert(std::lower_bound(bits.begin(), bits.end(), b), b);
-        if (j - i >= 2 && alone > together) {
+        if (j - i >= 2 && alone > 1.05 * together) {
             PlanLaunch l{4, int(p->encruns.size()), pass_bytes};
             sv_plan_s::EncRun run{int(ops.size()), int(j - i), int(bits.size()), {0, 0, 0, 0}};
             for (size_t k = 0; k < bits.size(); ++k) run.pos[k] = bits[k];
