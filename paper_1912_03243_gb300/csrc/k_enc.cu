@@ -1170,12 +1170,13 @@ cudaError_t launch_enc_run(sv_state *h, const EncRunOp *d_ops, int nops, int nbi
     uint4 *codes = static_cast<uint4 *>(h->data);
     const cudaError_t e = enc_attrs(h->device);
     if (e != cudaSuccess) return e;
-    // few tiles spread over the SMs, on CTAs of at least 8 warps (4 take 2 us
-    // longer to fill the decode table): 22 qubits, random circuit of depth 3, 485
-    // us on 64 CTAs of 16 warps, 355 on 128 of 8.  Full CTAs have the number of
-    // warps as a constant (27 qubits, 160 gates 11.02 ms, 11.04 without).
+    // few tiles spread over the SMs, on CTAs of at least 8 warps (22 qubits, random
+    // circuit of depth 3: 485 us on 64 CTAs of 16 warps, 355 on 128 of 8; 4 warps
+    // take 2 us longer to fill the decode table).  Tiles of one CTA take 16, which
+    // fill it sooner (12 qubits, two SX 6.3 us, 8.2 with 8).  Full CTAs have the
+    // number of warps as a constant (27 qubits, 160 gates 11.02 ms, 11.04 without).
     const uint64_t share = (a.ntiles + 151) / 152;
-    const unsigned warps = unsigned(share < 8 ? 8 : share > kRunWarps ? kRunWarps : share);
+    const unsigned warps = unsigned(a.ntiles <= kRunWarps || share > kRunWarps ? kRunWarps : share < 8 ? 8 : share);
     const unsigned block = 32 * warps;
     const uint64_t want = (a.ntiles + warps - 1) / warps;
     const uint64_t cap = 152 * (nbits == 0 ? kRunCtas0 : 1);

@@ -101,7 +101,7 @@ double enc_alone_us(const sv_state *h, const Gate1 &g) {
     if (k == "k_enc_xin") return 2.1 + 1.07 * pass * part;
     // (exchange of blocks: 2.6 passes once the code leaves L2)
     if (k == "k_enc_xblocks") return 2.1 + (h->n <= 25 ? 1.07 : 2.6) * pass * part;
-    return 4.2 + (k == "k_enc_gate_across<diag1>" ? 0.95 : 1.65) * pass * part;
+    return std::max(4.2, (h->n < 25 ? 3.0 : 2.1) + (k == "k_enc_gate_across<diag1>" ? 0.9 : 1.65) * pass * part);
 }
 double enc_in_run_us(int n, const EncRunOp &op) {
     const double pass = enc_pass_us(n), part = op.hi_mask ? 0.5 : 1.0;
@@ -160,7 +160,7 @@ sv_status build_enc_runs(sv_state *h, sv_plan_s *p) {
         // Runs inside the blocks have none and take one block per warp.
         for (int b = 0; nb_log >= 15 && !bits.empty() && int(bits.size()) < bmax; ++b)
             if (!std::binary_search(bits.begin(), bits.end(), b)) bits.insert(std::lower_bound(bits.begin(), bits.end(), b), b);
-        if (j - i >= 2 && alone > 1.05 * together) {
+        if (j - i >= 2 && alone > together) {
             PlanLaunch l{4, int(p->encruns.size()), pass_bytes};
             sv_plan_s::EncRun run{int(ops.size()), int(j - i), int(bits.size()), {0, 0, 0, 0}};
             for (size_t k = 0; k < bits.size(); ++k) run.pos[k] = bits[k];
