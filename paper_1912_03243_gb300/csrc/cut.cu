@@ -758,7 +758,7 @@ static sv_status cut_impl(const char *text, int n, const uint8_t *part_of, int P
         if (e != cudaSuccess) s = cuda_status(e, "cudaMemcpyAsync");
     }
     if (s == SV_OK) s = sync_stream(st, "sv_cut_amplitudes");
-    cudaStreamSynchronize(st);
+    if (s != SV_OK) cudaStreamSynchronize(st);
     cudaFree(mem);
     return s;
 }
